@@ -54,12 +54,72 @@ long long layout_strides_padded(const int dim[3], int a, int esz, int str[3]) {
     return row * dim[ord[1]] * dim[ord[2]];
 }
 
+double ray_reach(const vr_ctx *c, const Cube *cb) {
+    const Cam &m = c->cam;
+    double dist2 = 0.0, diag2 = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        const double eye = -((double)m.R[k] * m.t[0] + (double)m.R[3 + k] * m.t[1] + (double)m.R[6 + k] * m.t[2]);
+        const double cen = 0.5 * (double)cb->n[k];
+        dist2 += (eye - cen) * (eye - cen);
+        diag2 += (double)cb->n[k] * cb->n[k];
+    }
+    return std::sqrt(dist2) + std::sqrt(diag2);
+}
+
+// Atlas frames clamp no stencil index.  A brick's samples lie at stored coordinates [0.5, core +
+// 0.5] but for rounding, and its cells are inside the stored brick from -0.0 to core + 1: half a
+// voxel of room either way.  With t up to this reach the rounding is below 0.12: the slab
+// test's planes and k = ceil(t / step) 3 x 2^-24 t (0.047), a MIP sample's o + t d and its -0.5
+// at most 3 half-ulps of 2^18 (0.047), and within a segment of at most 113 500 voxels j step and
+// q + t d about 0.011.  Cameras further away (rounding of whole voxels) read the linear copy, whose
+// indices are clamped; the frames are the same.
+constexpr double kAtlasReach = 262144.0;
+
+// (1 / K is rounded up: floor(z / K) is then exact for the slices of any stored brick.)
+void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0) {
+    b.atlas = tex;
+    b.at_org[0] = (float)(x0 + 1);
+    b.at_org[1] = (float)(y0 + 1);
+    b.at_dim[0] = (float)b.dim[0];
+    b.at_dim[1] = (float)b.dim[1];
+    float inv = 1.0f / (float)std::max(rows, 1);
+    while ((double)inv * rows < 1.0) inv = std::nextafterf(inv, 2.0f);
+    b.at_inv = inv;
+    b.at_neg = -(float)rows;
+    b.at_rows = rows;
+}
+
+// What the 2D-gather size admits is decided by the squarest arrangement (2^l columns, no copies).
+// Columns are then as tall as fit, evened out: fewest copies (258^3 bricks: 3 columns of 86 slices
+// and a copy, 1.2 % more texels).  Between the two rules lie bricks of about a billion texels
+// (stored cubes from 993^3 to 1024^3): they are admitted, with rows = 0, and read the linear copy.
+int atlas_geom(int device, const int dim[3], bool pair, AtlasGeom &g) {
+    int gw = 0, gh = 0;
+    CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, device));
+    CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, device));
+    const int nt = pair ? dim[2] - 1 : dim[2];              // tiles
+    int l = 0;
+    while ((1ll << (2 * l)) < nt) ++l;
+    if (((long long)dim[0] << l) > gw || (long long)((nt + (1 << l) - 1) >> l) * dim[1] > gh)
+        return fail(VR_ERR_UNSUPPORTED, "bricks too large for a slice atlas (2D gather limit)");
+    g = AtlasGeom{};
+    const int fit = gh / dim[1], extra = pair ? 0 : 1;
+    const int cols = nt <= fit ? 1 : (fit > extra ? (nt + fit - extra - 1) / (fit - extra) : gw);
+    if ((long long)cols * dim[0] > gw) return VR_OK;         // rows = 0: no room for the copies
+    g.rows = (nt + cols - 1) / cols;
+    g.w = cols * dim[0];
+    g.h = (g.rows + (cols > 1 ? extra : 0)) * dim[1];
+    return VR_OK;
+}
+
 FrameLayout frame_layout(const vr_ctx *c, const Cube *cb) {
     FrameLayout f{0, 0, kRcLong, kRcShort, 0.0f, 0};
     float best = -1.0f;
     // resident cubes: atlases built with the pool; streamed and compressed cubes: atlases of the
     // brick cache's slots, packed as bricks become resident
-    const bool atlas = cb->streamed ? (cb->layouts & 8) != 0 : !cb->atlas_tex.empty();
+    // (within kAtlasReach: atlas frames clamp no index, see there)
+    const bool atlas = (cb->streamed ? (cb->layouts & 8) != 0 && cb->atlas_fit : !cb->atlas_tex.empty()) &&
+                       (!c->cam_set || ray_reach(c, cb) <= kAtlasReach);
     // with atlases, the image axis is fixed first: the one with the smaller z component
     const int only = atlas ? (std::fabs(c->cam.R[5]) < std::fabs(c->cam.R[2]) ? 1 : 0) : -1;
     for (int i = 0; i < 2; ++i)              // image axis: camera right (row 0), up (row 1)
@@ -619,15 +679,9 @@ int check_ready(vr_ctx *c, Cube *cb) {
     if (!c->cam_set) { g_last_error = "no camera"; return VR_ERR_STATE; }
     // every lattice index k = t/step reached inside the cube must fit comfortably in an int:
     // t <= |camera - cube centre| + half diagonal
-    const Cam &m = c->cam;
-    double eye[3], cen[3], dist2 = 0.0, diag2 = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        eye[k] = -((double)m.R[k] * m.t[0] + (double)m.R[3 + k] * m.t[1] + (double)m.R[6 + k] * m.t[2]);
-        cen[k] = 0.5 * (double)cb->n[k];
-        dist2 += (eye[k] - cen[k]) * (eye[k] - cen[k]);
-        diag2 += (double)cb->n[k] * cb->n[k];
-    }
-    const double tmax = std::sqrt(dist2) + std::sqrt(diag2);
+    double diag2 = 0.0;
+    for (int k = 0; k < 3; ++k) diag2 += (double)cb->n[k] * cb->n[k];
+    const double tmax = ray_reach(c, cb);
     if (tmax / (double)c->step > (double)(1 << 28) || std::sqrt(diag2) / c->step > (double)(1 << 24))
         return arg_fail("step too small for this camera and cube (lattice index would overflow)");
     return VR_OK;
@@ -646,13 +700,11 @@ void free_atlases(Cube *cb) {
     cb->atlas_arr.clear();
     cb->atlas_bytes = 0;
     cb->atlas_pair = false;
-    for (auto &d : cb->tmpl) { d.atlas = 0; d.alog = 0; }
+    for (auto &d : cb->tmpl) d.atlas = 0;
 }
 
-// Slice atlas of every brick (layout bit 3) from its x-contiguous copy in the pool: slice z
-// of a brick of dx x dy x dz stored elements becomes tile (z mod 2^alog, z div 2^alog) of a 2D
-// array of 2^alog dx x ceil(dz / 2^alog) dy texels, with 2^alog the smallest power of two whose
-// square is >= dz.  FP32 bricks keep their values, 16-bit bricks their codes (FP16 as half
+// Slice atlas of every brick (layout bit 3) from its x-contiguous copy in the pool, placed by
+// atlas_geom.  FP32 bricks keep their values, 16-bit bricks their codes (FP16 as half
 // texels, BF16 as 16-bit unsigned ones).  With layout bit 5, 16-bit bricks get pair atlases
 // instead: dz - 1 tiles of 32-bit texels, tile z holding the codes of slices z and z + 1 (one
 // gather per sample).  The array must fit the device's limit for 2D gathers.
@@ -662,21 +714,16 @@ int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
     const bool pair = (cb->layouts & 32) && cb->storage != VR_F32;
     const size_t bsz = cb->storage == VR_F32 ? 4 : 2;       // bytes of a stored element
     const size_t esz = pair ? 4 : bsz;                       // bytes of a texel
-    int gw = 0, gh = 0;
-    CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, c->device));
-    CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, c->device));
-    std::vector<int> lg(nbr);
+    std::vector<AtlasGeom> geo(nbr);
     size_t most = 16;
+    cb->atlas_fit = true;
     for (int i = 0; i < nbr; ++i) {
-        const int *dm = cb->tmpl[i].dim;
-        const int nt = pair ? dm[2] - 1 : dm[2];            // tiles
-        int l = 0;
-        while ((1ll << (2 * l)) < nt) ++l;
-        const long long w = (long long)dm[0] << l, h = (long long)((nt + (1 << l) - 1) >> l) * dm[1];
-        if (w > gw || h > gh) return fail(VR_ERR_UNSUPPORTED, "bricks too large for a slice atlas (2D gather limit)");
-        lg[i] = l;
-        most = std::max(most, (size_t)(w * h) * esz);
+        const int rc = atlas_geom(c->device, cb->tmpl[i].dim, pair, geo[i]);
+        if (rc != VR_OK) return rc;
+        if (geo[i].rows == 0) cb->atlas_fit = false;
+        most = std::max(most, (size_t)geo[i].w * geo[i].h * esz);
     }
+    if (!cb->atlas_fit) return VR_OK;        // frames read the linear copy
     void *tmp = nullptr;
     CK(cudaMalloc(&tmp, most));
     std::vector<cudaSurfaceObject_t> surfs;   // kept until the packs that write through them ran
@@ -700,8 +747,7 @@ int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
     cb->atlas_tex.assign(nbr, 0);
     for (int i = 0; i < nbr; ++i) {
         const int *dm = cb->tmpl[i].dim;
-        const int nt = pair ? dm[2] - 1 : dm[2];
-        const size_t w = (size_t)dm[0] << lg[i], h = (size_t)((nt + (1 << lg[i]) - 1) >> lg[i]) * dm[1];
+        const size_t w = (size_t)geo[i].w, h = (size_t)geo[i].h;
         cudaArray_t arr = nullptr;
         // written by the pack kernel through a surface where the device allows surface stores on
         // a gather array; else packed into staging and copied (the copy engine's array writes)
@@ -722,12 +768,12 @@ int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
             cudaSurfaceObject_t sf = 0;
             if ((e = cudaCreateSurfaceObject(&sf, &rd)) != cudaSuccess) return bail(e, "cudaCreateSurfaceObject");
             surfs.push_back(sf);
-            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], lg[i], nullptr, 0, (unsigned long long)sf, s)
-                     : launch_atlas_pack_surf(src, (int)esz, dm[0], dm[1], dm[2], lg[i], (unsigned long long)sf, s);
+            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], geo[i].rows, nullptr, 0, (unsigned long long)sf, s)
+                     : launch_atlas_pack_surf(src, (int)esz, dm[0], dm[1], dm[2], geo[i].rows, (unsigned long long)sf, s);
             if (e != cudaSuccess) return bail(e, "atlas pack launch");
         } else {
-            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], lg[i], tmp, w * esz, 0ull, s)
-                     : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], lg[i], tmp, w * esz, s);
+            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], geo[i].rows, tmp, w * esz, 0ull, s)
+                     : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], geo[i].rows, tmp, w * esz, s);
             if (e != cudaSuccess) return bail(e, "atlas pack launch");
             if ((e = cudaMemcpy2DToArrayAsync(arr, 0, 0, tmp, w * esz, w * esz, h, cudaMemcpyDeviceToDevice, s)) !=
                 cudaSuccess)
@@ -743,8 +789,7 @@ int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
             return bail(e, "cudaCreateTextureObject (slice atlas)");
         cb->atlas_tex[i] = t;
         cb->atlas_bytes += w * h * esz;
-        cb->tmpl[i].atlas = t;
-        cb->tmpl[i].alog = lg[i];
+        set_atlas(cb->tmpl[i], t, geo[i].rows, 0, 0);
     }
     e = cudaStreamSynchronize(s);
     for (auto sf : surfs) cudaDestroySurfaceObject(sf);

@@ -126,120 +126,81 @@ cudaError_t launch_brick_maxabs(const float *cube, int nx, int ny, int nz, const
     return cudaGetLastError();
 }
 
-// Slice atlas: element (x, y, z) of the x-contiguous brick goes to atlas column
-// (z & (2^alog - 1)) dx + x, row (z >> alog) dy + y.  Raw bits are moved (codes stay codes).
-template <typename T>
-__global__ void k_atlas_pack(const T *__restrict__ src, int dx, int dy, int dz, int alog, char *atlas,
-                             size_t pitch) {
-    const long long n = (long long)dx * dy * dz;
-    const int cm = (1 << alog) - 1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % dx);
-        const long long r = i / dx;
-        const int y = (int)(r % dy), z = (int)(r / dy);
-        const size_t row = (size_t)(z >> alog) * dy + y, col = (size_t)(z & cm) * dx + x;
-        reinterpret_cast<T *>(atlas + row * pitch)[col] = src[i];
+// Atlas placement: slice z of the x-contiguous brick is row z mod K (rows = K) of column z / K; a
+// slice that heads a later column is also stored below the column before it, so the slices iz
+// and iz + 1 of any sample stand one below the other.  One CTA per strip of brick rows; raw
+// bits are moved (codes stay codes).  PAIR: 32-bit texels of the codes at z and z + 1, no copies.
+template <typename T, bool PAIR>
+struct PackSrc {
+    const T *src;
+    int dx, dy;
+    __device__ __forceinline__ auto get(size_t row, int x) const {
+        if constexpr (PAIR)
+            return (unsigned int)src[row * dx + x] | ((unsigned int)src[(row + dy) * dx + x] << 16);
+        else
+            return src[row * dx + x];
     }
-}
-
-// The same placement written straight into the atlas array through a surface (no staging, no
-// array copy).  Coordinates are in range by construction; the zero boundary mode makes any
+};
+struct PackLinear {
+    char *atlas;
+    size_t pitch;
+    template <typename V>
+    __device__ __forceinline__ void put(V v, int col, int row) const {
+        reinterpret_cast<V *>(atlas + (size_t)row * pitch)[col] = v;
+    }
+};
+// Through a surface: coordinates are in range by construction; the zero boundary mode makes any
 // write outside the array a no-op rather than a fault.
-template <typename T>
-__global__ void k_atlas_pack_surf(const T *__restrict__ src, int dx, int dy, int dz, int alog,
-                                  cudaSurfaceObject_t surf) {
-    const long long n = (long long)dx * dy * dz;
-    const int cm = (1 << alog) - 1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % dx);
-        const long long r = i / dx;
-        const int y = (int)(r % dy), z = (int)(r / dy);
-        const int row = (z >> alog) * dy + y, col = (z & cm) * dx + x;
-        surf2Dwrite<T>(src[i], surf, col * (int)sizeof(T), row, cudaBoundaryModeZero);
+struct PackSurf {
+    cudaSurfaceObject_t surf;
+    template <typename V>
+    __device__ __forceinline__ void put(V v, int col, int row) const {
+        surf2Dwrite<V>(v, surf, col * (int)sizeof(V), row, cudaBoundaryModeZero);
+    }
+};
+template <typename T, bool PAIR, typename Dst>
+__global__ void __launch_bounds__(256) k_atlas_pack(PackSrc<T, PAIR> src, int dx, int dy, int nt, int rows, Dst dst) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n = (long long)dy * nt;
+    for (long long r = (long long)blockIdx.x * 8 + warp; r < n; r += (long long)gridDim.x * 8) {
+        const int z = (int)(r / dy), y = (int)(r - (long long)z * dy);
+        const int c = z / rows, zr = z - c * rows;
+        const bool twice = !PAIR && zr == 0 && c > 0;
+        for (int x = lane; x < dx; x += 32) {
+            const auto v = src.get((size_t)r, x);
+            dst.put(v, c * dx + x, zr * dy + y);
+            if (twice) dst.put(v, (c - 1) * dx + x, rows * dy + y);
+        }
     }
 }
 
-cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int alog,
+template <typename T, bool PAIR, typename Dst>
+static cudaError_t pack(const void *brick, int dx, int dy, int nt, int rows, Dst dst, cudaStream_t s) {
+    const long long n = (long long)dy * nt;
+    if (n <= 0 || dx <= 0) return cudaSuccess;
+    const int grid = (int)std::min<long long>((n + 7) / 8, 152 * 8);
+    k_atlas_pack<T, PAIR, Dst><<<grid, 256, 0, s>>>(PackSrc<T, PAIR>{static_cast<const T *>(brick), dx, dy}, dx, dy, nt, rows, dst);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows,
                                    unsigned long long surf, cudaStream_t s) {
-    const long long n = (long long)dx * dy * dz;
-    if (n <= 0) return cudaSuccess;
-    const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-    if (esz == 4)
-        k_atlas_pack_surf<unsigned int><<<grid, 256, 0, s>>>(static_cast<const unsigned int *>(brick), dx, dy, dz,
-                                                             alog, (cudaSurfaceObject_t)surf);
-    else
-        k_atlas_pack_surf<unsigned short><<<grid, 256, 0, s>>>(static_cast<const unsigned short *>(brick), dx, dy,
-                                                               dz, alog, (cudaSurfaceObject_t)surf);
-    return cudaGetLastError();
+    const PackSurf d{(cudaSurfaceObject_t)surf};
+    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, d, s)
+                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, d, s);
 }
 
-cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int alog, void *atlas,
+cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, void *atlas,
                               size_t pitch, cudaStream_t s) {
-    const long long n = (long long)dx * dy * dz;
-    if (n <= 0) return cudaSuccess;
-    const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-    if (esz == 4)
-        k_atlas_pack<unsigned int><<<grid, 256, 0, s>>>(static_cast<const unsigned int *>(brick), dx, dy, dz,
-                                                        alog, static_cast<char *>(atlas), pitch);
-    else
-        k_atlas_pack<unsigned short><<<grid, 256, 0, s>>>(static_cast<const unsigned short *>(brick), dx, dy,
-                                                          dz, alog, static_cast<char *>(atlas), pitch);
-    return cudaGetLastError();
+    const PackLinear d{static_cast<char *>(atlas), pitch};
+    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, d, s)
+                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, d, s);
 }
 
-// Pair atlas of a 16-bit brick: texel (x, y) of tile z (z < dz - 1), placed at column
-// (z & (2^alog - 1)) dx + x, row (z >> alog) dy + y, holds the code of element (x, y, z) in its
-// low half and that of (x, y, z + 1) in its high half.
-__device__ __forceinline__ void pair_texel(const unsigned short *src, int dx, int dy, int dz, int alog, long long i,
-                                           unsigned int &val, int &col, int &row) {
-    const int x = (int)(i % dx);
-    const long long r = i / dx;
-    const int y = (int)(r % dy), z = (int)(r / dy);
-    const size_t e = ((size_t)z * dy + y) * dx + x;
-    val = (unsigned int)src[e] | ((unsigned int)src[e + (size_t)dx * dy] << 16);
-    col = (z & ((1 << alog) - 1)) * dx + x;
-    row = (z >> alog) * dy + y;
-}
-
-__global__ void k_pair_pack(const unsigned short *__restrict__ src, int dx, int dy, int dz, int alog, char *atlas,
-                            size_t pitch) {
-    const long long n = (long long)dx * dy * (dz - 1);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        unsigned int v;
-        int col, row;
-        pair_texel(src, dx, dy, dz, alog, i, v, col, row);
-        reinterpret_cast<unsigned int *>(atlas + (size_t)row * pitch)[col] = v;
-    }
-}
-
-// The same through a surface (zero boundary mode: a write outside the array is a no-op).
-__global__ void k_pair_pack_surf(const unsigned short *__restrict__ src, int dx, int dy, int dz, int alog,
-                                 cudaSurfaceObject_t surf) {
-    const long long n = (long long)dx * dy * (dz - 1);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        unsigned int v;
-        int col, row;
-        pair_texel(src, dx, dy, dz, alog, i, v, col, row);
-        surf2Dwrite<unsigned int>(v, surf, col * (int)sizeof(unsigned int), row, cudaBoundaryModeZero);
-    }
-}
-
-cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int alog, void *atlas, size_t pitch,
+cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
                              unsigned long long surf, cudaStream_t s) {
-    const long long n = (long long)dx * dy * (dz - 1);
-    if (n <= 0) return cudaSuccess;
-    const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-    if (surf)
-        k_pair_pack_surf<<<grid, 256, 0, s>>>(static_cast<const unsigned short *>(brick), dx, dy, dz, alog,
-                                              (cudaSurfaceObject_t)surf);
-    else
-        k_pair_pack<<<grid, 256, 0, s>>>(static_cast<const unsigned short *>(brick), dx, dy, dz, alog,
-                                         static_cast<char *>(atlas), pitch);
-    return cudaGetLastError();
+    return surf ? pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackSurf{(cudaSurfaceObject_t)surf}, s)
+                : pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackLinear{static_cast<char *>(atlas), pitch}, s);
 }
 
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,

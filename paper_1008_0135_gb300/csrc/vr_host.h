@@ -92,6 +92,8 @@ struct Cube {
     std::vector<cudaArray_t> atlas_arr;          // per brick (layout bit 3)
     std::vector<unsigned long long> atlas_tex;   // texture objects over them
     size_t atlas_bytes = 0;
+    bool atlas_fit = true;             // (layout bit 3) the bricks' slices fit an array with the copies
+                                       // the columns carry; false: frames read the linear copy
     bool atlas_pair = false;           // the atlases are pair atlases (layout bit 5, 16-bit bricks)
     // streamed cubes: bricks are produced on the host and cached in HBM on demand
     bool streamed = false;
@@ -214,6 +216,17 @@ struct FrameLayout {
     int atlas;                        // 1: the ray caster gathers from the slice atlases
 };
 FrameLayout frame_layout(const vr_ctx *c, const Cube *cb);
+// How far a ray that meets the cube can reach from its origin: |camera - cube centre| + diagonal.
+double ray_reach(const vr_ctx *c, const Cube *cb);
+// Slice atlases: an array of w x h texels with columns of `rows` slices.
+struct AtlasGeom {
+    int rows = 0, w = 0, h = 0;
+};
+// The atlas of a stored brick of dim[0] x dim[1] x dim[2] (pair: pair atlas) on the current
+// device.  VR_ERR_UNSUPPORTED beyond the 2D-gather size.
+int atlas_geom(int device, const int dim[3], bool pair, AtlasGeom &g);
+// Puts an atlas (its texture, rows a column, corner in the array) in a brick's record.
+void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0);
 // Strides of the copy of a dim[0] x dim[1] x dim[2] brick whose axis a is contiguous, its rows
 // padded to a multiple of 16 bytes (esz-byte elements); returns the copy's elements.
 long long layout_strides_padded(const int dim[3], int a, int esz, int str[3]);

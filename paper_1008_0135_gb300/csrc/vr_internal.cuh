@@ -65,9 +65,14 @@ struct DrawBrick {
     long long frag_off;            // fragment offset (pixels) of the brick's sub-image
     long long bytes;               // stored bytes of the brick
     unsigned long long atlas;      // texture object over the brick's slice atlas (0: none): a 2D
-                                   // array whose tile (z & (2^alog - 1), z >> alog) of dim[0] x
-                                   // dim[1] texels holds stored slice z (FP32 values or 16-bit codes)
-    int alog;
+                                   // array in which the stored slices (FP32 values or 16-bit
+                                   // codes, dim[0] x dim[1] texels) stand below one another in
+                                   // columns of K, each column but the last followed by a copy of
+                                   // the next one's first slice (pair atlases: no copies)
+    float at_org[2];               // 1 + the first column's corner in the array
+    float at_dim[2];               // dim[0], dim[1]
+    float at_inv, at_neg;          // 1 / K rounded up, -K
+    int at_rows;                   // K
     int skip;                      // global termination: every sample of this brick adds nothing
                                    // (its values map only to zero opacity), walk through it
     long long pad_off;             // staged frames (fetch 4): element offset of the brick's copy
@@ -105,16 +110,17 @@ cudaError_t launch_minmax(const float *v, long long n, unsigned int *enc_minmax,
 cudaError_t launch_brick_maxabs(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                 int nbricks, unsigned int *maxbits, unsigned int *range,
                                 cudaStream_t s);
-// Packs one x-contiguous stored brick (dx*dy*dz elements of esz = 4 or 2 bytes) into a
-// pitch-linear slice atlas of (2^alog dx) x (ceil(dz / 2^alog) dy) elements, row pitch `pitch` bytes.
-cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int alog, void *atlas,
+// Packs one x-contiguous stored brick (dx*dy*dz elements of esz = 4 or 2 bytes) into its slice
+// atlas (columns of `rows` slices, placed as DrawBrick::atlas says): into a pitch-linear
+// buffer of row pitch `pitch` bytes, or through a surface.
+cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, void *atlas,
                               size_t pitch, cudaStream_t s);
-cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int alog,
+cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows,
                                    unsigned long long surf, cudaStream_t s);
 // Packs one x-contiguous 16-bit brick into its pair atlas (dz - 1 tiles of dx x dy 32-bit
-// texels, placed like the slice atlas's tiles): through surface `surf` when non-zero, else into
+// texels in columns of `rows`): through surface `surf` when non-zero, else into
 // the pitch-linear `atlas` of row pitch `pitch` bytes.
-cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int alog, void *atlas, size_t pitch,
+cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
                              unsigned long long surf, cudaStream_t s);
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                int nbricks, const unsigned int *maxbits, int storage, void *pool,

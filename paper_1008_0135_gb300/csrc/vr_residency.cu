@@ -258,7 +258,7 @@ struct Slot {
     cudaArray_t arr = nullptr;
     cudaTextureObject_t tex = 0;
     cudaSurfaceObject_t surf = 0;     // packs write the array through it (0: staging + copy)
-    int arr_storage = -1, arr_w = 0, arr_h = 0, alog = 0;
+    int arr_storage = -1, arr_w = 0, arr_h = 0, rows = 0;
     bool atlas_ok = false;            // the atlas holds this slot's brick
 };
 
@@ -567,32 +567,18 @@ static std::shared_ptr<BrickJob> produce_brick(Workers *pool, Cube *cb, const Dr
 }
 
 // Slice atlases of cache slots (streamed and compressed cubes whose layout mask has bit 3):
-// every brick of a cube uses the tile layout of the cube's largest stored brick (2^alog
-// z-slices per atlas row), so any of its bricks fits a slot's array.
-struct SlotAtlasGeom {
-    int w = 0, h = 0, alog = 0;
-};
-
-static int slot_atlas_geom(vr_ctx *c, Cube *cb, SlotAtlasGeom &g) {
+// every brick of a cube uses the columns of the cube's largest stored brick, so any of its
+// bricks fits a slot's array.
+static int slot_atlas_geom(vr_ctx *c, Cube *cb, AtlasGeom &g) {
     int mx[3] = {0, 0, 0};
     for (auto &b : cb->tmpl)
         for (int a = 0; a < 3; ++a) mx[a] = std::max(mx[a], b.dim[a]);
-    int l = 0;
-    while ((1ll << (2 * l)) < mx[2]) ++l;
-    const long long w = (long long)mx[0] << l, h = (long long)((mx[2] + (1 << l) - 1) >> l) * mx[1];
-    int gw = 0, gh = 0;
-    CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, c->device));
-    CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, c->device));
-    if (w > gw || h > gh) return fail(VR_ERR_UNSUPPORTED, "bricks too large for a slice atlas (2D gather limit)");
-    g.w = (int)w;
-    g.h = (int)h;
-    g.alog = l;
-    return VR_OK;
+    return atlas_geom(c->device, mx, false, g);
 }
 
 // Gives slot `si` an atlas array for cube `cb`'s bricks, creating or replacing it when it has
 // another texel type or is too small (after every reader and pending copy of the old one).
-static int slot_atlas_alloc(vr_ctx *c, Cube *cb, int si, const SlotAtlasGeom &g) {
+static int slot_atlas_alloc(vr_ctx *c, Cube *cb, int si, const AtlasGeom &g) {
     BrickCache *k = c->cache;
     Slot &s = k->slots[si];
     const size_t esz = cb->storage == VR_F32 ? 4 : 2;
@@ -643,7 +629,7 @@ static int slot_atlas_alloc(vr_ctx *c, Cube *cb, int si, const SlotAtlasGeom &g)
 
 // Packs slot `si`'s brick `b` (already queued into the slot on the copy stream) into the slot's
 // atlas on the copy stream.
-static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, const SlotAtlasGeom &g) {
+static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, const AtlasGeom &g) {
     BrickCache *k = c->cache;
     Slot &s = k->slots[si];
     const size_t esz = cb->storage == VR_F32 ? 4 : 2;
@@ -651,8 +637,8 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
     if (rc != VR_OK) return rc;
     if (s.surf) {
         CK(launch_atlas_pack_surf(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2],
-                                  g.alog, (unsigned long long)s.surf, k->copy));
-        s.alog = g.alog;
+                                  g.rows, (unsigned long long)s.surf, k->copy));
+        s.rows = g.rows;
         s.atlas_ok = true;
         return VR_OK;
     }
@@ -665,11 +651,12 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
         CK(cudaMalloc(&k->pack_tmp, need));
         k->pack_bytes = need;
     }
-    const size_t w = (size_t)b.dim[0] << g.alog, h = (size_t)((b.dim[2] + (1 << g.alog) - 1) >> g.alog) * b.dim[1];
-    CK(launch_atlas_pack(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2], g.alog,
+    const int cols = (b.dim[2] + g.rows - 1) / g.rows;
+    const size_t w = (size_t)cols * b.dim[0], h = (size_t)(cols > 1 ? g.rows + 1 : b.dim[2]) * b.dim[1];
+    CK(launch_atlas_pack(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2], g.rows,
                          k->pack_tmp, w * esz, k->copy));
     CK(cudaMemcpy2DToArrayAsync(s.arr, 0, 0, k->pack_tmp, w * esz, w * esz, h, cudaMemcpyDeviceToDevice, k->copy));
-    s.alog = g.alog;
+    s.rows = g.rows;
     s.atlas_ok = true;
     return VR_OK;
 }
@@ -681,10 +668,10 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
                          int64_t chunk) {
     BrickCache *k = c->cache;
     const size_t esz = cb->storage == VR_F32 ? 4 : 2;
-    const bool atlas = (cb->layouts & 8) != 0;
-    SlotAtlasGeom g;
+    AtlasGeom g;
     int rc = VR_OK;
-    if (atlas && (rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
+    if ((cb->layouts & 8) && (rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
+    const bool atlas = (cb->layouts & 8) && g.rows > 0;
     std::vector<std::pair<size_t, int>> misses;   // (db index, slot)
     for (size_t i = d0; i < d1; ++i) {
         auto it = k->where.find(key_of(cb->id, db[i].brick));
@@ -697,8 +684,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
             db[i].atlas = 0ull;
             if (atlas) {
                 if (!s.atlas_ok && (rc = slot_atlas_pack(c, cb, it->second, db[i], g)) != VR_OK) return rc;
-                db[i].atlas = s.tex;
-                db[i].alog = s.alog;
+                set_atlas(db[i], s.tex, s.rows, 0, 0);
             }
             k->hits++;
         } else {
@@ -755,8 +741,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
                     s.chunk = -1;
                     return rc;
                 }
-                db[mi.first].atlas = s.tex;
-                db[mi.first].alog = s.alog;
+                set_atlas(db[mi.first], s.tex, s.rows, 0, 0);
             }
         }
         return VR_OK;
@@ -833,8 +818,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
                 s.chunk = -1;
                 break;
             }
-            db[misses[m].first].atlas = s.tex;
-            db[misses[m].first].alog = s.alog;
+            set_atlas(db[misses[m].first], s.tex, s.rows, 0, 0);
         }
     }
     if (rc != VR_OK) {
@@ -1087,8 +1071,10 @@ int cache_prepare_atlases(vr_ctx *c, Cube *cb) {
     size_t max_bytes = 0;
     for (auto &b : cb->tmpl) max_bytes = std::max(max_bytes, (size_t)b.bytes);
     if ((rc = cache_size(c, max_bytes)) != VR_OK) return rc;
-    SlotAtlasGeom g;
+    AtlasGeom g;
     if ((rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
+    cb->atlas_fit = g.rows > 0;
+    if (!cb->atlas_fit) return VR_OK;        // frames read the slots' linear bricks
     const int n = (int)std::min<size_t>((size_t)k->nslots, cb->tmpl.size());
     for (int i = 0; i < n; ++i)
         if ((rc = slot_atlas_alloc(c, cb, i, g)) != VR_OK) return rc;
