@@ -687,98 +687,111 @@ int check_ready(vr_ctx *c, Cube *cb) {
     return VR_OK;
 }
 
+// Whether p is memory of device `dev` that a kernel there can read (another device's memory and host
+// memory registered or managed are left to the copy engine).
+bool own_device_memory(const void *p, int dev) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 // Releases a cube's slice atlases.  Frames in flight may still gather from them: the device is
-// drained first (atlases change only with the bricking or the voxels).
+// drained first (atlases go only with the bricking).
 void free_atlases(Cube *cb) {
     if (cb->atlas_arr.empty() && cb->atlas_tex.empty()) return;
     cudaDeviceSynchronize();
     for (auto t : cb->atlas_tex)
         if (t) cudaDestroyTextureObject(t);
+    for (auto f : cb->atlas_surf)
+        if (f) cudaDestroySurfaceObject(f);
     for (auto a : cb->atlas_arr)
         if (a) cudaFreeArray(a);
     cb->atlas_tex.clear();
+    cb->atlas_surf.clear();
     cb->atlas_arr.clear();
-    cb->atlas_bytes = 0;
+    cb->atlas_cells.clear();
+    cb->atlas_of.clear();
     cb->atlas_pair = false;
     for (auto &d : cb->tmpl) d.atlas = 0;
 }
 
-// Slice atlas of every brick (layout bit 3) from its x-contiguous copy in the pool, placed by
-// atlas_geom.  FP32 bricks keep their values, 16-bit bricks their codes (FP16 as half
-// texels, BF16 as 16-bit unsigned ones).  With layout bit 5, 16-bit bricks get pair atlases
-// instead: dz - 1 tiles of 32-bit texels, tile z holding the codes of slices z and z + 1 (one
-// gather per sample).  The array must fit the device's limit for 2D gathers.
-int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
+// Arrays for the slice atlas of every brick (layout bit 3), each brick's placed by
+// atlas_geom, several bricks to an array: an array costs the driver about 70 us to make and
+// free whatever its size (ingesting 120 bricks spent 8.3 of 12.6 ms there).  Bricks stand side
+// by side, tallest first, in shelves of at most kAtlasRowBytes (a brick wider than that alone).
+// Wider arrays spread a slice over more pages: 1720x1720x1024 FP32 frames take 3.41 ms with one
+// brick an array and with rows of 8 KB, 3.43 with 16 KB, 3.52 with 32 KB, 3.70 with 128 KB.
+// FP32 bricks keep their values, 16-bit bricks their codes (FP16 as half texels, BF16 as 16-bit
+// unsigned ones); with layout bit 5, 16-bit bricks get pair atlases instead: dz - 1 tiles of
+// 32-bit texels, tile z holding the codes of slices z and z + 1 (one gather per sample).
+// Arrays must fit the device's limit for 2D gathers.
+constexpr int kAtlasRowBytes = 8192;
+int make_atlases(vr_ctx *c, Cube *cb) {
     free_atlases(cb);
     const int nbr = (int)cb->tmpl.size();
     const bool pair = (cb->layouts & 32) && cb->storage != VR_F32;
-    const size_t bsz = cb->storage == VR_F32 ? 4 : 2;       // bytes of a stored element
-    const size_t esz = pair ? 4 : bsz;                       // bytes of a texel
     std::vector<AtlasGeom> geo(nbr);
-    size_t most = 16;
     cb->atlas_fit = true;
     for (int i = 0; i < nbr; ++i) {
         const int rc = atlas_geom(c->device, cb->tmpl[i].dim, pair, geo[i]);
         if (rc != VR_OK) return rc;
         if (geo[i].rows == 0) cb->atlas_fit = false;
-        most = std::max(most, (size_t)geo[i].w * geo[i].h * esz);
     }
     if (!cb->atlas_fit) return VR_OK;        // frames read the linear copy
-    void *tmp = nullptr;
-    CK(cudaMalloc(&tmp, most));
-    std::vector<cudaSurfaceObject_t> surfs;   // kept until the packs that write through them ran
+    int gw = 0, gh = 0;
+    CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, c->device));
+    CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, c->device));
+    gw = std::min(gw, kAtlasRowBytes / (pair || cb->storage == VR_F32 ? 4 : 2));
+    std::vector<int> ord(nbr);
+    for (int i = 0; i < nbr; ++i) ord[i] = i;
+    std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return geo[a].h > geo[b].h; });
+    struct Dim { int w, h; };
+    std::vector<Dim> dims;                   // of each array
+    cb->atlas_cells.assign(nbr, AtlasCell{0ull, 0, 0, 1});
+    cb->atlas_of.assign(nbr, 0);
+    int x = 0, y = 0, shelf = 0;
+    for (int i : ord) {
+        const AtlasGeom &g = geo[i];
+        if (!dims.empty() && x > 0 && x + g.w > gw) { x = 0; y += shelf; shelf = 0; }
+        if (dims.empty() || (x == 0 && y > 0 && y + g.h > gh) || x + g.w > std::max(gw, g.w)) {
+            dims.push_back(Dim{0, 0});
+            x = y = shelf = 0;
+        }
+        Dim &d = dims.back();
+        cb->atlas_cells[i] = AtlasCell{0ull, x, y, g.rows};
+        cb->atlas_of[i] = (int)dims.size() - 1;
+        x += g.w;
+        shelf = std::max(shelf, g.h);
+        d.w = std::max(d.w, x);
+        d.h = std::max(d.h, y + g.h);
+    }
+    const cudaChannelFormatDesc cd = pair ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
+                                   : cb->storage == VR_F32 ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindFloat)
+                                   : cb->storage == VR_F16 ? cudaCreateChannelDescHalf()
+                                                           : cudaCreateChannelDesc(16, 0, 0, 0, cudaChannelFormatKindUnsigned);
     auto bail = [&](cudaError_t e, const char *what) {
-        cudaStreamSynchronize(s);
-        for (auto sf : surfs) cudaDestroySurfaceObject(sf);
-        cudaFree(tmp);
         free_atlases(cb);
         return cuda_fail(e, what);
     };
-    cudaError_t e = cudaMemsetAsync(tmp, 0, most, s);
-    if (e != cudaSuccess) return bail(e, "cudaMemsetAsync");
-    // FP32 values; FP16 codes as half texels (gathers widen them to float exactly); BF16 codes as
-    // 16-bit unsigned texels (widened in the kernel)
-    // (pair atlases: two codes in one 32-bit unsigned texel, widened in the kernel)
-    const cudaChannelFormatDesc cd = pair ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
-                                   : esz == 4 ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindFloat)
-                                   : cb->storage == VR_F16 ? cudaCreateChannelDescHalf()
-                                                           : cudaCreateChannelDesc(16, 0, 0, 0, cudaChannelFormatKindUnsigned);
-    cb->atlas_arr.assign(nbr, nullptr);
-    cb->atlas_tex.assign(nbr, 0);
-    for (int i = 0; i < nbr; ++i) {
-        const int *dm = cb->tmpl[i].dim;
-        const size_t w = (size_t)geo[i].w, h = (size_t)geo[i].h;
+    cudaError_t e;
+    for (const Dim &d : dims) {
         cudaArray_t arr = nullptr;
-        // written by the pack kernel through a surface where the device allows surface stores on
-        // a gather array; else packed into staging and copied (the copy engine's array writes)
-        const bool surf_ok = cudaMallocArray(&arr, &cd, w, h, cudaArrayTextureGather | cudaArraySurfaceLoadStore) ==
-                             cudaSuccess;
+        // written through a surface where the device allows surface stores on a gather array; else
+        // packed into staging and copied (the copy engine's array writes)
+        const bool surf_ok = cudaMallocArray(&arr, &cd, d.w, d.h, cudaArrayTextureGather | cudaArraySurfaceLoadStore) == cudaSuccess;
         if (!surf_ok) {
             arr = nullptr;
             cudaGetLastError();
-            if ((e = cudaMallocArray(&arr, &cd, w, h, cudaArrayTextureGather)) != cudaSuccess)
+            if ((e = cudaMallocArray(&arr, &cd, d.w, d.h, cudaArrayTextureGather)) != cudaSuccess)
                 return bail(e, "cudaMallocArray (slice atlas)");
         }
-        cb->atlas_arr[i] = arr;
+        cb->atlas_arr.push_back(arr);
         cudaResourceDesc rd{};
         rd.resType = cudaResourceTypeArray;
         rd.res.array.array = arr;
-        const char *src = static_cast<const char *>(cb->d_pool) + (size_t)cb->loff[3 * (size_t)i] * bsz;
-        if (surf_ok) {
-            cudaSurfaceObject_t sf = 0;
-            if ((e = cudaCreateSurfaceObject(&sf, &rd)) != cudaSuccess) return bail(e, "cudaCreateSurfaceObject");
-            surfs.push_back(sf);
-            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], geo[i].rows, nullptr, 0, (unsigned long long)sf, s)
-                     : launch_atlas_pack_surf(src, (int)esz, dm[0], dm[1], dm[2], geo[i].rows, (unsigned long long)sf, s);
-            if (e != cudaSuccess) return bail(e, "atlas pack launch");
-        } else {
-            e = pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], geo[i].rows, tmp, w * esz, 0ull, s)
-                     : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], geo[i].rows, tmp, w * esz, s);
-            if (e != cudaSuccess) return bail(e, "atlas pack launch");
-            if ((e = cudaMemcpy2DToArrayAsync(arr, 0, 0, tmp, w * esz, w * esz, h, cudaMemcpyDeviceToDevice, s)) !=
-                cudaSuccess)
-                return bail(e, "cudaMemcpy2DToArrayAsync (slice atlas)");
-        }
         cudaTextureDesc td{};
         td.addressMode[0] = td.addressMode[1] = cudaAddressModeClamp;
         td.filterMode = cudaFilterModePoint;
@@ -787,79 +800,118 @@ int build_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
         cudaTextureObject_t t = 0;
         if ((e = cudaCreateTextureObject(&t, &rd, &td, nullptr)) != cudaSuccess)
             return bail(e, "cudaCreateTextureObject (slice atlas)");
-        cb->atlas_tex[i] = t;
-        cb->atlas_bytes += w * h * esz;
-        set_atlas(cb->tmpl[i], t, geo[i].rows, 0, 0);
+        cb->atlas_tex.push_back(t);
+        cudaSurfaceObject_t sf = 0;
+        if (surf_ok && (e = cudaCreateSurfaceObject(&sf, &rd)) != cudaSuccess) return bail(e, "cudaCreateSurfaceObject");
+        cb->atlas_surf.push_back((unsigned long long)sf);
     }
-    e = cudaStreamSynchronize(s);
-    for (auto sf : surfs) cudaDestroySurfaceObject(sf);
-    cudaFree(tmp);
-    if (e != cudaSuccess) {
-        free_atlases(cb);
-        return cuda_fail(e, "slice atlas build");
+    for (int i = 0; i < nbr; ++i) {
+        AtlasCell &cell = cb->atlas_cells[i];
+        cell.surf = cb->atlas_surf[cb->atlas_of[i]];
+        set_atlas(cb->tmpl[i], cb->atlas_tex[cb->atlas_of[i]], cell.rows, cell.x0, cell.y0);
     }
     cb->atlas_pair = pair;
     return VR_OK;
 }
 
+// The atlases from the pool's x-contiguous copies, through staging: where the device refuses
+// surface stores on a gather array.
+int stage_atlases(Cube *cb, cudaStream_t s) {
+    const size_t bsz = cb->storage == VR_F32 ? 4 : 2;        // bytes of a stored element
+    const size_t esz = cb->atlas_pair ? 4 : bsz;             // bytes of a texel
+    size_t most = 16;
+    auto extent = [&](size_t i, size_t &w, size_t &h) {
+        const int *dm = cb->tmpl[i].dim, rows = cb->atlas_cells[i].rows, nt = cb->atlas_pair ? dm[2] - 1 : dm[2];
+        const int cols = (nt + rows - 1) / rows;
+        w = (size_t)cols * dm[0];
+        h = (size_t)(cols > 1 ? rows + (cb->atlas_pair ? 0 : 1) : nt) * dm[1];
+    };
+    size_t w, h;
+    for (size_t i = 0; i < cb->tmpl.size(); ++i) {
+        extent(i, w, h);
+        most = std::max(most, w * h * esz);
+    }
+    void *tmp = nullptr;
+    CK(cudaMalloc(&tmp, most));
+    cudaError_t e = cudaMemsetAsync(tmp, 0, most, s);
+    for (size_t i = 0; i < cb->tmpl.size() && e == cudaSuccess; ++i) {
+        const AtlasCell &cell = cb->atlas_cells[i];
+        if (cell.surf) continue;
+        const int *dm = cb->tmpl[i].dim;
+        extent(i, w, h);
+        const char *src = static_cast<const char *>(cb->d_pool) + (size_t)cb->loff[3 * i] * bsz;
+        e = cb->atlas_pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, 0ull, s)
+                           : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpy2DToArrayAsync(cb->atlas_arr[cb->atlas_of[i]], (size_t)cell.x0 * esz, cell.y0, tmp, w * esz, w * esz,
+                                         h, cudaMemcpyDeviceToDevice, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(tmp);
+    if (e != cudaSuccess) {
+        free_atlases(cb);
+        return cuda_fail(e, "slice atlas build");
+    }
+    return VR_OK;
+}
+
+// (Re)builds every kept copy of the bricks from the cube's voxels; returns once it is done.  The
+// atlas arrays are made on the first build of a bricking and written again by later ones
+// (vr_update_cube).  One pass over the voxels for max |v| and the value ranges, one that writes the
+// x-contiguous copies and the atlases, one more per further copy; the host waits once, for the
+// ranges and exponents.
 int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
     const int nbr = (int)cb->tmpl.size();
+    int rc;
+    if (!(cb->layouts & 8)) free_atlases(cb);
+    else if (cb->atlas_arr.empty()) { if ((rc = make_atlases(c, cb)) != VR_OK) return rc; }
+    else CK(cudaDeviceSynchronize());        // frames in flight may still gather from the arrays
+    const bool atlas = !cb->atlas_arr.empty();
+    const bool surf = atlas && cb->atlas_surf[0] != 0;
     unsigned int *d_range = cb->d_bs + 2 * (size_t)nbr;
-    // max |v| (16-bit scales) and the value range (empty-space skipping) of every brick
-    CK(cudaMemsetAsync(cb->d_bs, 0, sizeof(unsigned int) * nbr, s));
-    {
-        std::vector<unsigned int> init(2 * (size_t)nbr);
-        for (int i = 0; i < nbr; ++i) { init[2 * i] = 0xffffffffu; init[2 * i + 1] = 0u; }
-        CK(cudaMemcpyAsync(d_range, init.data(), sizeof(unsigned int) * 2 * nbr, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(cb->d_tmpl, cb->tmpl.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice, s));
-        CK(launch_brick_maxabs(cb->d_src, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], cb->d_tmpl, nbr, cb->d_bs,
-                               d_range, s));
-        std::vector<unsigned int> r(2 * (size_t)nbr);
-        CK(cudaMemcpyAsync(r.data(), d_range, sizeof(unsigned int) * 2 * nbr, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        auto dec = [](unsigned int e) {
-            unsigned int b = (e & 0x80000000u) ? (e & 0x7fffffffu) : ~e;
-            float f;
-            std::memcpy(&f, &b, 4);
-            return f;
-        };
-        cb->vlo.resize(nbr);
-        cb->vhi.resize(nbr);
-        for (int i = 0; i < nbr; ++i) { cb->vlo[i] = dec(r[2 * i]); cb->vhi[i] = dec(r[2 * i + 1]); }
-    }
     int *d_exps = reinterpret_cast<int *>(cb->d_bs + nbr);
-    // one build per kept layout: the records carry that layout's offsets and strides
+    AtlasCell *d_cells = reinterpret_cast<AtlasCell *>(cb->d_tmpl + nbr);
+    const int nx = (int)cb->n[0], ny = (int)cb->n[1], nz = (int)cb->n[2];
+    // max |v| (16-bit scales), exponents and the value range (empty-space skipping) of every brick
+    std::vector<unsigned int> bs(4 * (size_t)nbr, 0u);
+    for (int i = 0; i < nbr; ++i) bs[2 * (size_t)nbr + 2 * i] = 0xffffffffu;
+    CK(cudaMemcpyAsync(cb->d_bs, bs.data(), sizeof(unsigned int) * bs.size(), cudaMemcpyHostToDevice, s));
+    if (surf)
+        CK(cudaMemcpyAsync(d_cells, cb->atlas_cells.data(), sizeof(AtlasCell) * nbr, cudaMemcpyHostToDevice, s));
+    // one build per kept copy: the records carry its offsets and strides
     std::vector<DrawBrick> rec(cb->tmpl);
-    for (int a = 0; a < 3; ++a) {
-        if (!(cb->layouts & (1 << a))) continue;
-        for (int i = 0; i < nbr; ++i) {
-            rec[i].data_off = cb->loff[3 * (size_t)i + a];
-            layout_strides(rec[i].dim, a, rec[i].str);
+    bool first = true;
+    for (int pad = 0; pad < 2; ++pad)
+        for (int a = 0; a < 3; ++a) {
+            if (pad ? (cb->loff_pad.empty() || cb->loff_pad[a] < 0) : !(cb->layouts & (1 << a))) continue;
+            for (int i = 0; i < nbr; ++i) {
+                rec[i].data_off = (pad ? cb->loff_pad : cb->loff)[3 * (size_t)i + a];
+                if (pad) layout_strides_padded(rec[i].dim, a, cb->storage == VR_F32 ? 4 : 2, rec[i].str);
+                else layout_strides(rec[i].dim, a, rec[i].str);
+            }
+            if (!first) CK(cudaStreamSynchronize(s));      // the last build has read its records
+            CK(cudaMemcpyAsync(cb->d_tmpl, rec.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice, s));
+            if (first) CK(launch_brick_maxabs(cb->d_src, nx, ny, nz, cb->d_tmpl, nbr, cb->d_bs, d_range, s));
+            CK(launch_brick_build(cb->d_src, nx, ny, nz, cb->d_tmpl, nbr, cb->d_bs, cb->storage, cb->d_pool, d_exps,
+                                  first && surf ? d_cells : nullptr, cb->atlas_pair, s));
+            first = false;
         }
-        CK(cudaMemcpyAsync(cb->d_tmpl, rec.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice, s));
-        CK(launch_brick_build(cb->d_src, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], cb->d_tmpl, nbr, cb->d_bs,
-                              cb->storage, cb->d_pool, d_exps, s));
-        CK(cudaStreamSynchronize(s));      // rec is rewritten for the next layout
+    CK(cudaMemcpyAsync(bs.data(), cb->d_bs, sizeof(unsigned int) * bs.size(), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    auto dec = [](unsigned int e) {
+        unsigned int b = (e & 0x80000000u) ? (e & 0x7fffffffu) : ~e;
+        float f;
+        std::memcpy(&f, &b, 4);
+        return f;
+    };
+    cb->vlo.resize(nbr);
+    cb->vhi.resize(nbr);
+    for (int i = 0; i < nbr; ++i) {
+        cb->vlo[i] = dec(bs[2 * (size_t)nbr + 2 * i]);
+        cb->vhi[i] = dec(bs[2 * (size_t)nbr + 2 * i + 1]);
+        if (cb->storage != VR_F32) cb->tmpl[i].exp2 = (int)bs[(size_t)nbr + i];
     }
-    for (int a = 0; a < 3 && !cb->loff_pad.empty(); ++a) {
-        if (cb->loff_pad[a] < 0) continue;
-        for (int i = 0; i < nbr; ++i) {
-            rec[i].data_off = cb->loff_pad[3 * (size_t)i + a];
-            layout_strides_padded(rec[i].dim, a, cb->storage == VR_F32 ? 4 : 2, rec[i].str);
-        }
-        CK(cudaMemcpyAsync(cb->d_tmpl, rec.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice, s));
-        CK(launch_brick_build(cb->d_src, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], cb->d_tmpl, nbr, cb->d_bs,
-                              cb->storage, cb->d_pool, d_exps, s));
-        CK(cudaStreamSynchronize(s));
-    }
-    if (cb->storage != VR_F32) {
-        std::vector<int> e(nbr);
-        CK(cudaMemcpyAsync(e.data(), d_exps, sizeof(int) * nbr, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        for (int i = 0; i < nbr; ++i) cb->tmpl[i].exp2 = e[i];
-    }
-    if (cb->layouts & 8) return build_atlases(c, cb, s);
-    free_atlases(cb);
+    if (atlas && !surf) return stage_atlases(cb, s);
     return VR_OK;
 }
 
@@ -1237,6 +1289,15 @@ static int vr_load_cube_body(vr_ctx *c, const void *voxels, int dtype, int64_t n
         free_cube(cb);
         return cuda_fail(e, "cudaDeviceSynchronize (device cube source)");
     }
+    if (where == VR_DEVICE && !sub_origin && own_device_memory(voxels, c->device)) {
+        // the whole array: one linear pass (the 3D copy below moves device memory at a quarter of HBM's rate)
+        e = launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)nx * ny * nz, c->load_stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->load_stream);
+        if (e != cudaSuccess) { free_cube(cb); return cuda_fail(e, "copy of the cube"); }
+        cb->id = *cube_id = c->next_id++;
+        c->cubes[cb->id] = cb;
+        return VR_OK;
+    }
     // 3D copy of the box: rows of ext[0] floats
     cudaMemcpy3DParms p{};
     p.srcPtr = make_cudaPitchedPtr(const_cast<void *>(voxels), sizeof(float) * nx, nx, ny);
@@ -1302,7 +1363,8 @@ static int vr_update_cube_body(vr_ctx *c, int cube_id, const void *voxels, int w
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t bytes = sizeof(float) * (size_t)cb->n[0] * cb->n[1] * cb->n[2];
     if (c->frame_pending) CK(cudaStreamWaitEvent(s, c->frame_done, 0));
-    CK(cudaMemcpyAsync(cb->d_src, voxels, bytes, where == VR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
+    if (where == VR_DEVICE && own_device_memory(voxels, c->device)) CK(launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)(bytes / sizeof(float)), s));
+    else CK(cudaMemcpyAsync(cb->d_src, voxels, bytes, where == VR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
     if (cb->bricked) return build_bricks(c, cb, s);
     CK(cudaStreamSynchronize(s));
     return VR_OK;
@@ -1421,6 +1483,7 @@ static int vr_set_bricking_body(vr_ctx *c, int cube_id, int bx, int by, int bz, 
         }
     }
     for (int64_t bi = 0; bi < nbr; ++bi) t[bi].data_off = loff[3 * bi];
+    free_atlases(cb);
     if (cb->d_pool) { cudaFree(cb->d_pool); cb->d_pool = nullptr; }
     if (cb->d_tmpl) { cudaFree(cb->d_tmpl); cb->d_tmpl = nullptr; }
     cb->bricked = false;
@@ -1437,8 +1500,7 @@ static int vr_set_bricking_body(vr_ctx *c, int cube_id, int bx, int by, int bz, 
     }
     CK(cudaMalloc(&cb->d_pool, std::max<size_t>(off * esz, 16)));
     cb->pool_bytes = off * esz;
-    CK(cudaMalloc(&cb->d_tmpl, sizeof(DrawBrick) * nbr));
-    CK(cudaMemcpy(cb->d_tmpl, t.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice));
+    CK(cudaMalloc(&cb->d_tmpl, (sizeof(DrawBrick) + sizeof(AtlasCell)) * nbr));   // records, then atlas cells
     if (cb->d_bs) { cudaFree(cb->d_bs); cb->d_bs = nullptr; }
     CK(cudaMalloc(&cb->d_bs, sizeof(unsigned int) * 4 * nbr));
     cb->tmpl = std::move(t);

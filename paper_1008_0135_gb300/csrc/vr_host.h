@@ -89,9 +89,12 @@ struct Cube {
     // layout bit 4: each kept linear copy again with its rows padded to 16 bytes (staged frames
     // copy rows of it into shared memory): offset of brick b's padded copy along a
     std::vector<long long> loff_pad;
-    std::vector<cudaArray_t> atlas_arr;          // per brick (layout bit 3)
-    std::vector<unsigned long long> atlas_tex;   // texture objects over them
-    size_t atlas_bytes = 0;
+    // (layout bit 3) arrays holding the bricks' atlases, several to an array, with a texture and,
+    // where the device allows it, a surface object over each; cells: where each brick's is
+    std::vector<cudaArray_t> atlas_arr;
+    std::vector<unsigned long long> atlas_tex, atlas_surf;
+    std::vector<AtlasCell> atlas_cells;
+    std::vector<int> atlas_of;         // brick -> array
     bool atlas_fit = true;             // (layout bit 3) the bricks' slices fit an array with the copies
                                        // the columns carry; false: frames read the linear copy
     bool atlas_pair = false;           // the atlases are pair atlases (layout bit 5, 16-bit bricks)

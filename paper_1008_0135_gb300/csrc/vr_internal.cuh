@@ -105,11 +105,19 @@ struct Counters {                  // device-side cumulative counters
 // ---------------------------------------------------------------------------------------------
 // launchers (return cudaError_t of the launch)
 // ---------------------------------------------------------------------------------------------
+// A device-to-device copy of n floats, ordered on s.
+cudaError_t launch_copy(const float *src, float *dst, long long n, cudaStream_t s);
 cudaError_t launch_minmax(const float *v, long long n, unsigned int *enc_minmax,
                           cudaStream_t s);
 cudaError_t launch_brick_maxabs(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                 int nbricks, unsigned int *maxbits, unsigned int *range,
                                 cudaStream_t s);
+// Where a brick's atlas is written: the surface over its array (0: none), the corner of its first
+// column and K, the slices a column.
+struct AtlasCell {
+    unsigned long long surf;
+    int x0, y0, rows;
+};
 // Packs one x-contiguous stored brick (dx*dy*dz elements of esz = 4 or 2 bytes) into its slice
 // atlas (columns of `rows` slices, placed as DrawBrick::atlas says): into a pitch-linear
 // buffer of row pitch `pitch` bytes, or through a surface.
@@ -122,9 +130,11 @@ cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, i
 // the pitch-linear `atlas` of row pitch `pitch` bytes.
 cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
                              unsigned long long surf, cudaStream_t s);
+// Writes every brick's stored region (records: geometry, data_off, str) into the pool, and, with
+// cells, into its atlas as well (pair: pair texels of 16-bit codes).
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                int nbricks, const unsigned int *maxbits, int storage, void *pool,
-                               int *exps, cudaStream_t s);
+                               int *exps, const AtlasCell *cells, bool pair, cudaStream_t s);
 cudaError_t launch_raycast(const FrameConsts &fc, const float4 *lut, const DrawBrick *db,
                            const TileItem *items, int nitems, const void *pool, void *frags,
                            Counters *ctr, cudaStream_t s);
