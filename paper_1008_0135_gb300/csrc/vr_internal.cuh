@@ -143,10 +143,22 @@ cudaError_t launch_raycast(const FrameConsts &fc, const float4 *lut, const DrawB
 constexpr int kWaveletRecordBytes = 544;
 cudaError_t launch_wavelet_encode(const float *cube, int nx, int ny, int nz, unsigned char *store,
                                   cudaStream_t s);
-// Decodes the stored region of one brick (global voxels clamp(org + [0, dim)), x-contiguous
-// FP32) from the block store.
-cudaError_t launch_wavelet_decode(const unsigned char *store, int nx, int ny, int nz, const int org[3],
-                                  const int dim[3], float *dst, cudaStream_t s);
+// Decodes the stored regions of up to kWaveletJobs bricks (global voxels clamp(org + [0, dim))) from
+// the block store: x-contiguous FP32 into dst, or (surf) into slice atlases with columns of `rows`
+// slices from (x0, y0) of the array behind the surface.  b0, nb: filled by the launcher.
+constexpr int kWaveletJobs = 16;
+struct WaveletJob {
+    int org[3], dim[3];
+    float *dst;
+    unsigned long long surf;
+    int x0, y0, rows;
+    int b0[3], nb[3];              // first block and blocks per axis the region touches
+};
+struct WaveletJobs {
+    WaveletJob job[kWaveletJobs];
+};
+cudaError_t launch_wavelet_decode(const unsigned char *store, int nx, int ny, int nz, WaveletJobs &jobs, int njobs, bool surf,
+                                  cudaStream_t s);
 // Global early termination: every pixel's ray walks the brick grid front to back in one
 // launch; premultiplied RGBA into out (W*H float4).  bricks: every brick of the cube in grid
 // order (x fastest), with the frame's layout offsets, atlases and skip flags.

@@ -260,6 +260,8 @@ struct Slot {
     cudaSurfaceObject_t surf = 0;     // packs write the array through it (0: staging + copy)
     int arr_storage = -1, arr_w = 0, arr_h = 0, rows = 0;
     bool atlas_ok = false;            // the atlas holds this slot's brick
+    bool linear_ok = false;           // the slot's linear copy holds it (a compressed cube's brick for
+                                      // atlas frames is decoded into the atlas alone)
 };
 
 struct Staging {
@@ -661,6 +663,32 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
     return VR_OK;
 }
 
+// Decodes bricks of a compressed cube (pairs of a work-list index and its slot) on the copy stream,
+// into the slots' atlases (whose arrays and columns are set) or into their linear copies, several
+// bricks a launch.
+static int decode_slots(vr_ctx *c, Cube *cb, const std::vector<std::pair<size_t, int>> &which, const std::vector<DrawBrick> &db,
+                        bool surf) {
+    BrickCache *k = c->cache;
+    WaveletJobs jobs;
+    for (size_t m0 = 0; m0 < which.size(); m0 += kWaveletJobs) {
+        const size_t m1 = std::min(which.size(), m0 + kWaveletJobs);
+        for (size_t m = m0; m < m1; ++m) {
+            Slot &s = k->slots[which[m].second];
+            const DrawBrick &b = db[which[m].first];
+            WaveletJob &jb = jobs.job[m - m0];
+            for (int a = 0; a < 3; ++a) { jb.org[a] = b.org[a]; jb.dim[a] = b.dim[a]; }
+            jb.dst = reinterpret_cast<float *>(k->d_base + (size_t)which[m].second * k->slot_bytes);
+            jb.surf = (unsigned long long)s.surf;
+            jb.x0 = jb.y0 = 0;
+            jb.rows = std::max(s.rows, 1);
+            if (s.used) CK(cudaStreamWaitEvent(k->copy, s.last_use, 0));
+        }
+        CK(launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], jobs, (int)(m1 - m0), surf, k->copy));
+        for (size_t m = m0; m < m1; ++m) (surf ? k->slots[which[m].second].atlas_ok : k->slots[which[m].second].linear_ok) = true;
+    }
+    return VR_OK;
+}
+
 // Makes the bricks of wl.db[d0, d1) resident: hits keep their slot, misses get the least
 // recently used slot not needed by this chunk, are produced on the workers and copied on the
 // cache's stream after the slot's previous reader finished.  Fills data_off / exp2.
@@ -671,7 +699,8 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
     AtlasGeom g;
     int rc = VR_OK;
     if ((cb->layouts & 8) && (rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
-    const bool atlas = (cb->layouts & 8) && g.rows > 0;
+    // whether this frame reads atlases (layout bit 3, a camera near enough) or linear copies
+    const bool atlas = (cb->layouts & 8) && g.rows > 0 && frame_layout(c, cb).atlas;
     std::vector<std::pair<size_t, int>> misses;   // (db index, slot)
     for (size_t i = d0; i < d1; ++i) {
         auto it = k->where.find(key_of(cb->id, db[i].brick));
@@ -682,8 +711,12 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
             db[i].data_off = (long long)((size_t)it->second * k->slot_bytes / esz);
             db[i].exp2 = s.exp2;
             db[i].atlas = 0ull;
+            if (!atlas && !s.linear_ok && (rc = decode_slots(c, cb, {{i, it->second}}, db, false)) != VR_OK) return rc;
             if (atlas) {
-                if (!s.atlas_ok && (rc = slot_atlas_pack(c, cb, it->second, db[i], g)) != VR_OK) return rc;
+                if (!s.atlas_ok) {     // from the linear copy, decoded first where there is none
+                    if (!s.linear_ok && (rc = decode_slots(c, cb, {{i, it->second}}, db, false)) != VR_OK) return rc;
+                    if ((rc = slot_atlas_pack(c, cb, it->second, db[i], g)) != VR_OK) return rc;
+                }
                 set_atlas(db[i], s.tex, s.rows, 0, 0);
             }
             k->hits++;
@@ -709,42 +742,47 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
         Slot &s = k->slots[si];
         if (s.cube >= 0) k->where.erase(key_of(s.cube, s.brick));
         s.cube = -1;                  // not valid until its copy is issued
-        s.atlas_ok = false;
+        s.atlas_ok = s.linear_ok = false;
         s.brick = db[misses[m].first].brick;
         s.chunk = chunk;
         s.lru = ++k->tick;
         misses[m].second = si;
     }
     if (cb->wavelet) {
-        // compressed cube: each missing brick is decoded from the HBM block store straight into
-        // its slot on the cache's stream, after the slot's previous reader
+        // compressed cube: missing bricks are decoded from the HBM block store on the cache's stream,
+        // after their slots' previous readers: into the slots' atlases (surfaces permitting) or
+        // into their linear copies, which atlases are then packed from
+        bool surf = atlas;
+        for (auto &mi : misses)
+            if (atlas) {
+                if ((rc = slot_atlas_alloc(c, cb, mi.second, g)) != VR_OK) break;
+                surf = surf && k->slots[mi.second].surf != 0;
+            }
+        if (rc == VR_OK && surf)
+            for (auto &mi : misses) k->slots[mi.second].rows = g.rows;
+        if (rc == VR_OK) rc = decode_slots(c, cb, misses, db, surf);
         for (auto &mi : misses) {
             Slot &s = k->slots[mi.second];
-            const DrawBrick &b = db[mi.first];
-            if (s.used) CK(cudaStreamWaitEvent(k->copy, s.last_use, 0));
-            CK(launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], b.org, b.dim,
-                                     reinterpret_cast<float *>(k->d_base + (size_t)mi.second * k->slot_bytes),
-                                     k->copy));
+            if (rc == VR_OK && atlas && !surf) rc = slot_atlas_pack(c, cb, mi.second, db[mi.first], g);
+            if (rc != VR_OK) break;
             s.cube = cb->id;
             s.exp2 = 0;
             k->where[key_of(cb->id, s.brick)] = mi.second;
             db[mi.first].data_off = (long long)((size_t)mi.second * k->slot_bytes / esz);
             db[mi.first].exp2 = 0;
             db[mi.first].atlas = 0ull;
+            if (atlas) set_atlas(db[mi.first], s.tex, s.rows, 0, 0);
             k->misses++;
-            k->bytes += b.bytes;
-            if (atlas) {
-                if ((rc = slot_atlas_pack(c, cb, mi.second, b, g)) != VR_OK) {
-                    k->where.erase(key_of(cb->id, s.brick));
-                    s.cube = -1;
-                    s.brick = -1;
-                    s.chunk = -1;
-                    return rc;
-                }
-                set_atlas(db[mi.first], s.tex, s.rows, 0, 0);
-            }
+            k->bytes += db[mi.first].bytes;
         }
-        return VR_OK;
+        if (rc != VR_OK)                // the slots not filled hold nothing
+            for (auto &mi : misses) {
+                Slot &s = k->slots[mi.second];
+                if (s.cube == cb->id) continue;
+                s.brick = -1;
+                s.chunk = -1;
+            }
+        return rc;
     }
     // produce in parallel, at most one staging buffer per brick in flight
     const size_t nstage = k->stage.size();
@@ -801,6 +839,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
             break;
         }
         sg.pending = true;
+        s.linear_ok = true;
         s.cube = cb->id;
         s.exp2 = job.exp2;
         k->where[key_of(cb->id, s.brick)] = si;
@@ -1089,8 +1128,14 @@ int streamed_brick(Cube *cb, int64_t brick, void *data, int *exp2) {
     if (cb->wavelet) {
         float *tmp = nullptr;
         CK(cudaMalloc(&tmp, (size_t)b.bytes));
-        cudaError_t er = launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], b.org,
-                                               b.dim, tmp, 0);
+        WaveletJobs jobs;
+        WaveletJob &jb = jobs.job[0];
+        for (int a = 0; a < 3; ++a) { jb.org[a] = b.org[a]; jb.dim[a] = b.dim[a]; }
+        jb.dst = tmp;
+        jb.surf = 0ull;
+        jb.x0 = jb.y0 = 0;
+        jb.rows = 1;
+        cudaError_t er = launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], jobs, 1, false, 0);
         if (er == cudaSuccess) er = cudaMemcpy(data, tmp, (size_t)b.bytes, cudaMemcpyDeviceToHost);
         cudaFree(tmp);
         if (er != cudaSuccess) return cuda_fail(er, "wavelet brick decode");
