@@ -178,9 +178,13 @@ cudaError_t launch_composite_backward(const FrameConsts &fc, const DrawBrick *db
                                       cudaStream_t s);
 cudaError_t launch_adjoint(const FrameConsts &fc, const float4 *lut, const DrawBrick *db,
                            const TileItem *items, int nitems, const float *pool,
-                           const float4 *frags, const float4 *gfrag, float *glut_partial,
-                           float *gvox, cudaStream_t s);
-// The table gradient from the adjoint's per-CTA partials (nparts x 4 nlut floats), summed in
+                           const float4 *frags, const float4 *gfrag, float *glut_partial, int rows,
+                           float *gvox, float4 *corners, cudaStream_t s);
+// Voxel gradients by way of corner sums (corners instead of gvox above): corner_records records,
+// zeroed before the first view, added to gvox after the last.
+size_t corner_records(int nx, int ny, int nz);
+cudaError_t launch_corner_gather(const float4 *corners, int nx, int ny, int nz, float *gvox, cudaStream_t s);
+// The table gradient from the adjoint's partial rows (nparts x 8 nlut floats), summed in
 // FP64 through `chunks` (kLutGradChunks x 4 nlut doubles of scratch): glut = the sum; with
 // several views, acc (4 nlut doubles) = (first ? 0 : acc) + the view's sum, and
 // glut = (float)acc after the last view.

@@ -38,7 +38,7 @@
 #define VR_RAYMARCH_MIN_BLOCKS 5
 #endif
 #ifndef VR_ADJ_MIN_BLOCKS
-#define VR_ADJ_MIN_BLOCKS 4
+#define VR_ADJ_MIN_BLOCKS 3
 #endif
 constexpr int kSampleUnroll = VR_SAMPLE_UNROLL;
 
@@ -179,11 +179,6 @@ __device__ __forceinline__ int floor_split(float x, float &fl) {
     const float t = __fadd_rd(x, kFloorMagic);
     fl = __fsub_rn(t, kFloorMagic);
     return __float_as_int(t) - kFloorMagicBits;
-}
-
-// An int n with |n| < 2^22 as a float, exactly, without a conversion instruction.
-__device__ __forceinline__ float small_int_float(int n) {
-    return __fsub_rn(__int_as_float(kFloorMagicBits + n), kFloorMagic);
 }
 
 // Brick-local coordinates are below 2^17 in magnitude (stored bricks span at most 65536 + 2
@@ -428,28 +423,6 @@ __device__ __forceinline__ CellF cell_f(float2 xy, float z) {
     return c;
 }
 __device__ __forceinline__ int small_float_int(float f) { return __float_as_int(__fadd_rn(f, kFloorMagic)) - kFloorMagicBits; }
-
-template <int S>
-__device__ __forceinline__ void dvr_sample(const void *src, const Strides &t, int mx, int my, int mz,
-                                           float scale, float x, float y, float z, float vmin,
-                                           float inv_range, float lutmax, int lmax,
-                                           const float4 *s_lut, const unsigned char *chmask,
-                                           int org_z, int nz, float vcode, DvrSample &o,
-                                           const Atlas *atl = nullptr) {
-    Cell c;
-    cell_of(x, y, z, mx, my, mz, c);
-    o.ix = c.ix; o.iy = c.iy; o.iz = c.iz;
-    float v[8];
-    if (atl) {                        // the same texels from the brick's slice atlas
-        float4 g0, g1;
-        gather_slices<S>(*atl, pair2(small_int_float(c.ix), small_int_float(c.iy)), small_int_float(c.iz), g0, g1);
-        gathers_to_stencil(g0, g1, v);
-    } else {
-        fetch8<S>(src, c.ix * t.x + c.iy * t.y + c.iz * t.z, t, v);
-    }
-    if (chmask) mask_channels(v, c.iz, org_z, nz, chmask, vcode);
-    interp_tf(v, c, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, o);
-}
 
 // Stencil cache of one ray: the 8 corner values of the previous sample's cell.  Moving to an
 // adjacent cell (each index changes by at most 1) keeps the corners the two cells share and
@@ -1388,11 +1361,10 @@ __device__ __forceinline__ void shift_face(float acc[8], bool up) {
     for (int c = 0; c < 8; ++c) acc[c] = nacc[c];
 }
 
-// Adds a ray's accumulated voxel gradients of cell (cx, cy, cz) (corner c = x + 2y + 4z) for
-// the corners in `mask` to the cube's gradient (ghost copies map back to their source voxel).
-__device__ __forceinline__ void flush_voxel_grads(float *__restrict__ gvox, const float acc[8], unsigned mask,
-                                                  int cx, int cy, int cz, const DrawBrick &b,
-                                                  const FrameConsts &fc) {
+// Adds a ray's accumulated voxel gradients of cell (cx, cy, cz) (corner c = x + 2y + 4z) to the
+// cube's gradient with one atomic per corner in `mask` (ghost copies map back to their source voxel).
+__device__ __forceinline__ void flush_voxels(float *__restrict__ gvox, const float acc[8], unsigned mask, int cx, int cy, int cz,
+                                             const DrawBrick &b, const FrameConsts &fc) {
     const int x0 = clampi(b.org[0] + cx, 0, fc.nx - 1), x1 = clampi(b.org[0] + cx + 1, 0, fc.nx - 1);
     const int y0 = clampi(b.org[1] + cy, 0, fc.ny - 1), y1 = clampi(b.org[1] + cy + 1, 0, fc.ny - 1);
     const int z0 = clampi(b.org[2] + cz, 0, fc.nz - 1), z1 = clampi(b.org[2] + cz + 1, 0, fc.nz - 1);
@@ -1407,6 +1379,17 @@ __device__ __forceinline__ void flush_voxel_grads(float *__restrict__ gvox, cons
             atomicAdd(p + ((c & 1) ? dx : 0) + ((c & 2) ? dy : 0) + ((c & 4) ? dz : 0), acc[c]);
 }
 
+// The same into corner sums (k_corner_gather): the record of xy cell (x, y) in plane z holds the
+// sums of its four corners, so a cell's eight corners are two vector atomics.  Cells run from -1 (the
+// ghost copy below the cube) to n - 1, planes from -1 to n.
+__device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, const float acc[8], int cx, int cy, int cz,
+                                              const DrawBrick &b, const FrameConsts &fc) {
+    const int row = fc.nx + 1, plane = row * (fc.ny + 1);
+    float4 *p = corners + ((long long)(b.org[2] + cz + 1) * plane + (b.org[1] + cy + 1) * row + (b.org[0] + cx + 1));
+    atomicAdd(p, make_float4(acc[0], acc[1], acc[2], acc[3]));
+    atomicAdd(p + plane, make_float4(acc[4], acc[5], acc[6], acc[7]));
+}
+
 // Adjoint ray cast (FP32 bricks).  Each (brick, pixel) segment is replayed front to back with
 // the forward's arithmetic; from the stored segment colour C_b and transmittance T_b the
 // gradient of every sample follows without per-sample storage:
@@ -1416,132 +1399,238 @@ __device__ __forceinline__ void flush_voxel_grads(float *__restrict__ gvox, cons
 // Table gradients accumulate per CTA in a partial row in L2 (two float4 atomics per sample; eight
 // float atomics per sample into shared-memory copies were 13 % slower per batch, their retries of
 // contended adds and the copy-out included).
-// Voxel gradients accumulate per ray for the 8 corners of its current cell and are added to the
-// cube's voxels when the ray leaves the cell (ghost copies map back to their source voxel); a
-// step into an adjacent cell keeps the shared face's 4 sums (before: 8 atomics per sample).
-// Bounded to 4 CTAs per SM (64 registers, a few spilled; 80 unbounded give 3 CTAs, 8 % slower).
+// Voxel gradients accumulate per ray for the 8 corners of its current cell and are added when the
+// ray leaves the cell.  VOX 0: none; 1: one float atomic per corner into the cube's gradient, a step
+// into an adjacent cell keeping the shared face's 4 sums; 2: two float4 atomics into corner
+// sums that k_corner_gather adds up afterwards.
+// Bound by L2's atomics (about 200 G 16-byte adds a second: without the table's adds, a timing copy,
+// 9.8 instead of 12.7 ms a batch of 8 views; with half of them 10.7) above the replay's gathers.  With
+// one atomic per corner it was bound by instruction issue: three variants of the flush, each run
+// by the few lanes that needed it, 17.8 of 32 lanes active and 1.25 G warp instructions a view
+// against 26.4 and 0.54 G.
+// Small launches are bound by the chain of samples: the next sample's gathers are issued ahead (80
+// registers, 3 CTAs an SM; one 256^2 view of 64^3 with the table's gradient alone 128 -> 114 us).
+// 256^3 cube, 8 views at 512^2, step 0.5, forward frames cast again: 18.5 -> 12.5 ms with both
+// gradients, 9.9 -> 9.4 ms with the table's alone.
 // ATLAS: the replay reads the stencils from the bricks' slice atlases (the forward's texels)
-// instead of the linear copy.
-template <bool ATLAS>
+// instead of the linear copy; then no index is clamped (make_consts).
+template <bool ATLAS, int VOX>
 __global__ void __launch_bounds__(256, VR_ADJ_MIN_BLOCKS)
 k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const float *__restrict__ pool,
           const float4 *__restrict__ frags, const float4 *__restrict__ gfrag,
-          float *__restrict__ glut_partial, float *__restrict__ gvox) {
+          float *__restrict__ glut_partial, int rows, void *__restrict__ gvox) {
     extern __shared__ float4 s_lut[];
     load_table(lut, fc.nlut, s_lut);
     __syncthreads();
     const TileItem it = items[blockIdx.x];
     const DrawBrick &b = dbs[it.db];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // this CTA's table-gradient partial: one float4 (the 4 channels) per entry, zeroed before the
-    // launch; each sample adds its two entries' channels with one vector atomic each (in L2)
-    float4 *g_row = reinterpret_cast<float4 *>(glut_partial) + (long long)blockIdx.x * fc.nlut;
+    const bool odd = lane & 1;
+    // this CTA's table-gradient partial (rows are zeroed before the launch)
+    float4 *g_row = reinterpret_cast<float4 *>(glut_partial) + (long long)(blockIdx.x % rows) * 2 * fc.nlut + (odd ? 1 : 0);
     // a warp's 32 rays are adjacent pixels along the image axis the brick layout follows
     int rx, ry;
     thread_pixel(fc.lanes_y, it, warp, lane, rx, ry);
-    if (rx < b.rect[2] && ry < b.rect[3]) {
+    float4 gf = make_float4(0.0f, 0.0f, 0.0f, 0.0f), fr = gf;
+    float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 0.0f};
+    int k0 = 0, k1 = 0;
+    bool live = rx < b.rect[2] && ry < b.rect[3];
+    if (live) {
         const long long fi = b.frag_off + (long long)ry * b.rect[2] + rx;
-        const float4 gf = gfrag[fi];
-        float o[3], d[3];
+        gf = gfrag[fi];
+        fr = frags[fi];
         ray_for_pixel(fc.cam, b.rect[0] + rx, b.rect[1] + ry, o, d);
-        int k0 = 0, k1 = 0;
-        if ((gf.x != 0.0f || gf.y != 0.0f || gf.z != 0.0f || gf.w != 0.0f) &&
-            box_krange(o, d, b.lo, b.hi, fc.step, k0, k1)) {
-            const float4 fr = frags[fi];
-            const float *src = pool + b.data_off;
-            const Strides st{b.str[0], b.str[1], b.str[2]};
-            const int mx = b.dim[0] - 2, my = b.dim[1] - 2, mz = b.dim[2] - 2;
-            const float qx = anchor(o[0], d[0], b.org_c[0], k0, fc.step);
-            const float qy = anchor(o[1], d[1], b.org_c[1], k0, fc.step);
-            const float qz = anchor(o[2], d[2], b.org_c[2], k0, fc.step);
-            const int n = k1 - k0;
-            const float dxdv = __fmul_rn(fc.lutmax, fc.inv_range);
-            float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, T = 1.0f;
-            // voxel gradients of the ray's current cell, added to the cube when the ray leaves it
-            float acc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            int ccx = -4, ccy = -4, ccz = -4;
-            const Atlas atl = ATLAS ? atlas_of(b) : Atlas{};
-            for (int j = 0; j < n; ++j) {
-                const float tj = __fmul_rn((float)j, fc.step);
-                DvrSample sm;
-                dvr_sample<0>(src, st, mx, my, mz, 1.0f, __fmaf_rn(tj, d[0], qx),
-                              __fmaf_rn(tj, d[1], qy), __fmaf_rn(tj, d[2], qz), fc.vmin,
-                              fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, fc.chmask, b.org[2],
-                              fc.nz, fc.vmin, sm, ATLAS ? &atl : nullptr);
-                const float Tb = T;
-                over(sm, c0, c1, c2, T);
-                const bool last = (T <= fc.thr) || (j == n - 1);
-                const float gcdot = gf.x * sm.r + gf.y * sm.g + gf.z * sm.b;
-                float ga;
-                if (last) {
-                    ga = Tb * (gcdot - gf.w);
-                } else {
-                    const float sdot = gf.x * (fr.x - c0) + gf.y * (fr.y - c1) + gf.z * (fr.z - c2);
-                    ga = Tb * (gcdot - (sdot + gf.w * fr.w) / T);
-                }
-                const float wa = Tb * sm.a;
-                const float gr = gf.x * wa, gg = gf.y * wa, gb = gf.z * wa;
-                const float w1 = sm.lf, w0 = 1.0f - sm.lf;
-                atomicAdd(g_row + sm.li, make_float4(w0 * gr, w0 * gg, w0 * gb, w0 * ga));
-                if (sm.li + 1 < fc.nlut)      // the last entry (u >= 1) has weight 1 and no next entry
-                    atomicAdd(g_row + sm.li + 1, make_float4(w1 * gr, w1 * gg, w1 * gb, w1 * ga));
-                if (gvox != nullptr && sm.u > 0.0f && sm.u < 1.0f) {
-                    const float gx = gr * sm.D.x + gg * sm.D.y + gb * sm.D.z + ga * sm.D.w;
-                    const float gv = gx * dxdv;
-                    if (gv != 0.0f) {
-                        const int ix = sm.ix, iy = sm.iy, iz = sm.iz;
-                        if (ix != ccx || iy != ccy || iz != ccz) {
-                            const int ddx = ix - ccx, ddy = iy - ccy, ddz = iz - ccz;
-                            const int ax = (ddx != 0) + (ddy != 0) + (ddz != 0);
-                            if (ax == 1 && ddx >= -1 && ddx <= 1 && ddy >= -1 && ddy <= 1 &&
-                                ddz >= -1 && ddz <= 1) {
-                                // one step along one axis: the face both cells share keeps accumulating
-                                const int sh = ddx != 0 ? 0 : (ddy != 0 ? 1 : 2);
-                                const int up = (ddx + ddy + ddz) > 0;
-                                const unsigned lowf = sh == 0 ? 0x55u : (sh == 1 ? 0x33u : 0x0Fu);
-                                flush_voxel_grads(gvox, acc, up ? lowf : (~lowf & 0xffu), ccx, ccy, ccz, b, fc);
-                                if (sh == 0) shift_face<0>(acc, up);
-                                else if (sh == 1) shift_face<1>(acc, up);
-                                else shift_face<2>(acc, up);
-                            } else {
-                                flush_voxel_grads(gvox, acc, 0xffu, ccx, ccy, ccz, b, fc);
-#pragma unroll
-                                for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-                            }
-                            ccx = ix; ccy = iy; ccz = iz;
-                        }
-                        const int gz0 = clampi(b.org[2] + iz, 0, fc.nz - 1), gz1 = clampi(b.org[2] + iz + 1, 0, fc.nz - 1);
-                        const float ux = sm.fx, uy = sm.fy;
-                        const float vx = 1.0f - ux, vy = 1.0f - uy;
-                        const float uz = (fc.chmask && !fc.chmask[gz1]) ? 0.0f : sm.fz;
-                        const float vz = (fc.chmask && !fc.chmask[gz0]) ? 0.0f : 1.0f - sm.fz;
-                        // trilinear weights of the 8 corners, factored by z, then y
-                        const float wz0 = gv * vz, wz1 = gv * uz;
-                        const float g00 = wz0 * vy, g10 = wz0 * uy, g01 = wz1 * vy, g11 = wz1 * uy;
-                        acc[0] = __fmaf_rn(g00, vx, acc[0]); acc[1] = __fmaf_rn(g00, ux, acc[1]);
-                        acc[2] = __fmaf_rn(g10, vx, acc[2]); acc[3] = __fmaf_rn(g10, ux, acc[3]);
-                        acc[4] = __fmaf_rn(g01, vx, acc[4]); acc[5] = __fmaf_rn(g01, ux, acc[5]);
-                        acc[6] = __fmaf_rn(g11, vx, acc[6]); acc[7] = __fmaf_rn(g11, ux, acc[7]);
-                    }
-                }
-                if (T <= fc.thr) break;
+        live = (gf.x != 0.0f || gf.y != 0.0f || gf.z != 0.0f || gf.w != 0.0f) && box_krange(o, d, b.lo, b.hi, fc.step, k0, k1);
+    }
+    const float *src = pool + b.data_off;
+    const Strides st{b.str[0], b.str[1], b.str[2]};
+    const int mx = b.dim[0] - 2, my = b.dim[1] - 2, mz = b.dim[2] - 2;
+    const float qx = anchor(o[0], d[0], b.org_c[0], k0, fc.step);
+    const float qy = anchor(o[1], d[1], b.org_c[1], k0, fc.step);
+    const float qz = anchor(o[2], d[2], b.org_c[2], k0, fc.step);
+    const float nf = (float)(k1 - k0);         // exact: at most 2^24 + 1
+    const float dxdv = __fmul_rn(fc.lutmax, fc.inv_range);
+    const float grest = gf.w * fr.w;
+    float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, T = 1.0f;
+    // voxel gradients of the ray's current cell, added to the cube when the ray leaves it
+    float acc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    CellF cc;
+    cc.ixy = pair2(-4.0f, -4.0f);
+    cc.iz = -4.0f;
+    const Atlas atl = ATLAS ? atlas_of(b) : Atlas{};
+    float jf = 0.0f;
+    // sample j's cell; atlas bricks: its gathers are issued one sample ahead (the last one's again
+    // at the end), so that their latency passes under a sample's arithmetic and atomics
+    auto cell_at = [&](float j) {
+        const float tj = __fmul_rn(j, fc.step);
+        return cell_f(__ffma2_rn(pair2(tj, tj), pair2(d[0], d[1]), pair2(qx, qy)), __fmaf_rn(tj, d[2], qz));
+    };
+    CellF cn = cell_at(0.0f);
+    float4 n0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), n1 = n0;
+    if (ATLAS && live) gather_slices<0>(atl, cn.ixy, cn.iz, n0, n1);
+    while (__any_sync(0xffffffffu, live)) {
+        int li = -1;
+        float4 lo = make_float4(0.0f, 0.0f, 0.0f, 0.0f), hi = lo;    // the sample's adds to entries li and li + 1
+        if (live) {
+            CellF cl = cn;
+            const float4 g0 = n0, g1 = n1;
+            jf = __fadd_rn(jf, 1.0f);
+            cn = cell_at(fminf(jf, nf - 1.0f));
+            if (ATLAS) {
+                gather_slices<0>(atl, cn.ixy, cn.iz, n0, n1);
+            } else {                               // indices clamped to the stored brick
+                cl.ixy = pair2(fminf(fmaxf(cl.ixy.x, 0.0f), (float)mx), fminf(fmaxf(cl.ixy.y, 0.0f), (float)my));
+                cl.iz = fminf(fmaxf(cl.iz, 0.0f), (float)mz);
             }
-            if (gvox != nullptr && ccx != -4) flush_voxel_grads(gvox, acc, 0xffu, ccx, ccy, ccz, b, fc);
+            const Cell ci{0, 0, 0, cl.fxy.x, cl.fxy.y, cl.fz};
+            DvrSample sm;
+            if (ATLAS && !fc.chmask) {
+                interp_tf(lerp_z(g0, g1, cl.fz), ci, false, 1.0f, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+            } else {
+                float v[8];
+                const int iz = small_float_int(cl.iz);
+                if (ATLAS) {
+                    gathers_to_stencil(g0, g1, v);
+                } else {
+                    fetch8<0>(src, small_float_int(cl.ixy.x) * st.x + small_float_int(cl.ixy.y) * st.y + iz * st.z, st, v);
+                }
+                if (fc.chmask) mask_channels(v, iz, b.org[2], fc.nz, fc.chmask, fc.vmin);
+                interp_tf(v, ci, false, 1.0f, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+            }
+            const float Tb = T;
+            over(sm, c0, c1, c2, T);
+            const bool last = (T <= fc.thr) || !(jf < nf);
+            const float gcdot = gf.x * sm.r + gf.y * sm.g + gf.z * sm.b;
+            float ga;
+            if (last) {
+                ga = Tb * (gcdot - gf.w);
+            } else {
+                const float sdot = gf.x * (fr.x - c0) + gf.y * (fr.y - c1) + gf.z * (fr.z - c2);
+                ga = Tb * (gcdot - (sdot + grest) / T);
+            }
+            const float wa = Tb * sm.a;
+            const float gr = gf.x * wa, gg = gf.y * wa, gb = gf.z * wa;
+            const float w1 = sm.lf, w0 = 1.0f - sm.lf;
+            li = sm.li;
+            lo = make_float4(w0 * gr, w0 * gg, w0 * gb, w0 * ga);
+            hi = make_float4(w1 * gr, w1 * gg, w1 * gb, w1 * ga);
+            if (VOX && sm.u > 0.0f && sm.u < 1.0f) {
+                const float gx = gr * sm.D.x + gg * sm.D.y + gb * sm.D.z + ga * sm.D.w;
+                const float gv = gx * dxdv;
+                if (cl.ixy.x != cc.ixy.x || cl.ixy.y != cc.ixy.y || cl.iz != cc.iz) {
+                    bool fresh = true;
+                    if (cc.iz >= 0.0f) {
+                        const int cx = small_float_int(cc.ixy.x), cy = small_float_int(cc.ixy.y), cz = small_float_int(cc.iz);
+                        if (VOX == 2) {
+                            flush_corners(static_cast<float4 *>(gvox), acc, cx, cy, cz, b, fc);
+                        } else {
+                            const float sx = cl.ixy.x - cc.ixy.x, sy = cl.ixy.y - cc.ixy.y, sz = cl.iz - cc.iz;
+                            if (fabsf(sx) + fabsf(sy) + fabsf(sz) == 1.0f) {
+                                // one step along one axis: the face both cells share keeps accumulating
+                                const bool up = sx + sy + sz > 0.0f;
+                                const unsigned lowf = sx != 0.0f ? 0x55u : (sy != 0.0f ? 0x33u : 0x0Fu);
+                                flush_voxels(static_cast<float *>(gvox), acc, up ? lowf : (~lowf & 0xffu), cx, cy, cz, b, fc);
+                                if (sx != 0.0f) shift_face<0>(acc, up);
+                                else if (sy != 0.0f) shift_face<1>(acc, up);
+                                else shift_face<2>(acc, up);
+                                fresh = false;
+                            } else {
+                                flush_voxels(static_cast<float *>(gvox), acc, 0xffu, cx, cy, cz, b, fc);
+                            }
+                        }
+                    }
+                    if (fresh)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
+                    cc.ixy = cl.ixy;
+                    cc.iz = cl.iz;
+                }
+                const float ux = sm.fx, uy = sm.fy;
+                const float vx = 1.0f - ux, vy = 1.0f - uy;
+                float uz = sm.fz, vz = 1.0f - sm.fz;
+                if (fc.chmask) {
+                    const int gz = b.org[2] + small_float_int(cl.iz);
+                    if (!fc.chmask[clampi(gz + 1, 0, fc.nz - 1)]) uz = 0.0f;
+                    if (!fc.chmask[clampi(gz, 0, fc.nz - 1)]) vz = 0.0f;
+                }
+                // trilinear weights of the 8 corners, factored by z, then y
+                const float wz0 = gv * vz, wz1 = gv * uz;
+                const float g00 = wz0 * vy, g10 = wz0 * uy, g01 = wz1 * vy, g11 = wz1 * uy;
+                acc[0] = __fmaf_rn(g00, vx, acc[0]); acc[1] = __fmaf_rn(g00, ux, acc[1]);
+                acc[2] = __fmaf_rn(g10, vx, acc[2]); acc[3] = __fmaf_rn(g10, ux, acc[3]);
+                acc[4] = __fmaf_rn(g01, vx, acc[4]); acc[5] = __fmaf_rn(g01, ux, acc[5]);
+                acc[6] = __fmaf_rn(g11, vx, acc[6]); acc[7] = __fmaf_rn(g11, ux, acc[7]);
+            }
+            live = !last;
         }
+        // Table gradient: the record of an interval is 32 bytes, its adds to the lower entry and to the
+        // upper one.  Two lanes add one sample's record together (even lanes the lower halves, odd
+        // lanes the upper ones), so that a sample is one 32-byte request to L2 instead of two of 16.
+        const float4 keep = odd ? hi : lo, send = odd ? lo : hi;
+        const int lp = __shfl_xor_sync(0xffffffffu, li, 1);
+        const float4 recv = make_float4(__shfl_xor_sync(0xffffffffu, send.x, 1), __shfl_xor_sync(0xffffffffu, send.y, 1),
+                                        __shfl_xor_sync(0xffffffffu, send.z, 1), __shfl_xor_sync(0xffffffffu, send.w, 1));
+        const int l1 = odd ? lp : li, l2 = odd ? li : lp;
+        if (l1 >= 0) atomicAdd(g_row + 2 * l1, odd ? recv : keep);
+        if (l2 >= 0) atomicAdd(g_row + 2 * l2, odd ? keep : recv);
+    }
+    if (VOX && cc.iz >= 0.0f) {
+        const int cx = small_float_int(cc.ixy.x), cy = small_float_int(cc.ixy.y), cz = small_float_int(cc.iz);
+        if (VOX == 2) flush_corners(static_cast<float4 *>(gvox), acc, cx, cy, cz, b, fc);
+        else flush_voxels(static_cast<float *>(gvox), acc, 0xffu, cx, cy, cz, b, fc);
+    }
+}
+
+// Corner sums -> voxel gradients: voxel (x, y, z) is the low corner of cell x, the high corner of cell
+// x - 1 and, at the cube's border, the corner that the ghost copy beyond it stands for; likewise
+// along y and z.  Bound by HBM: 16 B of sums read per voxel, the gradient read and written.
+__global__ void __launch_bounds__(256)
+k_corner_gather(const float4 *__restrict__ corners, int nx, int ny, int nz, float *__restrict__ gvox) {
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (x >= nx || y >= ny) return;
+    const int row = nx + 1;
+    const long long plane = (long long)row * (ny + 1);
+    // the xy sums of a plane of corners at (x, y)
+    auto xy_sum = [&](int p) {
+        const float4 *q = corners + p * plane + (long long)y * row + x;    // record (x, y) is cell (x - 1, y - 1)
+        float s = q[row + 1].x + q[row].y + q[1].z + q[0].w;
+        // beyond the border: the ghost cell's far corner is this voxel too
+        if (x == 0) s += q[row].x + q[0].z;
+        if (x == nx - 1) s += q[row + 1].y + q[1].w;
+        if (y == 0) s += q[1].x + q[0].y;
+        if (y == ny - 1) s += q[row + 1].z + q[row].w;
+        if (x == 0 && y == 0) s += q[0].x;
+        if (x == nx - 1 && y == 0) s += q[1].y;
+        if (x == 0 && y == ny - 1) s += q[row].z;
+        if (x == nx - 1 && y == ny - 1) s += q[row + 1].w;
+        return s;
+    };
+    for (int z = blockIdx.z; z < nz; z += gridDim.z) {
+        float s = xy_sum(z + 1);
+        if (z == 0) s += xy_sum(0);
+        if (z == nz - 1) s += xy_sum(nz + 1);
+        if (s != 0.0f) gvox[((long long)z * ny + y) * nx + x] += s;
     }
 }
 
 // Final reduction of the per-CTA table-gradient partials, in FP64 and in two stages so that
 // every entry's sum is spread over many threads yet formed in a fixed order: chunk y sums the
 // partials of parts [y q, (y + 1) q) in part order, then the chunk sums are added in chunk order.
+// A partial holds, per interval, 4 channels for its lower entry and 4 for its upper one: an
+// entry is the sum of its own lower record and the upper one of the interval before it.
 __global__ void k_lut_grad_chunks(const float *__restrict__ partial, int nparts, int n, double *__restrict__ chunks) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int q = (nparts + (int)gridDim.y - 1) / (int)gridDim.y;
     const int p0 = (int)blockIdx.y * q, p1 = min(nparts, p0 + q);
+    const int lo = (i >> 2) * 8 + (i & 3);
     double a = 0.0;
-    for (int p = p0; p < p1; ++p) a += (double)partial[(long long)p * n + i];
+    for (int p = p0; p < p1; ++p) {
+        const float *r = partial + (long long)p * 2 * n;
+        a += (double)r[lo];
+        if (i >= 4) a += (double)r[lo - 4];
+    }
     chunks[(long long)blockIdx.y * n + i] = a;
 }
 
@@ -1751,23 +1840,36 @@ cudaError_t launch_composite_backward(const FrameConsts &fc, const DrawBrick *db
     return cudaGetLastError();
 }
 
+template <bool ATLAS, int VOX>
+static cudaError_t adjoint(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items, int nitems,
+                           const float *pool, const float4 *frags, const float4 *gfrag, float *glut_partial, int rows, void *gvox,
+                           cudaStream_t s) {
+    static DeviceAttrs da;
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<ATLAS, VOX>), (int)(32 * kMaxLut), da);
+    if (e != cudaSuccess) return e;
+    k_adjoint<ATLAS, VOX><<<nitems, 256, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_adjoint(const FrameConsts &fc, const float4 *lut, const DrawBrick *db,
                            const TileItem *items, int nitems, const float *pool,
-                           const float4 *frags, const float4 *gfrag, float *glut_partial,
-                           float *gvox, cudaStream_t s) {
+                           const float4 *frags, const float4 *gfrag, float *glut_partial, int rows,
+                           float *gvox, float4 *corners, cudaStream_t s) {
     if (nitems <= 0) return cudaSuccess;
-    static DeviceAttrs da_lin, da_atl;
-    cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<false>), (int)(32 * kMaxLut), da_lin);
-    if (e == cudaSuccess)
-        e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<true>), (int)(32 * kMaxLut), da_atl);
+    const cudaError_t e = cudaMemsetAsync(glut_partial, 0, sizeof(float) * 8 * (size_t)fc.nlut * rows, s);
     if (e != cudaSuccess) return e;
-    const size_t smem = 32 * (size_t)fc.nlut;      // table + differences
-    e = cudaMemsetAsync(glut_partial, 0, sizeof(float) * 4 * (size_t)fc.nlut * nitems, s);
-    if (e != cudaSuccess) return e;
-    if (fc.fetch == 2)
-        k_adjoint<true><<<nitems, 256, smem, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, gvox);
-    else
-        k_adjoint<false><<<nitems, 256, smem, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, gvox);
+#define VR_ADJ(A, V, G) adjoint<A, V>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s)
+    if (fc.fetch == 2) return corners ? VR_ADJ(true, 2, corners) : gvox ? VR_ADJ(true, 1, gvox) : VR_ADJ(true, 0, nullptr);
+    return corners ? VR_ADJ(false, 2, corners) : gvox ? VR_ADJ(false, 1, gvox) : VR_ADJ(false, 0, nullptr);
+#undef VR_ADJ
+}
+
+size_t corner_records(int nx, int ny, int nz) { return (size_t)(nz + 2) * (ny + 1) * (nx + 1); }
+
+cudaError_t launch_corner_gather(const float4 *corners, int nx, int ny, int nz, float *gvox, cudaStream_t s) {
+    const int gx = (nx + 31) / 32, gy = (ny + 7) / 8;
+    const int gz = std::max(1, std::min(nz, 152 * 16 / std::max(1, gx * gy)));
+    k_corner_gather<<<dim3(gx, gy, gz), 256, 0, s>>>(corners, nx, ny, nz, gvox);
     return cudaGetLastError();
 }
 
