@@ -500,7 +500,13 @@ FrameConsts make_consts(vr_ctx *c, Cube *cb) {
     // atlases: two gathers per sample.  Linear copies: with a warp's rays along the contiguous
     // axis its loads are nearly coalesced and the stencil cache's bookkeeping costs more than
     // it saves; with a poor alignment it pays
-    fc.fetch = fl.atlas ? (cb->atlas_pair && !cb->streamed ? 5 : 2) : (fl.align < 0.9f ? 1 : 0);
+    // (MIP frames: no stencil cache).  Cameras beyond kAtlasReach: clamped indices.
+    if (fl.atlas) fc.fetch = cb->atlas_pair && !cb->streamed ? 5 : 2;
+    else if (c->cam_set && ray_reach(c, cb) > kAtlasReach) fc.fetch = 0;
+    else fc.fetch = fl.align < 0.9f && c->mode == VR_DVR ? 1 : 6 + fl.layout;
+    const int64_t planes = std::min<int64_t>(cb->B[2], cb->n[2]) + 1;      // stored z of the tallest brick, minus one
+    fc.mask_planes = !c->chmask.empty() && planes <= kMaskPlanes ? (int)planes : 0;
+
     fc.sub = c->subimage ? 1 : 0;
     // staged slabs: DVR frames of resident FP32 cubes that keep the padded copy of the frame
     // layout; the march axis is the view's dominant axis other than the contiguous one

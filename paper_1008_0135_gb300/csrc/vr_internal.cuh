@@ -12,6 +12,7 @@ namespace vr {
 constexpr int kTile = 16;          // compositing: 16x16 screen tiles
 constexpr int kRcLong = 32;        // ray-cast work item: 32x8 (or 8x32) pixels of a rectangle,
 constexpr int kRcShort = 8;        // one warp per 32-pixel row (or column)
+constexpr int kMaskPlanes = 4096;  // stencil planes of a brick whose channel bits shared memory holds
 constexpr int kMaxLut = 4096;      // transfer-function entries (float4 each) held in shared memory
 
 // Camera constants in the FP32 decision arithmetic (computed once per frame on the host).
@@ -36,12 +37,16 @@ struct FrameConsts {
     int lanes_y;                   // 0: a warp's 32 lanes run along image x (tiles 32x8);
                                    // 1: along image y (tiles 8x32)
     int fetch;                     // how a sample's 8 stencil corners are read: 0 = 8 loads from
-                                   // the linear brick, 1 = the same with the stencil cache (rays
-                                   // keep shared corners; poorly aligned layout), 2 = 2 gathers
-                                   // from the brick's slice-atlas texture, 4 = slabs of the
-                                   // brick staged in shared memory by bulk copies from the copy
-                                   // with 16-byte rows (DVR, FP32 bricks), 5 = 1 gather from
-                                   // the brick's pair atlas (16-bit bricks)
+                                   // the linear brick at clamped indices (cameras far away), 1 =
+                                   // loads of the corners a ray's last cell did not hold (poorly
+                                   // aligned layout), 2 = 2 gathers from the brick's slice-atlas
+                                   // texture, 4 = slabs of the brick staged in shared memory by
+                                   // bulk copies from the copy with 16-byte rows (DVR, FP32
+                                   // bricks), 5 = 1 gather from the brick's pair atlas (16-bit
+                                   // bricks), 6 / 7 / 8 = 4 pairs of loads from a linear brick
+                                   // whose x / y / z is contiguous
+    int mask_planes;               // with chmask: the most stencil planes (stored z - 1) a brick has,
+                                   // 0 when they do not fit shared memory
     const unsigned char *chmask;   // per spectral channel (cube z): 0 = disabled; null = none
     int sub;                       // 1: a part's sub-image -- DVR pixels keep the transmittance T
                                    // (not 1 - T), MIP pixels without samples stay -inf

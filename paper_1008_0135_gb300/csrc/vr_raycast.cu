@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "vr_internal.cuh"
 
@@ -27,6 +28,9 @@
 #endif
 #ifndef VR_DVR_MIN_BLOCKS
 #define VR_DVR_MIN_BLOCKS 6
+#endif
+#ifndef VR_ROWS_MIN_BLOCKS
+#define VR_ROWS_MIN_BLOCKS 4
 #endif
 #ifndef VR_MIP_MIN_BLOCKS
 #define VR_MIP_MIN_BLOCKS 0
@@ -384,6 +388,10 @@ __device__ __forceinline__ void gather_stencil(const Atlas &a, float2 ixy, float
     else gather_slices<S>(a, ixy, iz, g0, g1);
 }
 
+// Whether fetch mode F reads rows of a linear copy without clamps, and the copy's contiguous axis.
+constexpr bool straight(int F) { return F >= 6; }
+constexpr int row_axis(int F) { return F - 6; }
+
 // Whether fetch mode F reads a texture (the slice atlas, 2, or the pair atlas, 5).
 constexpr bool gathers(int F) { return F == 2 || F == 5; }
 
@@ -395,6 +403,21 @@ __device__ __forceinline__ void fetch8(const void *src, int i0, const Strides &t
     v[6] = ldv<S>(src, i0 + t.z + t.y); v[7] = ldv<S>(src, i0 + t.z + t.y + t.x);
 }
 
+// The stencil at element p of a linear copy whose axis AX is contiguous: four rows, two neighbours each
+// (the second at a constant offset: 4 addresses instead of 8).
+template <int S, int AX>
+__device__ __forceinline__ void fetch8_rows(const void *src, int i0, const Strides &t, float v[8]) {
+    using T = std::conditional_t<S == 0, float, unsigned short>;
+    const T *p = static_cast<const T *>(src) + i0;
+    const int s1 = AX == 0 ? t.y : t.x, s2 = AX == 2 ? t.y : t.z;
+    constexpr int a = 1 << AX, b1 = AX == 0 ? 2 : 1, b2 = AX == 2 ? 2 : 4;
+    const T *q = p + s1, *r = p + s2, *w = r + s1;
+    v[0] = ldv<S>(p, 0);       v[a] = ldv<S>(p, 1);
+    v[b1] = ldv<S>(q, 0);      v[b1 | a] = ldv<S>(q, 1);
+    v[b2] = ldv<S>(r, 0);      v[b2 | a] = ldv<S>(r, 1);
+    v[b2 | b1] = ldv<S>(w, 0); v[b2 | b1 | a] = ldv<S>(w, 1);
+}
+
 // Disabled spectral channels hold vmin (the bottom of the table range) in place of their data:
 // the stencil's two z-planes are global channels org_z + iz and + 1 (clamped at the cube
 // border, like the ghost copies).  `vcode` is vmin in the brick's stored units.
@@ -403,6 +426,17 @@ __device__ __forceinline__ void mask_channels(float v[8], int iz, int org_z, int
     const int z0 = clampi(org_z + iz, 0, nz - 1), z1 = clampi(org_z + iz + 1, 0, nz - 1);
     if (!chmask[z0]) { v[0] = vcode; v[1] = vcode; v[2] = vcode; v[3] = vcode; }
     if (!chmask[z1]) { v[4] = vcode; v[5] = vcode; v[6] = vcode; v[7] = vcode; }
+}
+
+// The same from a brick's plane bits in shared memory: bit 0 of byte iz is the channel of stored plane
+// iz, bit 1 that of iz + 1 (one load a sample instead of two from global memory and their clamps).
+__device__ __forceinline__ void load_mask_planes(const DrawBrick &b, int nz, const unsigned char *chmask, unsigned char *s) {
+    for (int i = threadIdx.x; i < b.dim[2] - 1; i += blockDim.x)
+        s[i] = (chmask[clampi(b.org[2] + i, 0, nz - 1)] ? 1 : 0) | (chmask[clampi(b.org[2] + i + 1, 0, nz - 1)] ? 2 : 0);
+}
+__device__ __forceinline__ void mask_planes(float v[8], unsigned m, float vcode) {
+    if (!(m & 1)) { v[0] = vcode; v[1] = vcode; v[2] = vcode; v[3] = vcode; }
+    if (!(m & 2)) { v[4] = vcode; v[5] = vcode; v[6] = vcode; v[7] = vcode; }
 }
 
 // A point's cell in whole-number floats: lower corner (x, y packed) and fractions, no clamps --
@@ -502,13 +536,15 @@ __device__ __forceinline__ void over(const DvrSample &s, float &c0, float &c1, f
 // within 1 % (8 CTAs at 32 registers without software pipelining against 6 with it).
 template <int S, int F, bool MASK>
 __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const CellF &c, float scale, const FrameConsts &fc,
-                                      const float4 *s_lut, int org_z, float vcode, float &c0, float &c1, float &c2, float &T) {
+                                      const float4 *s_lut, const unsigned char *s_mask, int org_z, float vcode, float &c0,
+                                      float &c1, float &c2, float &T) {
     const Cell cl{0, 0, 0, c.fxy.x, c.fxy.y, c.fz};
     DvrSample sm;
     if (MASK) {
         float v[8];
         gathers_to_stencil(g0, g1, v);
-        mask_channels(v, small_float_int(c.iz), org_z, fc.nz, fc.chmask, vcode);
+        if (s_mask) mask_planes(v, s_mask[small_float_int(c.iz)], vcode);
+        else mask_channels(v, small_float_int(c.iz), org_z, fc.nz, fc.chmask, vcode);
         interp_tf<!entries_only(F)>(lerp_z(v, cl.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
     } else {
         interp_tf<!entries_only(F)>(lerp_z(g0, g1, c.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
@@ -519,7 +555,7 @@ __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const 
 template <int S, int F, bool MASK>
 __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, float qx, float qy, float qz,
                                                  const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
-                                                 int org_z, float vcode, float &c0, float &c1, float &c2, float &T) {
+                                                 const unsigned char *s_mask, int org_z, float vcode, float &c0, float &c1, float &c2, float &T) {
     const float nf = (float)n;            // exact: n <= 2^24 + 1, checked by the host
     const float2 q = pair2(qx, qy), dd = pair2(d[0], d[1]);
     float jf = 0.0f;
@@ -529,7 +565,48 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
         const CellF cl = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
         float4 g0, g1;
         gather_stencil<S, F>(atl, cl.ixy, cl.iz, g0, g1);
-        shade<S, F, MASK>(g0, g1, cl, scale, fc, s_lut, org_z, vcode, c0, c1, c2, T);
+        shade<S, F, MASK>(g0, g1, cl, scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+        jf = __fadd_rn(jf, 1.0f);
+    } while (!(T <= fc.thr) && jf < nf);
+    return (int)jf;
+}
+
+// The segment loop over rows of a linear copy, for cameras near enough that no index needs a clamp.
+// Bound by the loads' latency and their L1 wavefronts.  Few instructions, as in the atlas loop; cell
+// indices come straight from the bits of the rounded-down positions, and the rows' second
+// neighbours are constant offsets.  768x768x512, 1024^2 orbit, aligned copies kept: 1.66 -> 1.48 ms; with
+// every third channel masked (plane bits in shared memory) 333x257x190 frames of 641x479 from the
+// default layout take 336 -> 299 us.
+template <int S, int AX, bool MASK>
+__device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &st, float scale, float qx, float qy, float qz,
+                                                const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
+                                                const unsigned char *s_mask, int org_z, float vcode,
+                                                float &c0, float &c1, float &c2, float &T) {
+    const float nf = (float)n;            // exact: n <= 2^24 + 1, checked by the host
+    const float2 q = pair2(qx, qy), dd = pair2(d[0], d[1]), mm = pair2(kFloorMagic, kFloorMagic);
+    // element of a cell: its rounded-down coordinates' bits times the strides, minus the magic's share
+    const unsigned bias = (unsigned)kFloorMagicBits * (unsigned)(st.x + st.y + st.z);
+    float jf = 0.0f;
+    do {
+        const float tj = __fmul_rn(jf, fc.step);
+        const float2 xy = __ffma2_rn(pair2(tj, tj), dd, q);
+        const float z = __fmaf_rn(tj, d[2], qz);
+        const float2 t = __fadd2_rd(xy, mm);
+        const float tz = __fadd_rd(z, kFloorMagic);
+        const float2 f = sub2(xy, sub2(t, mm));
+        const Cell cl{0, 0, 0, f.x, f.y, __fsub_rn(z, __fsub_rn(tz, kFloorMagic))};
+        const unsigned i0 = __float_as_uint(t.x) * (AX == 0 ? 1u : (unsigned)st.x) + __float_as_uint(t.y) * (AX == 1 ? 1u : (unsigned)st.y) +
+                            __float_as_uint(tz) * (AX == 2 ? 1u : (unsigned)st.z) - bias;
+        float v[8];
+        fetch8_rows<S, AX>(src, (int)i0, st, v);
+        if (MASK) {
+            const int iz = __float_as_int(tz) - kFloorMagicBits;
+            if (s_mask) mask_planes(v, s_mask[iz], vcode);
+            else mask_channels(v, iz, org_z, fc.nz, fc.chmask, vcode);
+        }
+        DvrSample sm;
+        interp_tf(v, cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+        over(sm, c0, c1, c2, T);
         jf = __fadd_rn(jf, 1.0f);
     } while (!(T <= fc.thr) && jf < nf);
     return (int)jf;
@@ -540,10 +617,12 @@ __device__ __forceinline__ int dvr_segment(const void *src, const Strides &st, c
                                            int mx, int my, int mz,
                                            float scale, float qx, float qy, float qz, const float d[3],
                                            int n, const FrameConsts &fc, const float4 *s_lut,
-                                           int org_z, float vcode,
+                                           const unsigned char *s_mask, int org_z, float vcode,
                                            float &c0, float &c1, float &c2, float &T) {
     if constexpr (gathers(F))
-        return dvr_segment_atlas<S, F, MASK>(atl, scale, qx, qy, qz, d, n, fc, s_lut, org_z, vcode, c0, c1, c2, T);
+        return dvr_segment_atlas<S, F, MASK>(atl, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+    if constexpr (straight(F))
+        return dvr_segment_rows<S, row_axis(F), MASK>(src, st, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
     const float vmin = fc.vmin, inv_range = fc.inv_range, lutmax = fc.lutmax, thr = fc.thr;
     const int lmax = fc.nlut - 2;
     int px = -4, py = -4, pz = -4;        // no cell cached yet
@@ -561,9 +640,17 @@ __device__ __forceinline__ int dvr_segment(const void *src, const Strides &st, c
             fetch8_cached<S>(src, st, cl, px, py, pz, v);
         else
             fetch8<S>(src, cl.ix * st.x + cl.iy * st.y + cl.iz * st.z, st, v);
-        if (MASK) mask_channels(v, cl.iz, org_z, fc.nz, fc.chmask, vcode);
         DvrSample sm;
-        interp_tf(v, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
+        if (MASK) {
+            float u[8];                   // (v keeps the stored values: the next cell may share them)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u[k] = v[k];
+            if (s_mask) mask_planes(u, s_mask[cl.iz], vcode);
+            else mask_channels(u, cl.iz, org_z, fc.nz, fc.chmask, vcode);
+            interp_tf(u, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
+        } else {
+            interp_tf(v, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
+        }
         over(sm, c0, c1, c2, T);
         if (T <= thr) return (int)jf + 1;
     }
@@ -594,7 +681,7 @@ template <int S, int MODE, int F, bool MASK>
 __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__restrict__ lut,
                                          DrawBrick *__restrict__ dbs, const TileItem it, int strip, int lane,
                                          const void *__restrict__ pool, void *__restrict__ frags,
-                                         Counters *__restrict__ ctr, float4 *s_lut) {
+                                         Counters *__restrict__ ctr, float4 *s_lut, const unsigned char *s_mask) {
     const DrawBrick &b = dbs[it.db];
     // a warp's 32 rays are adjacent pixels along the image axis the brick layout follows
     int rx, ry;
@@ -624,24 +711,9 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
                 const float qz = anchor(o[2], d[2], b.org_c[2], k0, fc.step);
                 const int n = k1 - k0;
                 const float vcode = S == 0 ? fc.vmin : ldexpf(fc.vmin, -b.exp2);
-                bool inside = true;           // atlas frames: every cell is inside (make_consts)
-                if (!gathers(F)) {
-                    // sample positions are monotone along the ray: when the segment's first and last
-                    // cells are inside the stored brick, every cell in between is too
-                    Cell e0, e1;
-                    const float tl = __fmul_rn((float)(n - 1), fc.step);
-                    cell_of<false>(qx, qy, qz, mx, my, mz, e0);
-                    cell_of<false>(__fmaf_rn(tl, d[0], qx), __fmaf_rn(tl, d[1], qy), __fmaf_rn(tl, d[2], qz),
-                                   mx, my, mz, e1);
-                    inside = min(e0.ix, e1.ix) >= 0 && max(e0.ix, e1.ix) <= mx &&
-                             min(e0.iy, e1.iy) >= 0 && max(e0.iy, e1.iy) <= my &&
-                             min(e0.iz, e1.iz) >= 0 && max(e0.iz, e1.iz) <= mz;
-                }
-                const int j = inside
-                    ? dvr_segment<S, F, false, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
-                                                     s_lut, b.org[2], vcode, c0, c1, c2, T)
-                    : dvr_segment<S, F, true, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
-                                                    s_lut, b.org[2], vcode, c0, c1, c2, T);
+                // (no clamps but for far cameras: every cell is inside the stored brick, kAtlasReach)
+                const int j = dvr_segment<S, F, F == 0, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
+                                                              s_lut, s_mask, b.org[2], vcode, c0, c1, c2, T);
                 nsamp = j;
             }
             // the pixel's place is formed again here, so that the sample loop's registers hold only its own state
@@ -671,15 +743,20 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
                                              __fsub_rn(flz, (float)b.org[2]), g0, g1);
                         gathers_to_stencil(g0, g1, v);
                         iz = jz - b.org[2];
+                    } else if constexpr (straight(F)) {
+                        iz = jz - b.org[2];
+                        fetch8_rows<S, row_axis(F)>(src, (jx - b.org[0]) * st.x + (jy - b.org[1]) * st.y + iz * st.z, st, v);
                     } else {
                         const int ix = clampi(jx - b.org[0], 0, mx);
                         const int iy = clampi(jy - b.org[1], 0, my);
                         iz = clampi(jz - b.org[2], 0, mz);
                         fetch8<S>(src, ix * st.x + iy * st.y + iz * st.z, st, v);
                     }
-                    if (MASK)
-                        mask_channels(v, iz, b.org[2], fc.nz, fc.chmask,
-                                      S == 0 ? fc.vmin : ldexpf(fc.vmin, -b.exp2));
+                    if (MASK) {
+                        const float vcode = S == 0 ? fc.vmin : ldexpf(fc.vmin, -b.exp2);
+                        if (s_mask) mask_planes(v, s_mask[iz], vcode);
+                        else mask_channels(v, iz, b.org[2], fc.nz, fc.chmask, vcode);
+                    }
                     const float c00 = lerp_rn(v[0], v[1], fx);
                     const float c10 = lerp_rn(v[2], v[3], fx);
                     const float c01 = lerp_rn(v[4], v[5], fx);
@@ -708,7 +785,7 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
 // atlas DVR loop without spills.
 template <int MODE, int F>
 constexpr int rc_min_blocks() {
-    return MODE == 0 ? (F == 5 ? VR_PAIR_MIN_BLOCKS : gathers(F) && VR_DVR_MIN_BLOCKS > 0 ? VR_DVR_MIN_BLOCKS : 1)
+    return MODE == 0 ? (straight(F) ? VR_ROWS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : gathers(F) && VR_DVR_MIN_BLOCKS > 0 ? VR_DVR_MIN_BLOCKS : 1)
                      : (VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1);
 }
 
@@ -719,11 +796,15 @@ k_raycast(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__res
           Counters *__restrict__ ctr) {
     extern __shared__ float4 s_lut[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (MODE == 0) {
-        load_table<!entries_only(F)>(lut, fc.nlut, s_lut);
-        __syncthreads();
+    const TileItem it = items[blockIdx.x];
+    unsigned char *s_mask = nullptr;
+    if (MASK && fc.mask_planes > 0) {
+        s_mask = reinterpret_cast<unsigned char *>(s_lut) + (MODE == 0 ? table_bytes(F, fc.nlut) : 0);
+        load_mask_planes(dbs[it.db], fc.nz, fc.chmask, s_mask);
     }
-    rc_strip<S, MODE, F, MASK>(fc, lut, dbs, items[blockIdx.x], warp, lane, pool, frags, ctr, s_lut);
+    if (MODE == 0) load_table<!entries_only(F)>(lut, fc.nlut, s_lut);
+    if (MODE == 0 || MASK) __syncthreads();
+    rc_strip<S, MODE, F, MASK>(fc, lut, dbs, it, warp, lane, pool, frags, ctr, s_lut, s_mask);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -937,7 +1018,7 @@ k_raycast_staged(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick
     bool done = !hit;
     if (hit && !staged) {               // every stencil of this ray from global memory
         j = dvr_segment<0, 0, true, MASK>(src, gst, Atlas{0ull, 0, 0, 0}, mx, my, mz, 1.0f, q[0], q[1], q[2], d,
-                                          n, fc, s_lut, b.org[2], fc.vmin, c0, c1, c2, T);
+                                          n, fc, s_lut, nullptr, b.org[2], fc.vmin, c0, c1, c2, T);
         done = true;
     }
     if (cmax >= cmin) {
@@ -1183,7 +1264,7 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
             wk[kWkSamp * kMarchThreads] = nsamp;
             wk[kWkY0 * kMarchThreads] = __float_as_int(y0); wk[kWkY1 * kMarchThreads] = __float_as_int(y1);
             const int j = dvr_segment<S, F, true, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
-                                                        s_lut, org_z, vcode, c0, c1, c2, T);
+                                                        s_lut, nullptr, org_z, vcode, c0, c1, c2, T);
             wk = march_stash<F>(s_lut, fc.nlut);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -1713,9 +1794,9 @@ template <int S, int MODE, int F, bool MASK>
 cudaError_t launch_rc(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items,
                       int nitems, const void *pool, void *frags, Counters *ctr, cudaStream_t s) {
     static DeviceAttrs da;
-    const size_t smem = MODE == 0 ? table_bytes(F, fc.nlut) : 0;
+    const size_t smem = (MODE == 0 ? table_bytes(F, fc.nlut) : 0) + (MASK ? (size_t)fc.mask_planes : 0);
     const void *kern = reinterpret_cast<const void *>(k_raycast<S, MODE, F, MASK>);
-    cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut), da);
+    cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut) + kMaskPlanes, da);
     if (e != cudaSuccess) return e;
     if (MODE == 0) {
         e = set_carveout(kern, smem, da);
@@ -1751,15 +1832,18 @@ cudaError_t launch_rc_s(const FrameConsts &fc, const float4 *lut, const DrawBric
             return fc.mode != 0 ? VR_RC(1, 5, false) : VR_RC(0, 5, false);
         }
     }
-    const bool atlas = fc.fetch == 2;
-    if (fc.chmask) {     // masked frames: no stencil cache (same values, fewer instantiations)
-        if (fc.mode != 0) return atlas ? VR_RC(1, 2, true) : VR_RC(1, 0, true);
-        return atlas ? VR_RC(0, 2, true) : VR_RC(0, 0, true);
+#define VR_RC_MASKED(MODE, F) (fc.chmask ? VR_RC(MODE, F, true) : VR_RC(MODE, F, false))
+#define VR_RC_MODE(F) (fc.mode != 0 ? VR_RC_MASKED(1, F) : VR_RC_MASKED(0, F))
+    switch (fc.fetch) {
+        case 1: return VR_RC_MASKED(0, 1);
+        case 2: return VR_RC_MODE(2);
+        case 6: return VR_RC_MODE(6);
+        case 7: return VR_RC_MODE(7);
+        case 8: return VR_RC_MODE(8);
+        default: return VR_RC_MODE(0);
     }
-    if (fc.mode != 0) return atlas ? VR_RC(1, 2, false) : VR_RC(1, 0, false);
-    if (atlas) return VR_RC(0, 2, false);
-    if (fc.fetch == 1) return VR_RC(0, 1, false);
-    return VR_RC(0, 0, false);
+#undef VR_RC_MODE
+#undef VR_RC_MASKED
 #undef VR_RC
 }
 
