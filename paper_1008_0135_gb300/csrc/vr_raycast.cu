@@ -19,24 +19,30 @@
 
 #include "vr_internal.cuh"
 
-// Tuning knobs of the ray-cast kernels (build-time): unroll factor of the DVR sample loop, the
-// blocks per SM the register allocation of the fragment kernel must allow for DVR frames read
-// through slice atlases and for MIP frames (0: no constraint), and the same for the one-pass
-// (global termination) kernel.
+// Tuning knobs of the ray-cast kernels (build-time): unroll factor of the linear sample loops, samples
+// fetched ahead (slice atlases, pair atlases, linear rows), the blocks per SM the register
+// allocation must allow for DVR frames read through atlases, through linear rows and for MIP
+// frames (0: no constraint), and the same for the one-pass (global termination) kernel.
 #ifndef VR_SAMPLE_UNROLL
 #define VR_SAMPLE_UNROLL 1
 #endif
 #ifndef VR_DVR_MIN_BLOCKS
-#define VR_DVR_MIN_BLOCKS 6
+#define VR_DVR_MIN_BLOCKS 4
+#endif
+#ifndef VR_AHEAD
+#define VR_AHEAD 2
+#endif
+#ifndef VR_AHEAD_PAIR
+#define VR_AHEAD_PAIR 3
+#endif
+#ifndef VR_AHEAD_ROWS
+#define VR_AHEAD_ROWS 2
 #endif
 #ifndef VR_ROWS_MIN_BLOCKS
 #define VR_ROWS_MIN_BLOCKS 4
 #endif
 #ifndef VR_MIP_MIN_BLOCKS
 #define VR_MIP_MIN_BLOCKS 0
-#endif
-#ifndef VR_PAIR_MIN_BLOCKS
-#define VR_PAIR_MIN_BLOCKS 8
 #endif
 #ifndef VR_RAYMARCH_MIN_BLOCKS
 #define VR_RAYMARCH_MIN_BLOCKS 5
@@ -235,9 +241,7 @@ __device__ __forceinline__ Corners lerp_z(const float4 &g0, const float4 &g1, fl
     return Corners{lo.y, lo.x, hi.x, hi.y};
 }
 
-// Trilinear value from the corners at the sample's z, then the table lookup.  DIFF: the table holds
-// the differences too; else the next entry is read and the (same) difference formed here.
-template <bool DIFF = true>
+// Trilinear value from the corners at the sample's z, then the table lookup.
 __device__ __forceinline__ void interp_tf(const Corners &q, const Cell &c, bool scaled, float scale,
                                           float vmin, float inv_range, float lutmax, int lmax,
                                           const float4 *s_lut, DvrSample &o) {
@@ -245,11 +249,8 @@ __device__ __forceinline__ void interp_tf(const Corners &q, const Cell &c, bool 
     const float b0 = __fmaf_rn(c.fx, __fsub_rn(q.c1, q.c0), q.c0);
     const float b1 = __fmaf_rn(c.fx, __fsub_rn(q.c3, q.c2), q.c2);
     const float val = __fmaf_rn(c.fy, __fsub_rn(b1, b0), b0);
-    // (a brick's scale is a power of two: val scale is exact, so either form rounds once; the pair
-    // kernel's 32 registers come out better with two operations)
-    const float off = !scaled ? __fsub_rn(val, vmin)
-                      : DIFF  ? __fmaf_rn(val, scale, -vmin)
-                              : __fsub_rn(__fmul_rn(val, scale), vmin);
+    // (a brick's scale is a power of two: val scale is exact, and the difference rounded once)
+    const float off = scaled ? __fmaf_rn(val, scale, -vmin) : __fsub_rn(val, vmin);
     o.u = __fmul_rn(off, inv_range);
     const float uc = __saturatef(o.u);          // clamp to [0, 1] (one instruction)
     // interval floor(uc lutmax) of the exact product, and the fraction with one rounding.  uc = 1
@@ -259,13 +260,7 @@ __device__ __forceinline__ void interp_tf(const Corners &q, const Cell &c, bool 
     o.li = __float_as_int(t) - kFloorMagicBits;
     o.lf = __fmaf_rn(uc, lutmax, -__fsub_rn(t, kFloorMagic));
     o.L0 = s_lut[tab_entry(o.li, lmax + 2)];
-    if (DIFF) {
-        o.D = s_lut[tab_diff(o.li, lmax + 2)];
-    } else {
-        const float4 e = s_lut[o.li + 1];
-        const float2 xy = sub2(pair2(e.x, e.y), pair2(o.L0.x, o.L0.y)), zw = sub2(pair2(e.z, e.w), pair2(o.L0.z, o.L0.w));
-        o.D = make_float4(xy.x, xy.y, zw.x, zw.y);
-    }
+    o.D = s_lut[tab_diff(o.li, lmax + 2)];
     const float2 ff = pair2(o.lf, o.lf);
     const float2 rg = __ffma2_rn(ff, pair2(o.D.x, o.D.y), pair2(o.L0.x, o.L0.y));
     const float2 ba = __ffma2_rn(ff, pair2(o.D.z, o.D.w), pair2(o.L0.z, o.L0.w));
@@ -277,23 +272,12 @@ __device__ __forceinline__ void interp_tf(const float v[8], const Cell &c, bool 
     interp_tf(lerp_z(v, c.fz), c, scaled, scale, vmin, inv_range, lutmax, lmax, s_lut, o);
 }
 
-// Pair-atlas frames keep the entries alone (the last one twice) in shared memory: their loop has
-// room for two packed subtractions a sample, and half the table leaves L1 to the texels of 8
-// resident CTAs (HIPASS-scale FP16 pair frames 3.39 ms with both arrays, 2.92 with entries only).
-constexpr bool entries_only(int F) { return F == 5; }
-constexpr size_t table_bytes(int F, int n) { return sizeof(float4) * (entries_only(F) ? (size_t)n + 1 : 2 * (size_t)n); }
-
 // The table in shared memory with its differences entry i+1 - entry i: the same IEEE
 // subtractions a lookup would do, made once per block instead of once per sample.
-template <bool DIFF = true>
+constexpr size_t table_bytes(int n) { return 2 * sizeof(float4) * (size_t)n; }
 __device__ __forceinline__ void load_table(const float4 *__restrict__ lut, int n, float4 *s) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const float4 a = lut[i];
-        if (!DIFF) {
-            s[i] = a;
-            if (i + 1 == n) s[n] = a;
-            continue;
-        }
         const float4 b = i + 1 < n ? lut[i + 1] : a;
         s[tab_entry(i, n)] = a;
         s[tab_diff(i, n)] = make_float4(__fsub_rn(b.x, a.x), __fsub_rn(b.y, a.y), __fsub_rn(b.z, a.z),
@@ -391,6 +375,9 @@ __device__ __forceinline__ void gather_stencil(const Atlas &a, float2 ixy, float
 // Whether fetch mode F reads rows of a linear copy without clamps, and the copy's contiguous axis.
 constexpr bool straight(int F) { return F >= 6; }
 constexpr int row_axis(int F) { return F - 6; }
+
+// Samples whose stencils a fragment kernel's segment loop fetches before it composites the first.
+constexpr int ahead(int F) { return F == 2 ? VR_AHEAD : F == 5 ? VR_AHEAD_PAIR : F >= 6 ? VR_AHEAD_ROWS : 1; }
 
 // Whether fetch mode F reads a texture (the slice atlas, 2, or the pair atlas, 5).
 constexpr bool gathers(int F) { return F == 2 || F == 5; }
@@ -531,10 +518,16 @@ __device__ __forceinline__ void over(const DvrSample &s, float &c0, float &c1, f
 // whole-number floats, the slices placed so that no sample tests for a column's end, z
 // interpolated first (packed), the two exits one branch.  No index is clamped: the host takes this
 // path only for cameras near enough that rounding cannot move a sample half a voxel (kAtlasReach).
-// Frames of 1024^2 at step 1, before -> after: 1720x1720x1024 FP32 3.43 -> 3.35 ms, FP16 2.88 ->
-// 2.79; 768x768x512 global termination 0.64 -> 0.59 ms, MIP 1.31 -> 1.27; pair atlases unchanged
-// within 1 % (8 CTAs at 32 registers without software pipelining against 6 with it).
-template <int S, int F, bool MASK>
+// The stencils of AHEAD samples are fetched before the first of them is composited: two with slice
+// atlases and three with pair atlases at 4 CTAs of 64 registers, which beats more warps with one
+// sample each (fewer rays share the texture cache) and more samples or fewer warps.
+// 1024^2 frames at step 1, ms: integer cells -> one sample at a time -> ahead.  1720x1720x1024 FP32
+// 3.54 -> 3.41 -> 3.26, FP16 2.95 -> 2.82 -> 2.74, FP16 pair atlas 2.94 -> 2.92 -> 2.56;
+// 768x768x512 FP32 1.36 -> 1.31 -> 1.29; 256^3 at 512^2, step 0.5: 0.35 -> 0.34 -> 0.31;
+// 2048x2048x256 BF16 pair atlas, step 0.5: 1.07 -> 1.06 -> 0.89.  Global termination (one sample at a
+// time: two spill) 768x768x512 0.64 -> 0.59.  Two ahead at 5 CTAs: 3.53 (FP32 1720x1720x1024), three
+// at 4: 3.44, four at 2: 3.71; pair atlas two at 4: 2.88, four at 4: 2.96, three at 5: 3.07.
+template <int S, bool MASK>
 __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const CellF &c, float scale, const FrameConsts &fc,
                                       const float4 *s_lut, const unsigned char *s_mask, int org_z, float vcode, float &c0,
                                       float &c1, float &c2, float &T) {
@@ -545,30 +538,51 @@ __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const 
         gathers_to_stencil(g0, g1, v);
         if (s_mask) mask_planes(v, s_mask[small_float_int(c.iz)], vcode);
         else mask_channels(v, small_float_int(c.iz), org_z, fc.nz, fc.chmask, vcode);
-        interp_tf<!entries_only(F)>(lerp_z(v, cl.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+        interp_tf(lerp_z(v, cl.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
     } else {
-        interp_tf<!entries_only(F)>(lerp_z(g0, g1, c.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+        interp_tf(lerp_z(g0, g1, c.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
     }
     over(sm, c0, c1, c2, T);
 }
 
-template <int S, int F, bool MASK>
+template <int S, int F, bool MASK, int AHEAD>
 __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, float qx, float qy, float qz,
                                                  const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
                                                  const unsigned char *s_mask, int org_z, float vcode, float &c0, float &c1, float &c2, float &T) {
     const float nf = (float)n;            // exact: n <= 2^24 + 1, checked by the host
     const float2 q = pair2(qx, qy), dd = pair2(d[0], d[1]);
     float jf = 0.0f;
-#pragma unroll kSampleUnroll
-    do {
-        const float tj = __fmul_rn(jf, fc.step);
-        const CellF cl = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
-        float4 g0, g1;
-        gather_stencil<S, F>(atl, cl.ixy, cl.iz, g0, g1);
-        shade<S, F, MASK>(g0, g1, cl, scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
-        jf = __fadd_rn(jf, 1.0f);
-    } while (!(T <= fc.thr) && jf < nf);
-    return (int)jf;
+    if constexpr (AHEAD > 1) {
+        // the gathers of AHEAD samples, then the samples in order (past the segment's end: its last
+        // sample's again, unused)
+        const float nl = __fsub_rn(nf, 1.0f);
+        for (;;) {
+            CellF cl[AHEAD];
+            float4 g0[AHEAD], g1[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                const float tj = __fmul_rn(u ? fminf(__fadd_rn(jf, (float)u), nl) : jf, fc.step);
+                cl[u] = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
+                gather_stencil<S, F>(atl, cl[u].ixy, cl[u].iz, g0[u], g1[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                shade<S, MASK>(g0[u], g1[u], cl[u], scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+                jf = __fadd_rn(jf, 1.0f);
+                if (T <= fc.thr || !(jf < nf)) return (int)jf;
+            }
+        }
+    } else {
+        do {
+            const float tj = __fmul_rn(jf, fc.step);
+            const CellF cl = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
+            float4 g0, g1;
+            gather_stencil<S, F>(atl, cl.ixy, cl.iz, g0, g1);
+            shade<S, MASK>(g0, g1, cl, scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+            jf = __fadd_rn(jf, 1.0f);
+        } while (!(T <= fc.thr) && jf < nf);
+        return (int)jf;
+    }
 }
 
 // The segment loop over rows of a linear copy, for cameras near enough that no index needs a clamp.
@@ -577,7 +591,7 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
 // neighbours are constant offsets.  768x768x512, 1024^2 orbit, aligned copies kept: 1.66 -> 1.48 ms; with
 // every third channel masked (plane bits in shared memory) 333x257x190 frames of 641x479 from the
 // default layout take 336 -> 299 us.
-template <int S, int AX, bool MASK>
+template <int S, int AX, bool MASK, int AHEAD>
 __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &st, float scale, float qx, float qy, float qz,
                                                 const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
                                                 const unsigned char *s_mask, int org_z, float vcode,
@@ -586,33 +600,44 @@ __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &
     const float2 q = pair2(qx, qy), dd = pair2(d[0], d[1]), mm = pair2(kFloorMagic, kFloorMagic);
     // element of a cell: its rounded-down coordinates' bits times the strides, minus the magic's share
     const unsigned bias = (unsigned)kFloorMagicBits * (unsigned)(st.x + st.y + st.z);
+    const float nl = __fsub_rn(nf, 1.0f);
     float jf = 0.0f;
-    do {
-        const float tj = __fmul_rn(jf, fc.step);
-        const float2 xy = __ffma2_rn(pair2(tj, tj), dd, q);
-        const float z = __fmaf_rn(tj, d[2], qz);
-        const float2 t = __fadd2_rd(xy, mm);
-        const float tz = __fadd_rd(z, kFloorMagic);
-        const float2 f = sub2(xy, sub2(t, mm));
-        const Cell cl{0, 0, 0, f.x, f.y, __fsub_rn(z, __fsub_rn(tz, kFloorMagic))};
-        const unsigned i0 = __float_as_uint(t.x) * (AX == 0 ? 1u : (unsigned)st.x) + __float_as_uint(t.y) * (AX == 1 ? 1u : (unsigned)st.y) +
-                            __float_as_uint(tz) * (AX == 2 ? 1u : (unsigned)st.z) - bias;
-        float v[8];
-        fetch8_rows<S, AX>(src, (int)i0, st, v);
-        if (MASK) {
-            const int iz = __float_as_int(tz) - kFloorMagicBits;
-            if (s_mask) mask_planes(v, s_mask[iz], vcode);
-            else mask_channels(v, iz, org_z, fc.nz, fc.chmask, vcode);
+    for (;;) {
+        float v[AHEAD][8], fx[AHEAD], fy[AHEAD], fz[AHEAD];
+        int iz[AHEAD];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {        // (past the end: the last sample's loads again)
+            const float tj = __fmul_rn(u ? fminf(__fadd_rn(jf, (float)u), nl) : jf, fc.step);
+            const float2 xy = __ffma2_rn(pair2(tj, tj), dd, q);
+            const float z = __fmaf_rn(tj, d[2], qz);
+            const float2 t = __fadd2_rd(xy, mm);
+            const float tz = __fadd_rd(z, kFloorMagic);
+            const float2 f = sub2(xy, sub2(t, mm));
+            fx[u] = f.x;
+            fy[u] = f.y;
+            fz[u] = __fsub_rn(z, __fsub_rn(tz, kFloorMagic));
+            iz[u] = __float_as_int(tz) - kFloorMagicBits;
+            const unsigned i0 = __float_as_uint(t.x) * (AX == 0 ? 1u : (unsigned)st.x) + __float_as_uint(t.y) * (AX == 1 ? 1u : (unsigned)st.y) +
+                                __float_as_uint(tz) * (AX == 2 ? 1u : (unsigned)st.z) - bias;
+            fetch8_rows<S, AX>(src, (int)i0, st, v[u]);
         }
-        DvrSample sm;
-        interp_tf(v, cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
-        over(sm, c0, c1, c2, T);
-        jf = __fadd_rn(jf, 1.0f);
-    } while (!(T <= fc.thr) && jf < nf);
-    return (int)jf;
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            if (MASK) {
+                if (s_mask) mask_planes(v[u], s_mask[iz[u]], vcode);
+                else mask_channels(v[u], iz[u], org_z, fc.nz, fc.chmask, vcode);
+            }
+            const Cell cl{0, 0, 0, fx[u], fy[u], fz[u]};
+            DvrSample sm;
+            interp_tf(v[u], cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
+            over(sm, c0, c1, c2, T);
+            jf = __fadd_rn(jf, 1.0f);
+            if (T <= fc.thr || !(jf < nf)) return (int)jf;
+        }
+    }
 }
 
-template <int S, int F, bool CLAMP, bool MASK>
+template <int S, int F, bool CLAMP, bool MASK, int AHEAD>
 __device__ __forceinline__ int dvr_segment(const void *src, const Strides &st, const Atlas &atl,
                                            int mx, int my, int mz,
                                            float scale, float qx, float qy, float qz, const float d[3],
@@ -620,9 +645,9 @@ __device__ __forceinline__ int dvr_segment(const void *src, const Strides &st, c
                                            const unsigned char *s_mask, int org_z, float vcode,
                                            float &c0, float &c1, float &c2, float &T) {
     if constexpr (gathers(F))
-        return dvr_segment_atlas<S, F, MASK>(atl, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+        return dvr_segment_atlas<S, F, MASK, AHEAD>(atl, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
     if constexpr (straight(F))
-        return dvr_segment_rows<S, row_axis(F), MASK>(src, st, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+        return dvr_segment_rows<S, row_axis(F), MASK, AHEAD>(src, st, scale, qx, qy, qz, d, n, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
     const float vmin = fc.vmin, inv_range = fc.inv_range, lutmax = fc.lutmax, thr = fc.thr;
     const int lmax = fc.nlut - 2;
     int px = -4, py = -4, pz = -4;        // no cell cached yet
@@ -712,7 +737,7 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
                 const int n = k1 - k0;
                 const float vcode = S == 0 ? fc.vmin : ldexpf(fc.vmin, -b.exp2);
                 // (no clamps but for far cameras: every cell is inside the stored brick, kAtlasReach)
-                const int j = dvr_segment<S, F, F == 0, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
+                const int j = dvr_segment<S, F, F == 0, MASK, ahead(F)>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
                                                               s_lut, s_mask, b.org[2], vcode, c0, c1, c2, T);
                 nsamp = j;
             }
@@ -785,7 +810,7 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
 // atlas DVR loop without spills.
 template <int MODE, int F>
 constexpr int rc_min_blocks() {
-    return MODE == 0 ? (straight(F) ? VR_ROWS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : gathers(F) && VR_DVR_MIN_BLOCKS > 0 ? VR_DVR_MIN_BLOCKS : 1)
+    return MODE == 0 ? (straight(F) ? VR_ROWS_MIN_BLOCKS : gathers(F) && VR_DVR_MIN_BLOCKS > 0 ? VR_DVR_MIN_BLOCKS : 1)
                      : (VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1);
 }
 
@@ -799,10 +824,10 @@ k_raycast(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__res
     const TileItem it = items[blockIdx.x];
     unsigned char *s_mask = nullptr;
     if (MASK && fc.mask_planes > 0) {
-        s_mask = reinterpret_cast<unsigned char *>(s_lut) + (MODE == 0 ? table_bytes(F, fc.nlut) : 0);
+        s_mask = reinterpret_cast<unsigned char *>(s_lut) + (MODE == 0 ? table_bytes(fc.nlut) : 0);
         load_mask_planes(dbs[it.db], fc.nz, fc.chmask, s_mask);
     }
-    if (MODE == 0) load_table<!entries_only(F)>(lut, fc.nlut, s_lut);
+    if (MODE == 0) load_table(lut, fc.nlut, s_lut);
     if (MODE == 0 || MASK) __syncthreads();
     rc_strip<S, MODE, F, MASK>(fc, lut, dbs, it, warp, lane, pool, frags, ctr, s_lut, s_mask);
 }
@@ -1017,7 +1042,7 @@ k_raycast_staged(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick
     int j = 0;
     bool done = !hit;
     if (hit && !staged) {               // every stencil of this ray from global memory
-        j = dvr_segment<0, 0, true, MASK>(src, gst, Atlas{0ull, 0, 0, 0}, mx, my, mz, 1.0f, q[0], q[1], q[2], d,
+        j = dvr_segment<0, 0, true, MASK, 1>(src, gst, Atlas{0ull, 0, 0, 0}, mx, my, mz, 1.0f, q[0], q[1], q[2], d,
                                           n, fc, s_lut, nullptr, b.org[2], fc.vmin, c0, c1, c2, T);
         done = true;
     }
@@ -1150,11 +1175,10 @@ constexpr size_t kMarchStashBytes = (size_t)kWkSlots * kMarchThreads * sizeof(in
 
 // This thread's first stash slot.  The thread index is read with a volatile move so that the
 // address is formed anew at each use instead of held in a register across the sample loop.
-template <int F>
 __device__ __forceinline__ volatile int *march_stash(float4 *s_lut, int nlut) {
     unsigned tid;
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
-    return reinterpret_cast<volatile int *>(s_lut + table_bytes(F, nlut) / sizeof(float4)) + tid;
+    return reinterpret_cast<volatile int *>(s_lut + table_bytes(nlut) / sizeof(float4)) + tid;
 }
 
 // One CTA = a 32x8 (8x32) pixel tile of the frame.  Each ray is clipped to the cube (and the
@@ -1175,7 +1199,7 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
            const MarchGrid g, const void *__restrict__ pool, float4 *__restrict__ out,
            Counters *__restrict__ ctr) {
     extern __shared__ float4 s_lut[];
-    load_table<!entries_only(F)>(lut, fc.nlut, s_lut);
+    load_table(lut, fc.nlut, s_lut);
     __syncthreads();
     int nsamp = 0;
     float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, T = 1.0f;
@@ -1191,7 +1215,7 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
         const int px = fc.lanes_y ? tx * kMarchWarps + w : tx * kRcLong + lane;
         const int py = fc.lanes_y ? ty * kRcLong + lane : ty * kMarchWarps + w;
         const bool inframe = px < fc.cam.W && py < fc.cam.H;
-        march_stash<F>(s_lut, fc.nlut)[kWkPix * kMarchThreads] = inframe ? py * fc.cam.W + px : -1;      // frames hold < 2^31 pixels
+        march_stash(s_lut, fc.nlut)[kWkPix * kMarchThreads] = inframe ? py * fc.cam.W + px : -1;      // frames hold < 2^31 pixels
         if (inframe) {
             ray_eye(fc.cam, px, py, y0, y1, d);
             float o[3];
@@ -1254,7 +1278,7 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
             const int n = kend - k;
             const float vcode = S == 0 ? fc.vmin : ldexpf(fc.vmin, -b.exp2);
             const int org_z = b.org[2];
-            volatile int *wk = march_stash<F>(s_lut, fc.nlut);
+            volatile int *wk = march_stash(s_lut, fc.nlut);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 wk[(kWkX0 + a) * kMarchThreads] = kx[a];
@@ -1263,9 +1287,9 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
             wk[kWkK1 * kMarchThreads] = K1; wk[kWkEnd * kMarchThreads] = kend; wk[kWkGuard * kMarchThreads] = guard;
             wk[kWkSamp * kMarchThreads] = nsamp;
             wk[kWkY0 * kMarchThreads] = __float_as_int(y0); wk[kWkY1 * kMarchThreads] = __float_as_int(y1);
-            const int j = dvr_segment<S, F, true, MASK>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
+            const int j = dvr_segment<S, F, true, MASK, 1>(src, st, atl, mx, my, mz, scale, qx, qy, qz, d, n, fc,
                                                         s_lut, nullptr, org_z, vcode, c0, c1, c2, T);
-            wk = march_stash<F>(s_lut, fc.nlut);
+            wk = march_stash(s_lut, fc.nlut);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 kx[a] = wk[(kWkX0 + a) * kMarchThreads];
@@ -1294,7 +1318,7 @@ k_raymarch(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__re
         if (out_of_grid) break;
         k = kend;
     }
-    const int pix = march_stash<F>(s_lut, fc.nlut)[kWkPix * kMarchThreads];
+    const int pix = march_stash(s_lut, fc.nlut)[kWkPix * kMarchThreads];
     if (pix >= 0) out[pix] = make_float4(c0, c1, c2, 1.0f - T);
     const unsigned int tot = __reduce_add_sync(0xffffffffu, (unsigned int)nsamp);
     if ((threadIdx.x & 31) == 0 && tot > 0) atomicAdd(&ctr->samples, (unsigned long long)tot);
@@ -1794,7 +1818,7 @@ template <int S, int MODE, int F, bool MASK>
 cudaError_t launch_rc(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items,
                       int nitems, const void *pool, void *frags, Counters *ctr, cudaStream_t s) {
     static DeviceAttrs da;
-    const size_t smem = (MODE == 0 ? table_bytes(F, fc.nlut) : 0) + (MASK ? (size_t)fc.mask_planes : 0);
+    const size_t smem = (MODE == 0 ? table_bytes(fc.nlut) : 0) + (MASK ? (size_t)fc.mask_planes : 0);
     const void *kern = reinterpret_cast<const void *>(k_raycast<S, MODE, F, MASK>);
     cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut) + kMaskPlanes, da);
     if (e != cudaSuccess) return e;
@@ -1864,7 +1888,7 @@ cudaError_t launch_march(const FrameConsts &fc, const float4 *lut, DrawBrick *br
     static DeviceAttrs da;
     const void *kern = reinterpret_cast<const void *>(k_raymarch<S, F, MASK>);
     cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut + kMarchStashBytes), da);
-    const size_t smem = table_bytes(F, fc.nlut) + kMarchStashBytes;
+    const size_t smem = table_bytes(fc.nlut) + kMarchStashBytes;
     if (e == cudaSuccess) e = set_carveout(kern, smem, da, kMarchWarps);
     if (e != cudaSuccess) return e;
     const int tw = fc.lanes_y ? kMarchWarps : kRcLong, th = fc.lanes_y ? kRcLong : kMarchWarps;
