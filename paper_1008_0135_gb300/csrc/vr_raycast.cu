@@ -1859,7 +1859,9 @@ cudaError_t launch_rc_s(const FrameConsts &fc, const float4 *lut, const DrawBric
 #define VR_RC_MASKED(MODE, F) (fc.chmask ? VR_RC(MODE, F, true) : VR_RC(MODE, F, false))
 #define VR_RC_MODE(F) (fc.mode != 0 ? VR_RC_MASKED(1, F) : VR_RC_MASKED(0, F))
     switch (fc.fetch) {
-        case 1: return VR_RC_MASKED(0, 1);
+        case 1:                        // (masked frames of 16-bit bricks read rows)
+            if constexpr (S == 0) return VR_RC_MASKED(0, 1);
+            else return VR_RC(0, 1, false);
         case 2: return VR_RC_MODE(2);
         case 6: return VR_RC_MODE(6);
         case 7: return VR_RC_MODE(7);
