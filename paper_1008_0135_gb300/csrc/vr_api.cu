@@ -28,6 +28,50 @@ int set_dev(vr_ctx *c) {
     return VR_OK;
 }
 
+static void idle_array_free(IdleArray &a) {
+    if (a.tex) cudaDestroyTextureObject(a.tex);
+    if (a.surf) cudaDestroySurfaceObject(a.surf);
+    if (a.arr) cudaFreeArray(a.arr);
+}
+
+void idle_slot_free(IdleSlot &s) {
+    if (s.h_stage) cudaFreeHost(s.h_stage);
+    if (s.d_stage.p) cudaFree(s.d_stage.p);
+    if (s.d_frags.p) cudaFree(s.d_frags.p);
+    if (s.d_out.p) cudaFree(s.d_out.p);
+    for (cudaEvent_t e : {s.done, s.upload_done, s.frame_done})
+        if (e) cudaEventDestroy(e);
+    if (s.s) cudaStreamDestroy(s.s);
+    s = IdleSlot{};
+}
+
+void idle_release(vr_ctx *c) {
+    if (c->parent) c = c->parent;
+    std::lock_guard<std::mutex> l(c->idle_mu);
+    for (auto &a : c->idle_arrays) idle_array_free(a);
+    c->idle_arrays.clear();
+    for (auto &s : c->idle_slots) idle_slot_free(s);
+    c->idle_slots.clear();
+    if (c->mem) {
+        cudaStreamSynchronize(c->load_stream);
+        cudaMemPoolTrimTo(c->mem, 0);
+    }
+}
+
+// cudaMalloc and cudaFree of a cube's buffers cost 0.1 - 0.2 ms each (mapping, device-wide waits): 1.0 of
+// the 3.4 ms that ingesting a 741 MB cube took, and 0.5 ms for its atlas arrays.
+cudaError_t mem_alloc(vr_ctx *c, void **p, size_t bytes) {
+    return alloc_retry(c, [&] {
+        return c->mem ? cudaMallocFromPoolAsync(p, bytes, c->mem, c->load_stream) : cudaMalloc(p, bytes);
+    });
+}
+
+void mem_free(vr_ctx *c, void *p) {
+    if (!p) return;
+    if (c->mem) cudaFreeAsync(p, c->load_stream);
+    else cudaFree(p);
+}
+
 void layout_strides(const int dim[3], int layout, int str[3]) {
     // the contiguous axis first, then the other two in x, y, z order
     int ord[3];
@@ -737,24 +781,55 @@ bool own_device_memory(const void *p, int dev) {
     return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
-// Releases a cube's slice atlases.  Frames in flight may still gather from them: the device is
-// drained first (atlases go only with the bricking).
-void free_atlases(Cube *cb) {
+// Releases a cube's slice atlases (to the context's idle arrays while those are few).  Frames in
+// flight may still gather from them: the device is drained first (atlases go only with the bricking).
+void free_atlases(vr_ctx *c, Cube *cb) {
     if (cb->atlas_arr.empty() && cb->atlas_tex.empty()) return;
     cudaDeviceSynchronize();
-    for (auto t : cb->atlas_tex)
-        if (t) cudaDestroyTextureObject(t);
-    for (auto f : cb->atlas_surf)
-        if (f) cudaDestroySurfaceObject(f);
-    for (auto a : cb->atlas_arr)
-        if (a) cudaFreeArray(a);
+    std::lock_guard<std::mutex> l(c->idle_mu);
+    size_t kept = 0;
+    for (auto &a : c->idle_arrays) kept += a.bytes;
+    for (size_t i = 0; i < cb->atlas_arr.size(); ++i) {
+        IdleArray a;
+        a.arr = cb->atlas_arr[i];
+        a.tex = i < cb->atlas_tex.size() ? cb->atlas_tex[i] : 0;
+        a.surf = i < cb->atlas_surf.size() ? cb->atlas_surf[i] : 0;
+        if (i < cb->atlas_dims.size()) {
+            a.w = cb->atlas_dims[i].first;
+            a.h = cb->atlas_dims[i].second;
+        }
+        a.kind = cb->atlas_kind;
+        a.bytes = (size_t)a.w * a.h * (a.kind == 0 || a.kind == 3 ? 4 : 2);
+        if (a.tex && a.surf && a.w > 0 && kept + a.bytes <= kIdleArrayBytes && c->idle_arrays.size() < 256) {
+            kept += a.bytes;
+            c->idle_arrays.push_back(a);
+        } else {
+            idle_array_free(a);
+        }
+    }
     cb->atlas_tex.clear();
     cb->atlas_surf.clear();
     cb->atlas_arr.clear();
+    cb->atlas_dims.clear();
     cb->atlas_cells.clear();
     cb->atlas_of.clear();
     cb->atlas_pair = false;
     for (auto &d : cb->tmpl) d.atlas = 0;
+}
+
+// An array of w x h texels that a freed cube left, for cb; every texel that a frame reads is written again.
+static bool take_idle_array(vr_ctx *c, Cube *cb, int w, int h) {
+    std::lock_guard<std::mutex> l(c->idle_mu);
+    for (auto it = c->idle_arrays.begin(); it != c->idle_arrays.end(); ++it) {
+        if (it->w != w || it->h != h || it->kind != cb->atlas_kind) continue;
+        cb->atlas_arr.push_back(it->arr);
+        cb->atlas_tex.push_back(it->tex);
+        cb->atlas_surf.push_back(it->surf);
+        cb->atlas_dims.push_back({w, h});
+        c->idle_arrays.erase(it);
+        return true;
+    }
+    return false;
 }
 
 // Arrays for the slice atlas of every brick (layout bit 3), each brick's placed by
@@ -769,7 +844,7 @@ void free_atlases(Cube *cb) {
 // Arrays must fit the device's limit for 2D gathers.
 constexpr int kAtlasRowBytes = 8192;
 int make_atlases(vr_ctx *c, Cube *cb) {
-    free_atlases(cb);
+    free_atlases(c, cb);
     const int nbr = (int)cb->tmpl.size();
     const bool pair = (cb->layouts & 32) && cb->storage != VR_F32;
     std::vector<AtlasGeom> geo(nbr);
@@ -812,15 +887,19 @@ int make_atlases(vr_ctx *c, Cube *cb) {
                                    : cb->storage == VR_F16 ? cudaCreateChannelDescHalf()
                                                            : cudaCreateChannelDesc(16, 0, 0, 0, cudaChannelFormatKindUnsigned);
     auto bail = [&](cudaError_t e, const char *what) {
-        free_atlases(cb);
+        free_atlases(c, cb);
         return cuda_fail(e, what);
     };
     cudaError_t e;
+    cb->atlas_kind = pair ? 3 : cb->storage == VR_F32 ? 0 : cb->storage == VR_F16 ? 1 : 2;
     for (const Dim &d : dims) {
+        if (take_idle_array(c, cb, d.w, d.h)) continue;
         cudaArray_t arr = nullptr;
         // written through a surface where the device allows surface stores on a gather array; else
         // packed into staging and copied (the copy engine's array writes)
-        const bool surf_ok = cudaMallocArray(&arr, &cd, d.w, d.h, cudaArrayTextureGather | cudaArraySurfaceLoadStore) == cudaSuccess;
+        const unsigned both = cudaArrayTextureGather | cudaArraySurfaceLoadStore;
+        e = alloc_retry(c, [&] { return cudaMallocArray(&arr, &cd, d.w, d.h, both); });
+        const bool surf_ok = e == cudaSuccess;
         if (!surf_ok) {
             arr = nullptr;
             cudaGetLastError();
@@ -828,6 +907,7 @@ int make_atlases(vr_ctx *c, Cube *cb) {
                 return bail(e, "cudaMallocArray (slice atlas)");
         }
         cb->atlas_arr.push_back(arr);
+        cb->atlas_dims.push_back({d.w, d.h});
         cudaResourceDesc rd{};
         rd.resType = cudaResourceTypeArray;
         rd.res.array.array = arr;
@@ -855,7 +935,7 @@ int make_atlases(vr_ctx *c, Cube *cb) {
 
 // The atlases from the pool's x-contiguous copies, through staging: where the device refuses
 // surface stores on a gather array.
-int stage_atlases(Cube *cb, cudaStream_t s) {
+int stage_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
     const size_t bsz = cb->storage == VR_F32 ? 4 : 2;        // bytes of a stored element
     const size_t esz = cb->atlas_pair ? 4 : bsz;             // bytes of a texel
     size_t most = 16;
@@ -871,7 +951,7 @@ int stage_atlases(Cube *cb, cudaStream_t s) {
         most = std::max(most, w * h * esz);
     }
     void *tmp = nullptr;
-    CK(cudaMalloc(&tmp, most));
+    CK(alloc_retry(c, [&] { return cudaMalloc(&tmp, most); }));
     cudaError_t e = cudaMemsetAsync(tmp, 0, most, s);
     for (size_t i = 0; i < cb->tmpl.size() && e == cudaSuccess; ++i) {
         const AtlasCell &cell = cb->atlas_cells[i];
@@ -888,7 +968,7 @@ int stage_atlases(Cube *cb, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(tmp);
     if (e != cudaSuccess) {
-        free_atlases(cb);
+        free_atlases(c, cb);
         return cuda_fail(e, "slice atlas build");
     }
     return VR_OK;
@@ -902,7 +982,7 @@ int stage_atlases(Cube *cb, cudaStream_t s) {
 int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
     const int nbr = (int)cb->tmpl.size();
     int rc;
-    if (!(cb->layouts & 8)) free_atlases(cb);
+    if (!(cb->layouts & 8)) free_atlases(c, cb);
     else if (cb->atlas_arr.empty()) { if ((rc = make_atlases(c, cb)) != VR_OK) return rc; }
     else CK(cudaDeviceSynchronize());        // frames in flight may still gather from the arrays
     const bool atlas = !cb->atlas_arr.empty();
@@ -950,17 +1030,14 @@ int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
         cb->vhi[i] = dec(bs[2 * (size_t)nbr + 2 * i + 1]);
         if (cb->storage != VR_F32) cb->tmpl[i].exp2 = (int)bs[(size_t)nbr + i];
     }
-    if (atlas && !surf) return stage_atlases(cb, s);
+    if (atlas && !surf) return stage_atlases(c, cb, s);
     return VR_OK;
 }
 
-void free_cube(Cube *cb) {
-    free_atlases(cb);
-    if (cb->d_wstore) cudaFree(cb->d_wstore);
-    if (cb->d_src) cudaFree(cb->d_src);
-    if (cb->d_pool) cudaFree(cb->d_pool);
-    if (cb->d_tmpl) cudaFree(cb->d_tmpl);
-    if (cb->d_bs) cudaFree(cb->d_bs);
+// (What reads the cube has been drained by the caller.)
+void free_cube(vr_ctx *c, Cube *cb) {
+    free_atlases(c, cb);
+    for (void *p : {(void *)cb->d_wstore, (void *)cb->d_src, cb->d_pool, (void *)cb->d_tmpl, (void *)cb->d_bs}) mem_free(c, p);
     delete cb;
 }
 
@@ -1249,6 +1326,16 @@ static int vr_create_body(vr_ctx **out, int device, size_t cache_bytes) {
         if ((e = cudaStreamCreateWithFlags(&c->load_stream, cudaStreamNonBlocking)) != cudaSuccess) { rc = cuda_fail(e, "stream"); break; }
         if ((e = cudaEventCreateWithFlags(&c->upload_done, cudaEventDisableTiming)) != cudaSuccess) { rc = cuda_fail(e, "event"); break; }
         if ((e = cudaEventCreateWithFlags(&c->frame_done, cudaEventDisableTiming)) != cudaSuccess) { rc = cuda_fail(e, "event"); break; }
+        int pools = 0;
+        if (cudaDeviceGetAttribute(&pools, cudaDevAttrMemoryPoolsSupported, device) == cudaSuccess && pools) {
+            cudaMemPoolProps mp{};
+            mp.allocType = cudaMemAllocationTypePinned;
+            mp.location.type = cudaMemLocationTypeDevice;
+            mp.location.id = device;
+            uint64_t keep = kIdleBytes;
+            if ((e = cudaMemPoolCreate(&c->mem, &mp)) != cudaSuccess) { rc = cuda_fail(e, "memory pool"); break; }
+            if ((e = cudaMemPoolSetAttribute(c->mem, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) { rc = cuda_fail(e, "memory pool"); break; }
+        }
         if ((e = cudaMalloc(&c->d_ctr, sizeof(Counters))) != cudaSuccess) { rc = cuda_fail(e, "counters"); break; }
         if ((e = cudaMemset(c->d_ctr, 0, sizeof(Counters))) != cudaSuccess) { rc = cuda_fail(e, "counters"); break; }
         if ((e = cudaMalloc(&c->d_mm, sizeof(unsigned int) * 2)) != cudaSuccess) { rc = cuda_fail(e, "minmax"); break; }
@@ -1270,7 +1357,9 @@ static void vr_destroy_body(vr_ctx *c) {
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     cache_destroy(c);
-    for (auto &kv : c->cubes) free_cube(kv.second);
+    for (auto &kv : c->cubes) free_cube(c, kv.second);
+    idle_release(c);
+    if (c->mem) cudaMemPoolDestroy(c->mem);
     if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->d_stage.p) cudaFree(c->d_stage.p);
     if (c->d_frags.p) cudaFree(c->d_frags.p);
@@ -1319,21 +1408,21 @@ static int vr_load_cube_body(vr_ctx *c, const void *voxels, int dtype, int64_t n
     if (!cb) return VR_ERR_OOM;
     for (int a = 0; a < 3; ++a) cb->n[a] = ext[a];
     const size_t bytes = sizeof(float) * (size_t)ext[0] * ext[1] * ext[2];
-    cudaError_t e = cudaMalloc(&cb->d_src, bytes);
-    if (e != cudaSuccess) { delete cb; return cuda_fail(e, "cudaMalloc(cube)"); }
+    cudaError_t e = mem_alloc(c, reinterpret_cast<void **>(&cb->d_src), bytes);
+    if (e != cudaSuccess) { delete cb; return cuda_fail(e, "allocation of the cube"); }
     cudaMemcpyKind kind = where == VR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     // a device source is read after all work already queued on the device (the caller's
     // writes to it may still be in flight on any of its streams: the copy runs on the
     // library's own non-blocking stream, which orders after none of them)
     if (where == VR_DEVICE && (e = cudaDeviceSynchronize()) != cudaSuccess) {
-        free_cube(cb);
+        free_cube(c, cb);
         return cuda_fail(e, "cudaDeviceSynchronize (device cube source)");
     }
     if (where == VR_DEVICE && !sub_origin && own_device_memory(voxels, c->device)) {
         // the whole array: one linear pass (the 3D copy below moves device memory at a quarter of HBM's rate)
         e = launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)nx * ny * nz, c->load_stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->load_stream);
-        if (e != cudaSuccess) { free_cube(cb); return cuda_fail(e, "copy of the cube"); }
+        if (e != cudaSuccess) { free_cube(c, cb); return cuda_fail(e, "copy of the cube"); }
         cb->id = *cube_id = c->next_id++;
         c->cubes[cb->id] = cb;
         return VR_OK;
@@ -1347,7 +1436,7 @@ static int vr_load_cube_body(vr_ctx *c, const void *voxels, int dtype, int64_t n
     p.kind = kind;
     e = cudaMemcpy3DAsync(&p, c->load_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->load_stream);
-    if (e != cudaSuccess) { free_cube(cb); return cuda_fail(e, "cudaMemcpy3D(cube)"); }
+    if (e != cudaSuccess) { free_cube(c, cb); return cuda_fail(e, "cudaMemcpy3D(cube)"); }
     int id = c->next_id++;
     cb->id = id;
     c->cubes[id] = cb;
@@ -1420,9 +1509,9 @@ static int vr_free_cube_body(vr_ctx *c, int cube_id) {
     Cube *cb = find_cube(c, cube_id);
     if (!cb) return VR_ERR_NOT_FOUND;
     set_dev(c);
-    if (c->frame_pending) cudaEventSynchronize(c->frame_done);
+    cudaDeviceSynchronize();             // frames in flight may still read the cube
     cache_forget_cube(c, cube_id);
-    free_cube(cb);
+    free_cube(c, cb);
     c->cubes.erase(cube_id);
     return VR_OK;
 }
@@ -1523,9 +1612,12 @@ static int vr_set_bricking_body(vr_ctx *c, int cube_id, int bx, int by, int bz, 
         }
     }
     for (int64_t bi = 0; bi < nbr; ++bi) t[bi].data_off = loff[3 * bi];
-    free_atlases(cb);
-    if (cb->d_pool) { cudaFree(cb->d_pool); cb->d_pool = nullptr; }
-    if (cb->d_tmpl) { cudaFree(cb->d_tmpl); cb->d_tmpl = nullptr; }
+    free_atlases(c, cb);
+    CK(cudaDeviceSynchronize());       // frames in flight may still read the bricks
+    mem_free(c, cb->d_pool);
+    mem_free(c, cb->d_tmpl);
+    cb->d_pool = nullptr;
+    cb->d_tmpl = nullptr;
     cb->bricked = false;
     if (cb->streamed) {                // bricks are produced on demand into the cache
         cache_forget_cube(c, cube_id);    // (a cache with smaller slots is re-cut by the next frame)
@@ -1538,11 +1630,12 @@ static int vr_set_bricking_body(vr_ctx *c, int cube_id, int bx, int by, int bz, 
         cb->bricked = true;
         return (cb->layouts & 8) ? cache_prepare_atlases(c, cb) : VR_OK;
     }
-    CK(cudaMalloc(&cb->d_pool, std::max<size_t>(off * esz, 16)));
+    CK(mem_alloc(c, &cb->d_pool, std::max<size_t>(off * esz, 16)));
     cb->pool_bytes = off * esz;
-    CK(cudaMalloc(&cb->d_tmpl, (sizeof(DrawBrick) + sizeof(AtlasCell)) * nbr));   // records, then atlas cells
-    if (cb->d_bs) { cudaFree(cb->d_bs); cb->d_bs = nullptr; }
-    CK(cudaMalloc(&cb->d_bs, sizeof(unsigned int) * 4 * nbr));
+    CK(mem_alloc(c, reinterpret_cast<void **>(&cb->d_tmpl), (sizeof(DrawBrick) + sizeof(AtlasCell)) * nbr));   // records, then atlas cells
+    mem_free(c, cb->d_bs);
+    cb->d_bs = nullptr;
+    CK(mem_alloc(c, reinterpret_cast<void **>(&cb->d_bs), sizeof(unsigned int) * 4 * nbr));
     cb->tmpl = std::move(t);
     cb->loff = std::move(loff);
     cb->loff_pad = std::move(loff_pad);
@@ -1574,22 +1667,22 @@ static int vr_compress_cube_body(vr_ctx *c, int cube_id) {
     for (int a = 0; a < 3; ++a) nb *= (size_t)((cb->n[a] + 7) / 8);
     const size_t bytes = nb * (size_t)kWaveletRecordBytes;
     unsigned char *store = nullptr;
-    CK(cudaMalloc(&store, bytes));
+    CK(mem_alloc(c, reinterpret_cast<void **>(&store), bytes));
     cudaError_t e = launch_wavelet_encode(cb->d_src, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], store,
                                           c->load_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->load_stream);
     if (e != cudaSuccess) {
-        cudaFree(store);
+        mem_free(c, store);
         return cuda_fail(e, "wavelet encode");
     }
     // the FP32 voxels, the brick pool and the atlases go; frames in flight may still read them
     CK(cudaDeviceSynchronize());
-    free_atlases(cb);
-    cudaFree(cb->d_src);
+    free_atlases(c, cb);
+    for (void *p : {(void *)cb->d_src, cb->d_pool, (void *)cb->d_tmpl, (void *)cb->d_bs}) mem_free(c, p);
     cb->d_src = nullptr;
-    if (cb->d_pool) { cudaFree(cb->d_pool); cb->d_pool = nullptr; }
-    if (cb->d_tmpl) { cudaFree(cb->d_tmpl); cb->d_tmpl = nullptr; }
-    if (cb->d_bs) { cudaFree(cb->d_bs); cb->d_bs = nullptr; }
+    cb->d_pool = nullptr;
+    cb->d_tmpl = nullptr;
+    cb->d_bs = nullptr;
     cb->pool_bytes = 0;
     cb->loff.clear();
     cb->loff_pad.clear();

@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 
 #include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <new>
 #include <stdexcept>
 #include <vector>
@@ -95,6 +97,8 @@ struct Cube {
     std::vector<unsigned long long> atlas_tex, atlas_surf;
     std::vector<AtlasCell> atlas_cells;
     std::vector<int> atlas_of;         // brick -> array
+    std::vector<std::pair<int, int>> atlas_dims;   // of each array
+    int atlas_kind = 0;                // their texels (IdleArray::kind)
     bool atlas_fit = true;             // (layout bit 3) the bricks' slices fit an array with the copies
                                        // the columns carry; false: frames read the linear copy
     bool atlas_pair = false;           // the atlases are pair atlases (layout bit 5, 16-bit bricks)
@@ -143,11 +147,37 @@ struct WorkList {
     size_t off_lut = 0, off_db = 0, off_items = 0, off_ts = 0, off_tl = 0, off_mask = 0, bytes = 0;
 };
 
+// An atlas array that no cube uses any more, with its texture and surface: 0 f32, 1 f16, 2 bf16, 3 pairs.
+struct IdleArray {
+    cudaArray_t arr = nullptr;
+    unsigned long long tex = 0, surf = 0;
+    int w = 0, h = 0, kind = 0;
+    size_t bytes = 0;
+};
+// A serving frame slot's stream, events and scratch, kept for the next serving loop.
+struct IdleSlot {
+    cudaStream_t s = nullptr;
+    cudaEvent_t done = nullptr, upload_done = nullptr, frame_done = nullptr;
+    char *h_stage = nullptr;
+    size_t h_cap = 0;
+    DevBuf<char> d_stage, d_frags;
+    DevBuf<float> d_out;
+    size_t bytes() const { return h_cap + d_stage.cap + d_frags.cap + sizeof(float) * d_out.cap; }
+};
+
 }  // namespace vrh
 
 struct vr_ctx {
     int device = 0;
     cudaStream_t load_stream = nullptr;
+    // What freed cubes and closed serving loops leave for the next ones, all bounded and released
+    // by vr_destroy: the cubes' memory (a stream-ordered pool on load_stream that keeps at most
+    // kIdleBytes unused), atlas arrays (kIdleArrayBytes) and frame slots (kIdleSlots, kIdleBytes)
+    cudaMemPool_t mem = nullptr;
+    std::vector<vrh::IdleArray> idle_arrays;
+    std::vector<vrh::IdleSlot> idle_slots;
+    std::mutex idle_mu;                  // guards the two lists
+    vr_ctx *parent = nullptr;            // of a serving slot's context
     std::map<int, vrh::Cube *> cubes;
     int next_id = 1;
     // transfer function (copied into every frame's upload)
@@ -242,6 +272,24 @@ void layout_strides(const int dim[3], int layout, int str[3]);
 // The brick grid a global-termination frame walks (the render window clips the rays).
 MarchGrid march_grid(const vr_ctx *c, const Cube *cb);
 
+constexpr size_t kIdleBytes = size_t(2) << 30, kIdleArrayBytes = size_t(1) << 30;
+constexpr size_t kIdleSlots = 16;
+// Memory of a cube.  Allocated and freed on load_stream: the caller of mem_free has drained whatever
+// reads it (cudaFree's implicit wait is not there), and what mem_alloc returned is written first
+// by work on load_stream or after waiting for it.
+cudaError_t mem_alloc(vr_ctx *c, void **p, size_t bytes);
+void mem_free(vr_ctx *c, void *p);
+void idle_release(vr_ctx *c);                     // everything idle back to the device
+// f(), once more after everything idle is given back if the device was out of memory
+template <typename F>
+cudaError_t alloc_retry(vr_ctx *c, F f) {
+    cudaError_t e = f();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    idle_release(c);
+    return f();
+}
+void idle_slot_free(IdleSlot &s);
 int set_dev(vr_ctx *c);
 Cube *find_cube(vr_ctx *c, int id);
 int ensure_host(vr_ctx *c, size_t bytes);
@@ -277,7 +325,7 @@ int check_ready(vr_ctx *c, Cube *cb);
 bool window_clip(const vr_ctx *c, const Cube *cb, const DrawBrick &b, float lo[3], float hi[3]);
 int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s);
 int render_frame_impl(vr_ctx *c, Cube *cb, float *out, int out_where, cudaStream_t s);
-void free_cube(Cube *cb);
+void free_cube(vr_ctx *c, Cube *cb);
 
 template <typename T>
 int ensure(DevBuf<T> &b, size_t n, vr_ctx *c) {
@@ -287,7 +335,7 @@ int ensure(DevBuf<T> &b, size_t n, vr_ctx *c) {
     if (b.p) CK(cudaFree(b.p));
     b.p = nullptr;
     b.cap = 0;
-    CK(cudaMalloc(&b.p, (want > 0 ? want : 1) * sizeof(T)));
+    CK(alloc_retry(c, [&] { return cudaMalloc(&b.p, (want > 0 ? want : 1) * sizeof(T)); }));
     b.cap = want;
     return VR_OK;
 }

@@ -429,31 +429,45 @@ static int cache_size(vr_ctx *c, size_t slot_bytes) {
         return fail(VR_ERR_OOM, "cache_bytes of vr_create is smaller than one brick");
     const size_t sb = align_up(slot_bytes, 256);
     const int nslots = (int)(c->cache_bytes / sb);
-    std::vector<Staging> stage(std::max(4, 2 * k->workers->size()));
     std::vector<Slot> slots(nslots);
     char *base = nullptr;
     auto undo = [&](int status, const std::string &what) {
-        for (auto &s : stage) {
-            if (s.host) cudaFreeHost(s.host);
-            if (s.done) cudaEventDestroy(s.done);
-        }
         for (auto &s : slots)
             if (s.last_use) cudaEventDestroy(s.last_use);
         if (base) cudaFree(base);
         return fail(status, what);
     };
-    for (auto &s : stage) {
-        if (c->fault_kind == 2) return undo(VR_ERR_OOM, "pinned staging allocation failed (injected)");
-        if (cudaMallocHost(&s.host, sb) != cudaSuccess) return undo(VR_ERR_OOM, "pinned staging allocation failed");
-        if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) return undo(VR_ERR_CUDA, "event");
-    }
     for (auto &s : slots)
         if (cudaEventCreateWithFlags(&s.last_use, cudaEventDisableTiming) != cudaSuccess) return undo(VR_ERR_CUDA, "event");
-    if (cudaMalloc(&base, (size_t)nslots * sb) != cudaSuccess) return undo(VR_ERR_OOM, "brick cache allocation failed");
+    if (alloc_retry(c, [&] { return cudaMalloc(&base, (size_t)nslots * sb); }) != cudaSuccess) return undo(VR_ERR_OOM, "brick cache allocation failed");
     k->d_base = base;
     k->slot_bytes = sb;
     k->nslots = nslots;
     k->slots = std::move(slots);
+    return VR_OK;
+}
+
+// Pinned staging for bricks produced on the host, made when the first one is needed (a compressed
+// cube's bricks never are: page-locking 2.2 GB took 80 ms of its first frame).
+static int cache_stage(vr_ctx *c) {
+    BrickCache *k = c->cache;
+    if (!k->stage.empty()) return VR_OK;
+    std::vector<Staging> stage(std::max(4, 2 * k->workers->size()));
+    auto undo = [&](int status, const char *what) {
+        for (auto &s : stage) {
+            if (s.host) cudaFreeHost(s.host);
+            if (s.done) cudaEventDestroy(s.done);
+        }
+        return fail(status, what);
+    };
+    for (auto &s : stage) {
+        if (c->fault_kind == 2) return undo(VR_ERR_OOM, "pinned staging allocation failed (injected)");
+        if (cudaMallocHost(&s.host, k->slot_bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return undo(VR_ERR_OOM, "pinned staging allocation failed");
+        }
+        if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) return undo(VR_ERR_CUDA, "event");
+    }
     k->stage = std::move(stage);
     return VR_OK;
 }
@@ -600,8 +614,9 @@ static int slot_atlas_alloc(vr_ctx *c, Cube *cb, int si, const AtlasGeom &g) {
             : cb->storage == VR_F16 ? cudaCreateChannelDescHalf()
                                     : cudaCreateChannelDesc(16, 0, 0, 0, cudaChannelFormatKindUnsigned);
         // writable through a surface when the device allows it with gathers, else filled by copies
-        bool surf_ok = cudaMallocArray(&s.arr, &cd, (size_t)g.w, (size_t)g.h,
-                                       cudaArrayTextureGather | cudaArraySurfaceLoadStore) == cudaSuccess;
+        bool surf_ok = alloc_retry(c, [&] {
+            return cudaMallocArray(&s.arr, &cd, (size_t)g.w, (size_t)g.h, cudaArrayTextureGather | cudaArraySurfaceLoadStore);
+        }) == cudaSuccess;
         if (!surf_ok) {
             s.arr = nullptr;
             cudaGetLastError();
@@ -650,7 +665,7 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
         if (k->pack_tmp) cudaFree(k->pack_tmp);
         k->pack_tmp = nullptr;
         k->pack_bytes = 0;
-        CK(cudaMalloc(&k->pack_tmp, need));
+        CK(alloc_retry(c, [&] { return cudaMalloc(&k->pack_tmp, need); }));
         k->pack_bytes = need;
     }
     const int cols = (b.dim[2] + g.rows - 1) / g.rows;
@@ -785,6 +800,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
         return rc;
     }
     // produce in parallel, at most one staging buffer per brick in flight
+    rc = cache_stage(c);
     const size_t nstage = k->stage.size();
     std::vector<std::shared_ptr<BrickJob>> jobs(misses.size());
     std::vector<size_t> st_of(misses.size());

@@ -55,6 +55,7 @@ struct FrameSlot {
 vr_ctx *slot_context(vr_ctx *parent) {
     vr_ctx *c = new vr_ctx();
     c->device = parent->device;
+    c->parent = parent;
     c->cubes = parent->cubes;
     c->next_id = -1;
     c->d_ctr = parent->d_ctr;
@@ -66,16 +67,57 @@ vr_ctx *slot_context(vr_ctx *parent) {
     return c;
 }
 
-void slot_release(vr_ctx *c) {
-    if (!c) return;
-    if (c->frame_pending) cudaEventSynchronize(c->frame_done);
-    if (c->h_stage) cudaFreeHost(c->h_stage);
-    if (c->d_stage.p) cudaFree(c->d_stage.p);
-    if (c->d_frags.p) cudaFree(c->d_frags.p);
-    if (c->d_out.p) cudaFree(c->d_out.p);
-    if (c->upload_done) cudaEventDestroy(c->upload_done);
-    if (c->frame_done) cudaEventDestroy(c->frame_done);
-    delete c;                          // cubes, counters and cache belong to the parent
+// Gives a slot a stream, events and scratch: those an earlier loop of this context left (making and
+// freeing them cost a loop of 12 small frames 1.7 ms), or new ones.
+bool slot_open(vr_ctx *parent, FrameSlot &sl) {
+    sl.c = slot_context(parent);
+    IdleSlot is;
+    std::lock_guard<std::mutex> l(parent->idle_mu);
+    if (!parent->idle_slots.empty()) {
+        is = parent->idle_slots.back();
+        parent->idle_slots.pop_back();
+    }
+    sl.s = is.s;
+    sl.done = is.done;
+    sl.c->upload_done = is.upload_done;
+    sl.c->frame_done = is.frame_done;
+    sl.c->h_stage = is.h_stage;
+    sl.c->h_cap = is.h_cap;
+    sl.c->d_stage = is.d_stage;
+    sl.c->d_frags = is.d_frags;
+    sl.c->d_out = is.d_out;
+    if (sl.s) return true;
+    return cudaStreamCreateWithFlags(&sl.s, cudaStreamNonBlocking) == cudaSuccess &&
+           cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&sl.c->upload_done, cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&sl.c->frame_done, cudaEventDisableTiming) == cudaSuccess;
+}
+
+// The slot's work is done (its stream was waited for): what it holds is left to the context while that
+// is little, else released.
+void slot_close(vr_ctx *parent, FrameSlot &sl) {
+    IdleSlot is;
+    is.s = sl.s;
+    is.done = sl.done;
+    if (sl.c) {
+        is.upload_done = sl.c->upload_done;
+        is.frame_done = sl.c->frame_done;
+        is.h_stage = sl.c->h_stage;
+        is.h_cap = sl.c->h_cap;
+        is.d_stage = sl.c->d_stage;
+        is.d_frags = sl.c->d_frags;
+        is.d_out = sl.c->d_out;
+        delete sl.c;                    // cubes, counters and cache belong to the parent
+        sl.c = nullptr;
+    }
+    sl.s = nullptr;
+    sl.done = nullptr;
+    std::lock_guard<std::mutex> l(parent->idle_mu);
+    size_t kept = is.bytes();
+    for (auto &o : parent->idle_slots) kept += o.bytes();
+    const bool whole = is.s && is.done && is.upload_done && is.frame_done;
+    if (whole && kept <= kIdleBytes && parent->idle_slots.size() < kIdleSlots) parent->idle_slots.push_back(is);
+    else idle_slot_free(is);
 }
 
 double ms_since(std::chrono::steady_clock::time_point t0) {
@@ -117,14 +159,8 @@ struct ServeCore {
         c = parent;
         t0 = std::chrono::steady_clock::now();
         slots.resize(max_inflight);
-        for (auto &sl : slots) {
-            sl.c = slot_context(c);
-            if (cudaStreamCreateWithFlags(&sl.s, cudaStreamNonBlocking) != cudaSuccess ||
-                cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) != cudaSuccess ||
-                cudaEventCreateWithFlags(&sl.c->upload_done, cudaEventDisableTiming) != cudaSuccess ||
-                cudaEventCreateWithFlags(&sl.c->frame_done, cudaEventDisableTiming) != cudaSuccess)
-                return fail(VR_ERR_CUDA, "could not create the frame slots' streams and events");
-        }
+        for (auto &sl : slots)
+            if (!slot_open(c, sl)) return fail(VR_ERR_CUDA, "could not create the frame slots' streams and events");
         return VR_OK;
     }
 
@@ -139,9 +175,7 @@ struct ServeCore {
                 c->bricks_drawn += sl.c->bricks_drawn;
                 if (sl.cube && !sl.held.empty()) cache_hold(c, sl.cube, sl.held, -1, true);
             }
-            slot_release(sl.c);
-            if (sl.done) cudaEventDestroy(sl.done);
-            if (sl.s) cudaStreamDestroy(sl.s);
+            slot_close(c, sl);
         }
         for (auto &h : holds) cache_hold(c, h.cube, h.bricks, h.delta, true);
         holds.clear();
