@@ -20,26 +20,29 @@
 #include "vr_internal.cuh"
 
 // Tuning knobs of the ray-cast kernels (build-time): unroll factor of the linear sample loops, samples
-// fetched ahead (slice atlases, pair atlases, linear rows), the blocks per SM the register
-// allocation must allow for DVR frames read through atlases, through linear rows and for MIP
-// frames (0: no constraint), and the same for the one-pass (global termination) kernel.
+// fetched ahead (slice atlases, pair atlases, linear rows), the CTAs of 128 threads per SM the
+// register allocation must allow for DVR frames read through these and for MIP frames (0: no
+// constraint), and the same for the one-pass (global termination, 256 threads) kernel.
 #ifndef VR_SAMPLE_UNROLL
 #define VR_SAMPLE_UNROLL 1
 #endif
-#ifndef VR_DVR_MIN_BLOCKS
-#define VR_DVR_MIN_BLOCKS 4
-#endif
 #ifndef VR_AHEAD
-#define VR_AHEAD 2
+#define VR_AHEAD 3
 #endif
 #ifndef VR_AHEAD_PAIR
-#define VR_AHEAD_PAIR 3
+#define VR_AHEAD_PAIR 4
 #endif
 #ifndef VR_AHEAD_ROWS
 #define VR_AHEAD_ROWS 2
 #endif
+#ifndef VR_ATLAS_MIN_BLOCKS
+#define VR_ATLAS_MIN_BLOCKS 6
+#endif
+#ifndef VR_PAIR_MIN_BLOCKS
+#define VR_PAIR_MIN_BLOCKS 5
+#endif
 #ifndef VR_ROWS_MIN_BLOCKS
-#define VR_ROWS_MIN_BLOCKS 4
+#define VR_ROWS_MIN_BLOCKS 8
 #endif
 #ifndef VR_MIP_MIN_BLOCKS
 #define VR_MIP_MIN_BLOCKS 0
@@ -502,7 +505,7 @@ __device__ __forceinline__ void over(const DvrSample &s, float &c0, float &c1, f
 }
 
 // ----------------------------------------------------------------------------------------------
-// ray cast: one CTA = 32x8 (or 8x32) pixels of one brick's rendering rectangle; warp = 32 pixels
+// ray cast: a work item = 32x8 (or 8x32) pixels of one brick's rendering rectangle, one or two CTAs; warp = 32 pixels
 // along the image axis that the brick layout follows
 // ----------------------------------------------------------------------------------------------
 // One brick segment of a ray: n >= 1 lattice samples from the anchor q, composited front to back
@@ -518,21 +521,22 @@ __device__ __forceinline__ void over(const DvrSample &s, float &c0, float &c1, f
 // whole-number floats, the slices placed so that no sample tests for a column's end, z
 // interpolated first (packed), the two exits one branch.  No index is clamped: the host takes this
 // path only for cameras near enough that rounding cannot move a sample half a voxel (kAtlasReach).
-// The stencils of AHEAD samples are fetched before the first of them is composited: two with slice
-// atlases and three with pair atlases at 4 CTAs of 64 registers, which beats more warps with one
-// sample each (fewer rays share the texture cache) and more samples or fewer warps.
-// 1024^2 frames at step 1, ms: integer cells -> one sample at a time -> ahead.  1720x1720x1024 FP32
-// 3.54 -> 3.41 -> 3.26, FP16 2.95 -> 2.82 -> 2.74, FP16 pair atlas 2.94 -> 2.92 -> 2.56;
-// 768x768x512 FP32 1.36 -> 1.31 -> 1.29; 256^3 at 512^2, step 0.5: 0.35 -> 0.34 -> 0.31;
-// 2048x2048x256 BF16 pair atlas, step 0.5: 1.07 -> 1.06 -> 0.89.  Global termination (one sample at a
-// time: two spill) 768x768x512 0.64 -> 0.59.  Two ahead at 5 CTAs: 3.53 (FP32 1720x1720x1024), three
-// at 4: 3.44, four at 2: 3.71; pair atlas two at 4: 2.88, four at 4: 2.96, three at 5: 3.07.
+// The stencils of AHEAD samples are fetched before the first of them is looked up, and all are looked
+// up before the first is composited, so that a ray waits once for several samples (short
+// launches are bound by that chain: 64-sample segments, 128^3 at 256^2, 73 -> 62 us): three with slice
+// atlases at 6 CTAs of 128 threads (72 registers), four with pair atlases at 5 (72).
+// 1024^2 frames at step 1, ms: integer cells -> one sample at a time -> two (pair atlas three) ahead,
+// composited one by one, 4 CTAs of 256 threads -> now.  1720x1720x1024 FP32 3.54 -> 3.41 -> 3.26 ->
+// 3.18, FP16 2.95 -> 2.82 -> 2.74 -> 2.73, FP16 pair atlas 2.94 -> 2.92 -> 2.56 -> 2.43;
+// 768x768x512 FP32 1.36 -> 1.31 -> 1.29 -> 1.24; 256^3 at 512^2, step 0.5: 0.35 -> 0.34 -> 0.31 -> 0.30;
+// 2048x2048x256 BF16 pair atlas, step 0.5: 1.07 -> 1.06 -> 0.89 -> 0.82.  FP32 1720x1720x1024 and
+// 768x768x512 with two ahead at 8 CTAs 3.25 and 1.26, three at 7 3.40 and 1.31, four at 5 3.24 and
+// 1.28; pair atlas (FP16 1720x1720x1024) three at 6 2.51, three at 8 2.47, four at 7 2.43 (BF16 0.83).
+// Global termination (one sample at a time: two spill) 768x768x512 0.64 -> 0.59.
 template <int S, bool MASK>
 __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const CellF &c, float scale, const FrameConsts &fc,
-                                      const float4 *s_lut, const unsigned char *s_mask, int org_z, float vcode, float &c0,
-                                      float &c1, float &c2, float &T) {
+                                      const float4 *s_lut, const unsigned char *s_mask, int org_z, float vcode, DvrSample &sm) {
     const Cell cl{0, 0, 0, c.fxy.x, c.fxy.y, c.fz};
-    DvrSample sm;
     if (MASK) {
         float v[8];
         gathers_to_stencil(g0, g1, v);
@@ -542,7 +546,6 @@ __device__ __forceinline__ void shade(const float4 &g0, const float4 &g1, const 
     } else {
         interp_tf(lerp_z(g0, g1, c.fz), cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
     }
-    over(sm, c0, c1, c2, T);
 }
 
 template <int S, int F, bool MASK, int AHEAD>
@@ -565,9 +568,13 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
                 cl[u] = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
                 gather_stencil<S, F>(atl, cl[u].ixy, cl[u].iz, g0[u], g1[u]);
             }
+            DvrSample sm[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u)
+                shade<S, MASK>(g0[u], g1[u], cl[u], scale, fc, s_lut, s_mask, org_z, vcode, sm[u]);
 #pragma unroll
             for (int u = 0; u < AHEAD; ++u) {
-                shade<S, MASK>(g0[u], g1[u], cl[u], scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+                over(sm[u], c0, c1, c2, T);
                 jf = __fadd_rn(jf, 1.0f);
                 if (T <= fc.thr || !(jf < nf)) return (int)jf;
             }
@@ -578,7 +585,9 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
             const CellF cl = cell_f(__ffma2_rn(pair2(tj, tj), dd, q), __fmaf_rn(tj, d[2], qz));
             float4 g0, g1;
             gather_stencil<S, F>(atl, cl.ixy, cl.iz, g0, g1);
-            shade<S, MASK>(g0, g1, cl, scale, fc, s_lut, s_mask, org_z, vcode, c0, c1, c2, T);
+            DvrSample sm;
+            shade<S, MASK>(g0, g1, cl, scale, fc, s_lut, s_mask, org_z, vcode, sm);
+            over(sm, c0, c1, c2, T);
             jf = __fadd_rn(jf, 1.0f);
         } while (!(T <= fc.thr) && jf < nf);
         return (int)jf;
@@ -590,7 +599,7 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
 // indices come straight from the bits of the rounded-down positions, and the rows' second
 // neighbours are constant offsets.  768x768x512, 1024^2 orbit, aligned copies kept: 1.66 -> 1.48 ms; with
 // every third channel masked (plane bits in shared memory) 333x257x190 frames of 641x479 from the
-// default layout take 336 -> 299 us.
+// default layout take 336 -> 299 us.  CTAs of 128 threads and lookups before compositing: 1.53 -> 1.50 ms.
 template <int S, int AX, bool MASK, int AHEAD>
 __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &st, float scale, float qx, float qy, float qz,
                                                 const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
@@ -621,6 +630,7 @@ __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &
                                 __float_as_uint(tz) * (AX == 2 ? 1u : (unsigned)st.z) - bias;
             fetch8_rows<S, AX>(src, (int)i0, st, v[u]);
         }
+        DvrSample sm[AHEAD];
 #pragma unroll
         for (int u = 0; u < AHEAD; ++u) {
             if (MASK) {
@@ -628,9 +638,11 @@ __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &
                 else mask_channels(v[u], iz[u], org_z, fc.nz, fc.chmask, vcode);
             }
             const Cell cl{0, 0, 0, fx[u], fy[u], fz[u]};
-            DvrSample sm;
-            interp_tf(v[u], cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm);
-            over(sm, c0, c1, c2, T);
+            interp_tf(v[u], cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            over(sm[u], c0, c1, c2, T);
             jf = __fadd_rn(jf, 1.0f);
             if (T <= fc.thr || !(jf < nf)) return (int)jf;
         }
@@ -700,6 +712,14 @@ __device__ __forceinline__ void thread_pixel(int lanes, const TileItem &it, int 
     }
 }
 
+// Threads of a ray-cast CTA.  A CTA's registers and table are held until its last ray ends, so half
+// a work item (4 warps) leaves fewer of them idle than a whole one: MIP 2 - 3 % faster, atlases
+// up to 14 %.  The stencil cache wants the whole item: its rows share lines in L1 (2.24 ms, halves 2.35).
+template <int MODE, int F>
+constexpr int rc_threads() {
+    return MODE == 1 || gathers(F) || straight(F) ? 128 : 256;
+}
+
 // The 32 rays of one warp: strip `strip` (0..7) of work item `it`; writes their fragments and
 // adds the warp's samples to the counters.
 template <int S, int MODE, int F, bool MASK>
@@ -744,6 +764,11 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
             // the pixel's place is formed again here, so that the sample loop's registers hold only its own state
             unsigned tid;
             asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+            if constexpr (rc_threads<MODE, F>() < 256) {
+                unsigned cta;
+                asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+                tid += cta * rc_threads<MODE, F>() & 255u;
+            }
             int wx, wy;
             thread_pixel(fc.lanes_y, it, (int)(tid >> 5), (int)(tid & 31), wx, wy);
             static_cast<float4 *>(frags)[b.frag_off + (long long)wy * b.rect[2] + wx] = make_float4(c0, c1, c2, T);
@@ -805,23 +830,23 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
     }
 }
 
-// Blocks per SM the registers of k_raycast<., MODE, F, .> must allow (1: no constraint beyond
-// one block): the kernel's speed follows its resident warps, and 40 registers (6 CTAs) hold the
-// atlas DVR loop without spills.
+// CTAs per SM the registers of k_raycast<., MODE, F, .> must allow (1: no constraint beyond one):
+// the fewest that the samples fetched ahead fit without spills.
 template <int MODE, int F>
 constexpr int rc_min_blocks() {
-    return MODE == 0 ? (straight(F) ? VR_ROWS_MIN_BLOCKS : gathers(F) && VR_DVR_MIN_BLOCKS > 0 ? VR_DVR_MIN_BLOCKS : 1)
-                     : (VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1);
+    if (MODE != 0) return VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1;
+    return F == 2 ? VR_ATLAS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : straight(F) ? VR_ROWS_MIN_BLOCKS : 1;
 }
 
 template <int S, int MODE, int F, bool MASK>
-__global__ void __launch_bounds__(256, rc_min_blocks<MODE, F>())
+__global__ void __launch_bounds__(rc_threads<MODE, F>(), rc_min_blocks<MODE, F>())
 k_raycast(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const void *__restrict__ pool, void *__restrict__ frags,
           Counters *__restrict__ ctr) {
     extern __shared__ float4 s_lut[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const TileItem it = items[blockIdx.x];
+    constexpr int per = 256 / rc_threads<MODE, F>();      // CTAs of a work item
+    const int warp = (blockIdx.x % per) * (8 / per) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const TileItem it = items[blockIdx.x / per];
     unsigned char *s_mask = nullptr;
     if (MASK && fc.mask_planes > 0) {
         s_mask = reinterpret_cast<unsigned char *>(s_lut) + (MODE == 0 ? table_bytes(fc.nlut) : 0);
@@ -1798,7 +1823,7 @@ cudaError_t ensure_smem_limit(const void *kernel, int bytes, DeviceAttrs &da) {
 // default 3.75, 50 % 3.98).  Registers are allocated per warp in units of 256, 64 K per SM, at
 // most 64 warps and 32 CTAs.  The kernel's current preference on this device is remembered in
 // `da`.
-cudaError_t set_carveout(const void *kernel, size_t smem_per_cta, DeviceAttrs &da, int warps = 8) {
+cudaError_t set_carveout(const void *kernel, size_t smem_per_cta, DeviceAttrs &da, int warps) {
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
     if (e != cudaSuccess) return e;
@@ -1823,10 +1848,11 @@ cudaError_t launch_rc(const FrameConsts &fc, const float4 *lut, const DrawBrick 
     cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut) + kMaskPlanes, da);
     if (e != cudaSuccess) return e;
     if (MODE == 0) {
-        e = set_carveout(kern, smem, da);
+        e = set_carveout(kern, smem, da, rc_threads<MODE, F>() / 32);
         if (e != cudaSuccess) return e;
     }
-    k_raycast<S, MODE, F, MASK><<<nitems, 256, smem, s>>>(fc, lut, const_cast<DrawBrick *>(db), items, pool, frags, ctr);
+    constexpr int threads = rc_threads<MODE, F>();
+    k_raycast<S, MODE, F, MASK><<<nitems * (256 / threads), threads, smem, s>>>(fc, lut, const_cast<DrawBrick *>(db), items, pool, frags, ctr);
     return cudaGetLastError();
 }
 
