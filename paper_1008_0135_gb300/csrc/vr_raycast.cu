@@ -22,7 +22,7 @@
 // Tuning knobs of the ray-cast kernels (build-time): unroll factor of the linear sample loops, samples
 // fetched ahead (slice atlases, pair atlases, linear rows), the CTAs of 128 threads per SM the
 // register allocation must allow for DVR frames read through these and for MIP frames (0: no
-// constraint), and the same for the one-pass (global termination, 256 threads) kernel.
+// constraint), and the same for the one-pass (global termination, 256 threads) kernel and the adjoint.
 #ifndef VR_SAMPLE_UNROLL
 #define VR_SAMPLE_UNROLL 1
 #endif
@@ -51,7 +51,7 @@
 #define VR_RAYMARCH_MIN_BLOCKS 5
 #endif
 #ifndef VR_ADJ_MIN_BLOCKS
-#define VR_ADJ_MIN_BLOCKS 3
+#define VR_ADJ_MIN_BLOCKS 5
 #endif
 constexpr int kSampleUnroll = VR_SAMPLE_UNROLL;
 
@@ -1563,14 +1563,16 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 // one atomic per corner it was bound by instruction issue: three variants of the flush, each run
 // by the few lanes that needed it, 17.8 of 32 lanes active and 1.25 G warp instructions a view
 // against 26.4 and 0.54 G.
-// Small launches are bound by the chain of samples: the next sample's gathers are issued ahead (80
-// registers, 3 CTAs an SM; one 256^2 view of 64^3 with the table's gradient alone 128 -> 114 us).
-// 256^3 cube, 8 views at 512^2, step 0.5, forward frames cast again: 18.5 -> 12.5 ms with both
-// gradients, 9.9 -> 9.4 ms with the table's alone.
+// Small launches are bound by the chain of samples: the next sample's gathers are issued ahead (one
+// 256^2 view of 64^3 with the table's gradient alone 128 -> 117 us).  CTAs of half a work item, which
+// hold their registers until their longest ray ends, and no spills (5 an SM, 91 registers): 117 -> 110.
+// 256^3 cube, 8 views at 512^2, step 0.5, forward frames cast again: 18.5 -> 12.0 -> 11.2 ms with both
+// gradients, 9.9 -> 8.9 -> 8.1 ms with the table's alone.
 // ATLAS: the replay reads the stencils from the bricks' slice atlases (the forward's texels)
 // instead of the linear copy; then no index is clamped (make_consts).
+constexpr int kAdjThreads = 128;
 template <bool ATLAS, int VOX>
-__global__ void __launch_bounds__(256, VR_ADJ_MIN_BLOCKS)
+__global__ void __launch_bounds__(kAdjThreads, VR_ADJ_MIN_BLOCKS)
 k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const float *__restrict__ pool,
           const float4 *__restrict__ frags, const float4 *__restrict__ gfrag,
@@ -1578,9 +1580,10 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
     extern __shared__ float4 s_lut[];
     load_table(lut, fc.nlut, s_lut);
     __syncthreads();
-    const TileItem it = items[blockIdx.x];
+    constexpr int per = 256 / kAdjThreads;       // CTAs of a work item
+    const TileItem it = items[blockIdx.x / per];
     const DrawBrick &b = dbs[it.db];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x % per) * (8 / per) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool odd = lane & 1;
     // this CTA's table-gradient partial (rows are zeroed before the launch)
     float4 *g_row = reinterpret_cast<float4 *>(glut_partial) + (long long)(blockIdx.x % rows) * 2 * fc.nlut + (odd ? 1 : 0);
@@ -2018,7 +2021,7 @@ static cudaError_t adjoint(const FrameConsts &fc, const float4 *lut, const DrawB
     static DeviceAttrs da;
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<ATLAS, VOX>), (int)(32 * kMaxLut), da);
     if (e != cudaSuccess) return e;
-    k_adjoint<ATLAS, VOX><<<nitems, 256, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
+    k_adjoint<ATLAS, VOX><<<nitems * (256 / kAdjThreads), kAdjThreads, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
     return cudaGetLastError();
 }
 
