@@ -204,14 +204,15 @@ int vr_wavelet_store(vr_ctx *ctx, int cube_id, void *dst, size_t *bytes);
  * copy whose contiguous axis is most aligned with an image axis and runs its warps along that
  * image axis, so the 32 rays of a warp load neighbouring addresses (each extra layout costs one
  * more copy of the pool in HBM).  Bit 3 also keeps a slice atlas of every brick: a 2D texture
- * array whose tiles are the brick's z-slices, from which a sample's 8 stencil voxels are read
- * by two texture gathers (exact texels; images identical to the linear copies).  When atlases
- * are kept every DVR and MIP frame reads them, and so does the adjoint's replay.  An atlas must
- * fit the device's 2D-gather size (32768 texels a side; 258^3 stored bricks need 8256 x 2322).
+ * array in which the brick's z-slices stand in columns, from which a sample's 8 stencil voxels are
+ * read by two texture gathers (exact texels; images identical to the linear copies).  When atlases
+ * are kept every DVR and MIP frame whose camera is within 2^18 voxels reads them (farther ones the
+ * linear copy), and so does the adjoint's replay.  An atlas must fit the device's 2D-gather size
+ * (32768 texels a side: stored bricks up to about 1000^3).
  * A bricked cube is rebuilt.  Streamed and compressed cubes (bricks made resident in the brick
  * cache) take mask 1 or 9: with 9, each cache slot holding one of the cube's bricks also holds
- * its slice atlas (a 2D array sized for the cube's largest brick, packed from the slot on the
- * cache's stream when the brick becomes resident).  The arrays of as many slots as the cube
+ * its slice atlas (a 2D array sized for the cube's largest brick, packed from the slot or, for
+ * compressed cubes, decoded into it on the cache's stream when the brick becomes resident).  The arrays of as many slots as the cube
  * has bricks (at most all slots: up to as much device memory again as cache_bytes, outside
  * it) are made by this call (and by vr_set_bricking of such a cube), so that frames only pack; the call
  * then sizes the brick cache (VR_ERR_OOM without one, or when an array cannot be had; a frame
