@@ -396,16 +396,20 @@ __device__ __forceinline__ void fetch8(const void *src, int i0, const Strides &t
 // The stencil at element p of a linear copy whose axis AX is contiguous: four rows, two neighbours each
 // (the second at a constant offset: 4 addresses instead of 8).
 template <int S, int AX>
-__device__ __forceinline__ void fetch8_rows(const void *src, int i0, const Strides &t, float v[8]) {
+__device__ __forceinline__ void fetch8_rows(const void *src, int i0, const Strides &t, float v[8], unsigned planes = 3) {
     using T = std::conditional_t<S == 0, float, unsigned short>;
     const T *p = static_cast<const T *>(src) + i0;
     const int s1 = AX == 0 ? t.y : t.x, s2 = AX == 2 ? t.y : t.z;
     constexpr int a = 1 << AX, b1 = AX == 0 ? 2 : 1, b2 = AX == 2 ? 2 : 4;
     const T *q = p + s1, *r = p + s2, *w = r + s1;
-    v[0] = ldv<S>(p, 0);       v[a] = ldv<S>(p, 1);
-    v[b1] = ldv<S>(q, 0);      v[b1 | a] = ldv<S>(q, 1);
-    v[b2] = ldv<S>(r, 0);      v[b2 | a] = ldv<S>(r, 1);
-    v[b2 | b1] = ldv<S>(w, 0); v[b2 | b1 | a] = ldv<S>(w, 1);
+    // (corners of a z-plane not in `planes` keep their values)
+    auto ld = [&](const T *row, int k, int c) {
+        if ((planes >> (c >> 2)) & 1) v[c] = ldv<S>(row, k);
+    };
+    ld(p, 0, 0);       ld(p, 1, a);
+    ld(q, 0, b1);      ld(q, 1, b1 | a);
+    ld(r, 0, b2);      ld(r, 1, b2 | a);
+    ld(w, 0, b2 | b1); ld(w, 1, b2 | b1 | a);
 }
 
 // Disabled spectral channels hold vmin (the bottom of the table range) in place of their data:
@@ -427,6 +431,12 @@ __device__ __forceinline__ void load_mask_planes(const DrawBrick &b, int nz, con
 __device__ __forceinline__ void mask_planes(float v[8], unsigned m, float vcode) {
     if (!(m & 1)) { v[0] = vcode; v[1] = vcode; v[2] = vcode; v[3] = vcode; }
     if (!(m & 2)) { v[4] = vcode; v[5] = vcode; v[6] = vcode; v[7] = vcode; }
+}
+
+// Which of a cell's two z-planes are on: bit 0 the lower, bit 1 the upper one.
+__device__ __forceinline__ unsigned plane_bits(const FrameConsts &fc, const unsigned char *s_mask, int iz, int org_z) {
+    if (s_mask) return s_mask[iz];
+    return (fc.chmask[clampi(org_z + iz, 0, fc.nz - 1)] ? 1u : 0u) | (fc.chmask[clampi(org_z + iz + 1, 0, fc.nz - 1)] ? 2u : 0u);
 }
 
 // A point's cell in whole-number floats: lower corner (x, y packed) and fractions, no clamps --
@@ -536,10 +546,6 @@ __device__ __forceinline__ void over(const DvrSample &s, float &c0, float &c1, f
 // With a channel mask a slice whose channel is off is not gathered at all: its texels hold vcode.
 // (A band of 20 % of the channels on, FP32: 1720x1720x1024 3.37 -> 2.26 ms, 768x768x512 1.33 -> 0.97,
 // with global termination and an opaque table 1.51 -> 1.13; every slice gathered before.)
-__device__ __forceinline__ unsigned plane_bits(const FrameConsts &fc, const unsigned char *s_mask, int iz, int org_z) {
-    if (s_mask) return s_mask[iz];
-    return (fc.chmask[clampi(org_z + iz, 0, fc.nz - 1)] ? 1u : 0u) | (fc.chmask[clampi(org_z + iz + 1, 0, fc.nz - 1)] ? 2u : 0u);
-}
 template <int S, int F, bool MASK>
 __device__ __forceinline__ unsigned gather_masked(const Atlas &atl, const CellF &c, const FrameConsts &fc, const unsigned char *s_mask,
                                                   int org_z, float vcode, float4 &g0, float4 &g1) {
@@ -621,6 +627,8 @@ __device__ __forceinline__ int dvr_segment_atlas(const Atlas &atl, float scale, 
 // neighbours are constant offsets.  768x768x512, 1024^2 orbit, aligned copies kept: 1.66 -> 1.48 ms; with
 // every third channel masked (plane bits in shared memory) 333x257x190 frames of 641x479 from the
 // default layout take 336 -> 299 us.  CTAs of 128 threads and lookups before compositing: 1.53 -> 1.50 ms.
+// Disabled channels are not loaded: the masked 333x257x190 frames 300 -> 227 us, a band of 20 % of the channels
+// of 768x768x512 from the default layout 2.34 -> 1.10 ms (the stencil cache, which loads them, before).
 template <int S, int AX, bool MASK, int AHEAD>
 __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &st, float scale, float qx, float qy, float qz,
                                                 const float d[3], int n, const FrameConsts &fc, const float4 *s_lut,
@@ -649,15 +657,17 @@ __device__ __forceinline__ int dvr_segment_rows(const void *src, const Strides &
             iz[u] = __float_as_int(tz) - kFloorMagicBits;
             const unsigned i0 = __float_as_uint(t.x) * (AX == 0 ? 1u : (unsigned)st.x) + __float_as_uint(t.y) * (AX == 1 ? 1u : (unsigned)st.y) +
                                 __float_as_uint(tz) * (AX == 2 ? 1u : (unsigned)st.z) - bias;
-            fetch8_rows<S, AX>(src, (int)i0, st, v[u]);
+            unsigned planes = 3;
+            if (MASK) {                    // disabled channels are not loaded
+                planes = plane_bits(fc, s_mask, iz[u], org_z);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[u][c] = vcode;
+            }
+            fetch8_rows<S, AX>(src, (int)i0, st, v[u], planes);
         }
         DvrSample sm[AHEAD];
 #pragma unroll
         for (int u = 0; u < AHEAD; ++u) {
-            if (MASK) {
-                if (s_mask) mask_planes(v[u], s_mask[iz[u]], vcode);
-                else mask_channels(v[u], iz[u], org_z, fc.nz, fc.chmask, vcode);
-            }
             const Cell cl{0, 0, 0, fx[u], fy[u], fz[u]};
             interp_tf(v[u], cl, S != 0, scale, fc.vmin, fc.inv_range, fc.lutmax, fc.nlut - 2, s_lut, sm[u]);
         }
@@ -699,16 +709,12 @@ __device__ __forceinline__ int dvr_segment(const void *src, const Strides &st, c
         else
             fetch8<S>(src, cl.ix * st.x + cl.iy * st.y + cl.iz * st.z, st, v);
         DvrSample sm;
+        static_assert(F != 1 || !MASK);       // (a cached stencil keeps the stored values)
         if (MASK) {
-            float u[8];                   // (v keeps the stored values: the next cell may share them)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) u[k] = v[k];
-            if (s_mask) mask_planes(u, s_mask[cl.iz], vcode);
-            else mask_channels(u, cl.iz, org_z, fc.nz, fc.chmask, vcode);
-            interp_tf(u, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
-        } else {
-            interp_tf(v, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
+            if (s_mask) mask_planes(v, s_mask[cl.iz], vcode);
+            else mask_channels(v, cl.iz, org_z, fc.nz, fc.chmask, vcode);
         }
+        interp_tf(v, cl, S != 0, scale, vmin, inv_range, lutmax, lmax, s_lut, sm);
         over(sm, c0, c1, c2, T);
         if (T <= thr) return (int)jf + 1;
     }
@@ -1934,9 +1940,7 @@ cudaError_t launch_rc_s(const FrameConsts &fc, const float4 *lut, const DrawBric
 #define VR_RC_MASKED(MODE, F) (fc.chmask ? VR_RC(MODE, F, true) : VR_RC(MODE, F, false))
 #define VR_RC_MODE(F) (fc.mode != 0 ? VR_RC_MASKED(1, F) : VR_RC_MASKED(0, F))
     switch (fc.fetch) {
-        case 1:                        // (masked frames of 16-bit bricks read rows)
-            if constexpr (S == 0) return VR_RC_MASKED(0, 1);
-            else return VR_RC(0, 1, false);
+        case 1: return VR_RC(0, 1, false);      // (masked frames read rows)
         case 2: return VR_RC_MODE(2);
         case 6: return VR_RC_MODE(6);
         case 7: return VR_RC_MODE(7);

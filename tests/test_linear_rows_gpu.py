@@ -54,7 +54,7 @@ def test_linear_frames_match_the_oracle(ctx, orc, shape, brick, storage, masked)
 
 # a disabled channel's voxels hold the bottom of the table range: FP32 frames equal, bit for bit, those of a
 # cube edited so.  4097 stencil planes do not fit shared memory (the mask is read from global
-# memory), 4096 just do; cached stencils (oblique views of layout 1), rows and gathers
+# memory), 4096 just do; rows of layouts 1 and 7, gathers
 @pytest.mark.parametrize("nz", [40, 4095, 4096])
 @pytest.mark.parametrize("layouts", [1, 7, 9])
 def test_masked_frames_equal_frames_of_the_edited_cube(ctx, nz, layouts):
