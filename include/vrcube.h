@@ -206,7 +206,7 @@ int vr_wavelet_store(vr_ctx *ctx, int cube_id, void *dst, size_t *bytes);
  * more copy of the pool in HBM).  Bit 3 also keeps a slice atlas of every brick: a 2D texture
  * array in which the brick's z-slices stand in columns, from which a sample's 8 stencil voxels are
  * read by two texture gathers (exact texels; images identical to the linear copies).  When atlases
- * are kept every DVR and MIP frame whose camera is within 2^18 voxels reads them (farther ones the
+ * are kept every DVR and MIP frame whose rays start within 2^18 voxels reads them (others the
  * linear copy), and so does the adjoint's replay.  An atlas must fit the device's 2D-gather size
  * (32768 texels a side: stored bricks up to about 1000^3).
  * A bricked cube is rebuilt.  Streamed and compressed cubes (bricks made resident in the brick

@@ -117,7 +117,41 @@ double ray_reach(const vr_ctx *c, const Cube *cb) {
 // at most 3 half-ulps of 2^18 (0.047), and within a segment of at most 113 500 voxels j step and
 // q + t d about 0.011.  Cameras further away (rounding of whole voxels) read the linear copy, whose
 // indices are clamped; the frames are the same.
+// The argument takes a ray's origin to lie within its length of the cube, so the reach is that of the
+// origins the kernels form, R^T (e - t): with orthonormal rows |camera - cube centre| + diagonal covers
+// every ray that meets the cube, wherever on the image plane it starts.  Other view matrices are
+// accepted too (a sheared one can start its rays 10^7 voxels away while -R^T t is beside the cube, and cells
+// then leave the stored brick by several voxels): for them the frame's corners and the rounding of
+// the sum that forms an origin are counted.
 constexpr double kAtlasReach = 262144.0;
+bool within_reach(const vr_ctx *c, const Cube *cb) {
+    const Cam &m = c->cam;
+    double off = 0.0;                         // |R R^T - I|, largest element
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {
+            double d = i == j ? -1.0 : 0.0;
+            for (int k = 0; k < 3; ++k) d += (double)m.R[3 * i + k] * m.R[3 * j + k];
+            off = std::max(off, std::fabs(d));
+        }
+    if (off <= 1e-3) return ray_reach(c, cb) <= kAtlasReach;
+    double reach = 0.0, diag2 = 0.0;
+    for (int a = 0; a < 3; ++a) diag2 += (double)cb->n[a] * cb->n[a];
+    for (int k = 0; k < 4; ++k) {
+        const double hx = m.proj == VR_ORTHO ? (double)m.half_w : 0.0, hy = m.proj == VR_ORTHO ? (double)m.half_h : 0.0;
+        const double y[3] = {((k & 1) ? hx : -hx) - m.t[0], ((k & 2) ? hy : -hy) - m.t[1], -(double)m.t[2]};
+        double dist2 = 0.0, mag = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            double o = -0.5 * (double)cb->n[a];
+            for (int r = 0; r < 3; ++r) {
+                o += (double)m.R[3 * r + a] * y[r];
+                mag += std::fabs((double)m.R[3 * r + a] * y[r]);
+            }
+            dist2 += o * o;
+        }
+        reach = std::max(reach, std::sqrt(dist2) + mag * 0x1p-22);
+    }
+    return reach + std::sqrt(diag2) <= kAtlasReach;
+}
 
 // (1 / K is rounded up: floor(z / K) is then exact for the slices of any stored brick.)
 void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0) {
@@ -163,7 +197,7 @@ FrameLayout frame_layout(const vr_ctx *c, const Cube *cb) {
     // brick cache's slots, packed as bricks become resident
     // (within kAtlasReach: atlas frames clamp no index, see there)
     const bool atlas = (cb->streamed ? (cb->layouts & 8) != 0 && cb->atlas_fit : !cb->atlas_tex.empty()) &&
-                       (!c->cam_set || ray_reach(c, cb) <= kAtlasReach);
+                       (!c->cam_set || within_reach(c, cb));
     // with atlases, the image axis is fixed first: the one with the smaller z component
     const int only = atlas ? (std::fabs(c->cam.R[5]) < std::fabs(c->cam.R[2]) ? 1 : 0) : -1;
     for (int i = 0; i < 2; ++i)              // image axis: camera right (row 0), up (row 1)
@@ -546,7 +580,7 @@ FrameConsts make_consts(vr_ctx *c, Cube *cb) {
     // it saves; with a poor alignment it pays
     // (MIP frames: no stencil cache).  Cameras beyond kAtlasReach: clamped indices.
     if (fl.atlas) fc.fetch = cb->atlas_pair && !cb->streamed ? 5 : 2;
-    else if (c->cam_set && ray_reach(c, cb) > kAtlasReach) fc.fetch = 0;
+    else if (c->cam_set && !within_reach(c, cb)) fc.fetch = 0;
     // (masked frames read rows at every view, only those of enabled channels: 227 against 300 us a 641x479 frame
     // with every third channel off)
     else fc.fetch = fl.align < 0.9f && c->mode == VR_DVR && c->chmask.empty() ? 1 : 6 + fl.layout;

@@ -252,6 +252,8 @@ struct FrameLayout {
 FrameLayout frame_layout(const vr_ctx *c, const Cube *cb);
 // How far a ray that meets the cube can reach from its origin: |camera - cube centre| + diagonal.
 double ray_reach(const vr_ctx *c, const Cube *cb);
+// Whether the current camera's rays start near enough that no stencil index needs a clamp.
+bool within_reach(const vr_ctx *c, const Cube *cb);
 // Slice atlases: an array of w x h texels with columns of `rows` slices.
 struct AtlasGeom {
     int rows = 0, w = 0, h = 0;

@@ -1,0 +1,52 @@
+"""What the library's host code decides, on a stand-in runtime: no device."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from host_helpers import Host, fake_lib, launches
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return fake_lib(tmp_path_factory.mktemp("fake"))
+
+
+def _view(R, t):
+    v = np.eye(4)
+    v[:3, :3], v[:3, 3] = R, t
+    return v
+
+
+SHEAR = np.eye(3)
+SHEAR[0, 2] = 1e6
+STEEP = np.eye(3)
+STEEP[0, 2] = 2.0 ** 40
+# view, projection, whether unclamped reads are safe: rays of the sheared view start up to 6 10^7 voxels away
+# although R^T t is beside the cube; the steep one's eye is a sum of terms of 3 10^13, whose FP32 rounding is 10^6
+VIEWS = [(_view(np.eye(3), (-32, -32, -100)), 0, True), (_view(1.1 * np.eye(3), (-32, -32, -100)), 0, True),
+         (_view(np.eye(3), (-32, -32, -100)), 1, True), (_view(np.eye(3), (-32, -32, -3e5)), 1, False),
+         (_view(SHEAR, (0, -32, -80)), 0, False), (_view(STEEP, (-32, -32, 2.0 ** 45)), 1, False)]
+
+
+@pytest.mark.parametrize("view,proj,near", VIEWS)
+def test_cameras_whose_rays_start_far_away_read_clamped_stencils(lib, view, proj, near):
+    with Host(lib) as h:
+        for layouts in (1, 7, 9):
+            cid = h.load((64, 60, 62))
+            h.ok(h.brick(cid, (32, 32, 32), layouts))
+            for mode in (0, 1):
+                for mask in (None, bytes([1, 0] * 31)):
+                    h.ok(lib.vr_set_channel_mask(h.h, mask, 62 if mask else 0))
+                    h.camera(view, proj, 64.0 if proj == 0 else 1.0, mode=mode)
+                    launches(lib)
+                    h.ok(h.frame(cid))
+                    fetch = [a[2] for k, a in launches(lib) if k == "k_raycast"]
+                    assert len(fetch) == 1 and (fetch[0] == 0) == (not near), (layouts, mode, fetch)
+            h.ok(lib.vr_set_channel_mask(h.h, None, 0))
+            h.camera(view, proj, 64.0 if proj == 0 else 1.0)
+            launches(lib)
+            g, gl, gv = np.zeros((24, 32, 4), np.float32), np.zeros((2, 4), np.float32), np.zeros((62, 60, 64), np.float32)
+            h.ok(lib.vr_render_backward(h.h, cid, g.ctypes.data, gl.ctypes.data, gv.ctypes.data, None))
+            atlas = [a[0] for k, a in launches(lib) if k == "k_adjoint"]
+            assert atlas == [int(near and layouts == 9)]
