@@ -804,15 +804,28 @@ int check_ready(vr_ctx *c, Cube *cb) {
     return VR_OK;
 }
 
-// Whether p is memory of device `dev` that a kernel there can read (another device's memory and host
-// memory registered or managed are left to the copy engine).
-bool own_device_memory(const void *p, int dev) {
+// Whether a kernel on device `dev` may read [p, p + bytes) as floats: one allocation there holds all of
+// it, 4-byte aligned.  Everything else is left to the copy engine, which takes any alignment, another
+// device's memory and host memory registered or managed, and refuses a range that is not there.
+bool own_device_floats(const void *p, size_t bytes, int dev) {
+    using Range = int (*)(unsigned long long *, size_t *, unsigned long long);      // cuMemGetAddressRange
+    static const Range range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && r == cudaDriverEntryPointSuccess ? reinterpret_cast<Range>(f) : nullptr;
+    }();
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    const unsigned long long q = reinterpret_cast<uintptr_t>(p);
+    unsigned long long base = 0;
+    size_t size = 0;
+    return at.type == cudaMemoryTypeDevice && at.device == dev && q % sizeof(float) == 0 && range &&
+           range(&base, &size, q) == 0 && q - base <= size && bytes <= size - (q - base);
 }
 
 // Releases a cube's slice atlases (to the context's idle arrays while those are few).  Frames in
@@ -1452,7 +1465,7 @@ static int vr_load_cube_body(vr_ctx *c, const void *voxels, int dtype, int64_t n
         free_cube(c, cb);
         return cuda_fail(e, "cudaDeviceSynchronize (device cube source)");
     }
-    if (where == VR_DEVICE && !sub_origin && own_device_memory(voxels, c->device)) {
+    if (where == VR_DEVICE && !sub_origin && own_device_floats(voxels, bytes, c->device)) {
         // the whole array: one linear pass (the 3D copy below moves device memory at a quarter of HBM's rate)
         e = launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)nx * ny * nz, c->load_stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->load_stream);
@@ -1526,7 +1539,7 @@ static int vr_update_cube_body(vr_ctx *c, int cube_id, const void *voxels, int w
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t bytes = sizeof(float) * (size_t)cb->n[0] * cb->n[1] * cb->n[2];
     if (c->frame_pending) CK(cudaStreamWaitEvent(s, c->frame_done, 0));
-    if (where == VR_DEVICE && own_device_memory(voxels, c->device)) CK(launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)(bytes / sizeof(float)), s));
+    if (where == VR_DEVICE && own_device_floats(voxels, bytes, c->device)) CK(launch_copy(static_cast<const float *>(voxels), cb->d_src, (long long)(bytes / sizeof(float)), s));
     else CK(cudaMemcpyAsync(cb->d_src, voxels, bytes, where == VR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
     if (cb->bricked) return build_bricks(c, cb, s);
     CK(cudaStreamSynchronize(s));

@@ -1,6 +1,8 @@
 """Bricking kernels at their edges: sources off a 16-byte boundary and of sizes that are no multiple
 of 4, rows shorter and longer than a warp, scale exponents beyond one multiplication, more bricks
 than one shelf of an atlas array holds, and arrays written again by an update."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -77,3 +79,23 @@ def test_shelves_of_small_bricks_and_updates(ctx, storage, mask):
         ctx.free_cube(cid)
     assert np.array_equal(frames[0], frames[2]) and np.array_equal(frames[1], frames[3])
     assert not np.array_equal(frames[0], frames[1])
+
+
+@pytest.mark.parametrize("offset", [1, 2, 4, 12])
+def test_device_voxels_at_any_address(offset):
+    """Sources that start between floats (copied by the copy engine) and between 16-byte pieces."""
+    import torch
+    ctx = gpu_ctx()
+    cube = np.random.default_rng(4).standard_normal((11, 13, 21)).astype(np.float32)
+    buf = torch.zeros(cube.nbytes + 16, dtype=torch.uint8, device="cuda")
+    buf[offset:offset + cube.nbytes] = torch.from_numpy(cube.view(np.uint8).ravel()).cuda()
+    torch.cuda.synchronize()
+    cid = C.c_int()
+    assert ctx._L.vr_load_cube(ctx._h, buf.data_ptr() + offset, 0, 21, 13, 11, 1, None, None, C.byref(cid)) == 0
+    ctx.set_bricking(cid.value, (32, 32, 32), 1, "f32")
+    assert np.array_equal(ctx.get_brick(cid.value, 0)[3][1:-1, 1:-1, 1:-1], cube)
+    buf[offset:offset + cube.nbytes] = torch.from_numpy((2 * cube).view(np.uint8).ravel()).cuda()
+    torch.cuda.synchronize()
+    assert ctx._L.vr_update_cube(ctx._h, cid.value, buf.data_ptr() + offset, 1, None) == 0
+    assert np.array_equal(ctx.get_brick(cid.value, 0)[3][1:-1, 1:-1, 1:-1], 2 * cube)
+    ctx.close()

@@ -50,3 +50,18 @@ def test_cameras_whose_rays_start_far_away_read_clamped_stencils(lib, view, proj
             h.ok(lib.vr_render_backward(h.h, cid, g.ctypes.data, gl.ctypes.data, gv.ctypes.data, None))
             atlas = [a[0] for k, a in launches(lib) if k == "k_adjoint"]
             assert atlas == [int(near and layouts == 9)]
+
+
+@pytest.mark.parametrize("offset,short,kernel", [(0, 0, True), (4, 0, True), (12, 0, True), (1, 0, False), (2, 0, False),
+                                                 (0, 4, False), (4, 4, False)])
+def test_device_sources_that_a_kernel_cannot_read_go_to_the_copy_engine(lib, offset, short, kernel):
+    """Voxels at an address that is no multiple of 4, or (from the copy engine: an error) beyond their allocation."""
+    n, cid = 4 * 9 * 7 * 5, C.c_int()
+    with Host(lib) as h:
+        src = lib.fake_device_alloc(n + offset - short) + offset
+        launches(lib)
+        h.ok(lib.vr_load_cube(h.h, src, 0, 9, 7, 5, 1, None, None, C.byref(cid)))
+        assert launches(lib) == [("k_copy" if kernel else "cudaMemcpy3DAsync", ())]
+        rc = lib.vr_update_cube(h.h, cid.value, src, 1, None)
+        assert launches(lib) == [("k_copy" if kernel else "cudaMemcpyAsync", ())]
+        assert rc == (-3 if short else 0)
