@@ -1002,7 +1002,6 @@ int stage_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(tmp, 0, most, s);
     for (size_t i = 0; i < cb->tmpl.size() && e == cudaSuccess; ++i) {
         const AtlasCell &cell = cb->atlas_cells[i];
-        if (cell.surf) continue;
         const int *dm = cb->tmpl[i].dim;
         extent(i, w, h);
         const char *src = static_cast<const char *>(cb->d_pool) + (size_t)cb->loff[3 * i] * bsz;
@@ -1033,7 +1032,8 @@ int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
     else if (cb->atlas_arr.empty()) { if ((rc = make_atlases(c, cb)) != VR_OK) return rc; }
     else CK(cudaDeviceSynchronize());        // frames in flight may still gather from the arrays
     const bool atlas = !cb->atlas_arr.empty();
-    const bool surf = atlas && cb->atlas_surf[0] != 0;
+    // (one array without a surface, which any failure to make one with it leaves: all through staging)
+    const bool surf = atlas && std::count(cb->atlas_surf.begin(), cb->atlas_surf.end(), 0ull) == 0;
     unsigned int *d_range = cb->d_bs + 2 * (size_t)nbr;
     int *d_exps = reinterpret_cast<int *>(cb->d_bs + nbr);
     AtlasCell *d_cells = reinterpret_cast<AtlasCell *>(cb->d_tmpl + nbr);

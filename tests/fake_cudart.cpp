@@ -62,7 +62,7 @@ int address_range(unsigned long long *base, size_t *size, unsigned long long p) 
 
 #define API extern "C" __attribute__((visibility("default")))
 // ---- what the tests ask for
-API void fake_reset() { launches.clear(); limit = ~size_t(0); surf_calls = 0; surf_fail = -1; }
+API void fake_reset() { last = cudaSuccess; launches.clear(); limit = ~size_t(0); surf_calls = 0; surf_fail = -1; }
 API void fake_limit(size_t bytes) { limit = bytes; }
 API size_t fake_reserved() { return used + idle; }
 API int fake_arrays() { return (int)arrays.size(); }

@@ -36,9 +36,11 @@ def fake_lib(tmp):
 def launches(L):
     """[(kernel, template arguments)] launched (and copies made) since the last call."""
     out = []
-    for m in L.fake_launches().decode().split():
-        k = re.search(r"\d(k_[a-z_]+?)(?:I((?:L[ib]\d+E)+)[^P]*)?E?[vRP]", m)
-        out.append((k.group(1), tuple(int(x) for x in re.findall(r"L[ib](\d+)E", k.group(2) or ""))) if k else (m, ()))
+    names = subprocess.run(["c++filt"], input=L.fake_launches().decode(), capture_output=True, text=True, check=True).stdout
+    for name in names.splitlines():
+        k = re.search(r"\b(k_\w+)(?:<([^(]*)>)?\(", name.replace("(anonymous namespace)::", ""))
+        args = (k.group(2) or "").replace("true", "1").replace("false", "0").split(", ") if k else []
+        out.append((k.group(1) if k else name, tuple(int(x) for x in args if x.isdigit())))
     return out
 
 

@@ -65,3 +65,19 @@ def test_device_sources_that_a_kernel_cannot_read_go_to_the_copy_engine(lib, off
         rc = lib.vr_update_cube(h.h, cid.value, src, 1, None)
         assert launches(lib) == [("k_copy" if kernel else "cudaMemcpyAsync", ())]
         assert rc == (-3 if short else 0)
+
+
+@pytest.mark.parametrize("without", [(), (0,), (1,)])
+def test_atlas_arrays_with_and_without_surfaces(lib, without):
+    """Two arrays, one of which the device gives no surface: both bricks' atlases are packed through staging."""
+    with Host(lib) as h:
+        cid = h.load((2048, 64, 248))                  # a shelf each: 1026 texels wide, 16500 high
+        launches(lib)
+        for nth in without:
+            lib.fake_fail_surface_array(nth, 801)
+        h.ok(h.brick(cid, (1024, 64, 248)))
+        assert lib.fake_arrays() == 2
+        ran = launches(lib)
+        assert [a for k, a in ran if k == "k_brick_build"] == [(0, 0 if without else 1)]
+        assert [k for k, _ in ran].count("k_atlas_pack") == [k for k, _ in ran].count("cudaMemcpy2DToArrayAsync")
+        assert [k for k, _ in ran].count("k_atlas_pack") == (2 if without else 0)
