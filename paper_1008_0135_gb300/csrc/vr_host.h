@@ -22,7 +22,10 @@ using namespace vr;
 // Detail of the last failure on this thread (vr_last_error_message).
 inline thread_local std::string g_last_error;
 
+// (The runtime keeps a failed call's error for the next cudaGetLastError, which every launch asks: it is
+// taken back here, or the call after a failed one would fail with its error.)
 inline int cuda_fail(cudaError_t e, const char *where) {
+    cudaGetLastError();
     g_last_error = std::string(where) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
     return e == cudaErrorMemoryAllocation ? VR_ERR_OOM : VR_ERR_CUDA;
 }
@@ -289,7 +292,8 @@ cudaError_t alloc_retry(vr_ctx *c, F f) {
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
     idle_release(c);
-    return f();
+    if ((e = f()) != cudaSuccess) cudaGetLastError();
+    return e;
 }
 void idle_slot_free(IdleSlot &s);
 int set_dev(vr_ctx *c);

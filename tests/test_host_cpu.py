@@ -81,3 +81,29 @@ def test_atlas_arrays_with_and_without_surfaces(lib, without):
         assert [a for k, a in ran if k == "k_brick_build"] == [(0, 0 if without else 1)]
         assert [k for k, _ in ran].count("k_atlas_pack") == [k for k, _ in ran].count("cudaMemcpy2DToArrayAsync")
         assert [k for k, _ in ran].count("k_atlas_pack") == (2 if without else 0)
+
+
+@pytest.mark.parametrize("what", ["load", "short source", "bricking", "cache"])
+def test_the_call_after_a_failed_one_does_not_fail_with_its_error(lib, what):
+    with Host(lib, cache=1 << 20) as h:
+        cid, other = h.load((64, 60, 62)), C.c_int()
+        h.ok(h.brick(cid, (32, 32, 32)))
+        h.camera(_view(np.eye(3), (-32, -32, -100)))
+        h.ok(h.frame(cid))
+        src = lib.fake_device_alloc(64)
+        lib.fake_limit(lib.fake_reserved() + (1 << 16))
+        if what == "load":
+            cube = np.zeros((64, 64, 64), np.float32)
+            rc = lib.vr_load_cube(h.h, cube.ctypes.data, 0, 64, 64, 64, 0, None, None, C.byref(other))
+        elif what == "short source":
+            rc = lib.vr_update_cube(h.h, cid, src, 1, None)
+        elif what == "bricking":
+            rc = lib.vr_set_brick_layouts(h.h, cid, 31)
+        else:
+            h.ok(lib.vr_load_cube_procedural(h.h, 1, 20, 20, 20, C.byref(other)))
+            h.ok(h.brick(other.value, (16, 16, 16), 1))
+            rc = h.frame(other.value)
+        assert rc == (-3 if what == "short source" else -2)
+        h.ok(lib.vr_compute_minmax(h.h, cid, C.byref(C.c_float()), C.byref(C.c_float())))
+        if what != "bricking":
+            h.ok(h.frame(cid))
