@@ -124,8 +124,7 @@ double ray_reach(const vr_ctx *c, const Cube *cb) {
 // then leave the stored brick by several voxels): for them the frame's corners and the rounding of
 // the sum that forms an origin are counted.
 constexpr double kAtlasReach = 262144.0;
-bool within_reach(const vr_ctx *c, const Cube *cb) {
-    const Cam &m = c->cam;
+static bool orthonormal(const Cam &m) {
     double off = 0.0;                         // |R R^T - I|, largest element
     for (int i = 0; i < 3; ++i)
         for (int j = 0; j < 3; ++j) {
@@ -133,7 +132,11 @@ bool within_reach(const vr_ctx *c, const Cube *cb) {
             for (int k = 0; k < 3; ++k) d += (double)m.R[3 * i + k] * m.R[3 * j + k];
             off = std::max(off, std::fabs(d));
         }
-    if (off <= 1e-3) return ray_reach(c, cb) <= kAtlasReach;
+    return off <= 1e-3;
+}
+bool within_reach(const vr_ctx *c, const Cube *cb) {
+    const Cam &m = c->cam;
+    if (orthonormal(m)) return ray_reach(c, cb) <= kAtlasReach;
     double reach = 0.0, diag2 = 0.0;
     for (int a = 0; a < 3; ++a) diag2 += (double)cb->n[a] * cb->n[a];
     for (int k = 0; k < 4; ++k) {
@@ -788,6 +791,23 @@ int stage_frame(vr_ctx *c, Cube *cb, WorkList &wl, cudaStream_t s, cudaEvent_t e
     return VR_OK;
 }
 
+// The length of an orthographic view's ray direction, at most 1: rows that are not orthonormal give a
+// direction of another length, and a short one puts that many more samples into a brick.
+// (Perspective directions differ from pixel to pixel; a ray's samples are bounded in box_krange.)
+static double direction_length(const Cam &m) {
+    if (m.proj != VR_ORTHO || orthonormal(m)) return 1.0;
+    double l2 = 0.0;
+    for (int k = 0; k < 3; ++k) l2 += (double)m.R[6 + k] * m.R[6 + k];
+    return std::min(1.0, std::sqrt(l2));
+}
+
+// Sample indices count as floats up to 2^24 along a segment (beyond, a ray's loop would not end).
+static bool countable(const Cam &m, const Cube *cb, float step) {
+    double diag2 = 0.0;
+    for (int k = 0; k < 3; ++k) diag2 += (double)cb->n[k] * cb->n[k];
+    return !(std::sqrt(diag2) / ((double)step * direction_length(m)) > (double)(1 << 24));
+}
+
 int check_ready(vr_ctx *c, Cube *cb) {
     if (!cb->bricked) { g_last_error = "cube has no bricking"; return VR_ERR_STATE; }
     if (!c->chmask.empty() && (int64_t)c->chmask.size() != cb->n[2])
@@ -796,10 +816,8 @@ int check_ready(vr_ctx *c, Cube *cb) {
     if (!c->cam_set) { g_last_error = "no camera"; return VR_ERR_STATE; }
     // every lattice index k = t/step reached inside the cube must fit comfortably in an int:
     // t <= |camera - cube centre| + half diagonal
-    double diag2 = 0.0;
-    for (int k = 0; k < 3; ++k) diag2 += (double)cb->n[k] * cb->n[k];
     const double tmax = ray_reach(c, cb);
-    if (tmax / (double)c->step > (double)(1 << 28) || std::sqrt(diag2) / c->step > (double)(1 << 24))
+    if (tmax / (double)c->step > (double)(1 << 28) || !countable(c->cam, cb, c->step))
         return arg_fail("step too small for this camera and cube (lattice index would overflow)");
     return VR_OK;
 }
@@ -2246,8 +2264,10 @@ static int vr_render_backward_views_body(vr_ctx *c, int cube_id, int n_views, co
     if (reinterpret_cast<uintptr_t>(grad_out) % 16 != 0) return arg_fail("grad_out must be 16-byte aligned");
     const int W = c->cam.W, H = c->cam.H;
     Cam probe;
-    for (int v = 0; v < n_views; ++v)      // every view valid before any work is queued
+    for (int v = 0; v < n_views; ++v) {    // every view valid before any work is queued
         if ((rc = make_cam(views[v].view, views[v].proj, views[v].param, W, H, probe)) != VR_OK) return rc;
+        if (!countable(probe, cb, c->step)) return arg_fail("step too small for this camera and cube (lattice index would overflow)");
+    }
     if ((rc = set_dev(c)) != VR_OK) return rc;
     if ((rc = ensure(c->d_gacc, (size_t)4 * c->lut.size(), c)) != VR_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);

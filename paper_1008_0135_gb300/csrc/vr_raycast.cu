@@ -119,6 +119,9 @@ __device__ __forceinline__ bool box_krange(const float o[3], const float d[3], c
     if (!(tout > tin) || !(tout < INFINITY)) return false;   // no direction: no samples
     k0 = (int)ceilf(__fdiv_rn(tin, step));
     k1 = (int)ceilf(__fdiv_rn(tout, step));
+    // samples are counted in floats: with a direction far shorter than 1 (a view matrix whose rows are
+    // not orthonormal) more of them would never be counted to the end.  The host admits no others.
+    if (k1 - k0 > (1 << 24) + 1) k1 = k0 + (1 << 24) + 1;
     return k1 > k0;
 }
 
@@ -1634,7 +1637,7 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
     const float qx = anchor(o[0], d[0], b.org_c[0], k0, fc.step);
     const float qy = anchor(o[1], d[1], b.org_c[1], k0, fc.step);
     const float qz = anchor(o[2], d[2], b.org_c[2], k0, fc.step);
-    const float nf = (float)(k1 - k0);         // exact: at most 2^24 + 1
+    const float nf = (float)(k1 - k0);         // at most 2^24 + 1, which rounds to 2^24
     const float dxdv = __fmul_rn(fc.lutmax, fc.inv_range);
     const float grest = gf.w * fr.w;
     float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, T = 1.0f;

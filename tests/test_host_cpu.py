@@ -4,6 +4,7 @@ import ctypes as C
 import numpy as np
 import pytest
 
+from paper_1008_0135_gb300 import _abi
 from host_helpers import Host, fake_lib, launches
 
 
@@ -107,3 +108,27 @@ def test_the_call_after_a_failed_one_does_not_fail_with_its_error(lib, what):
         h.ok(lib.vr_compute_minmax(h.h, cid, C.byref(C.c_float()), C.byref(C.c_float())))
         if what != "bricking":
             h.ok(h.frame(cid))
+
+
+FLAT = np.diag([1e3, 1e3, 1e-6])
+
+
+@pytest.mark.parametrize("R,proj,counts", [(np.eye(3), 0, True), (np.eye(3), 1, True), (0.9 * np.eye(3), 1, True), (SHEAR, 0, True),
+                                           (FLAT, 0, False), (FLAT, 1, True)])
+def test_directions_too_short_to_count_samples_along_are_refused(lib, R, proj, counts):
+    """A direction of length 1e-6 puts 2 10^8 samples of step 0.5 into 110 voxels: a float does not count them.
+    (A perspective view's directions are only as short in single pixels.)"""
+    view, err = _view(R, (-32, -32, -100)), -1
+    with Host(lib) as h:
+        cid = h.load((64, 60, 62))
+        h.ok(h.brick(cid, (32, 32, 32)))
+        g, gl = np.zeros((24, 32, 4), np.float32), np.zeros((2, 4), np.float32)
+        arr = (_abi.VrView * 1)()
+        arr[0].view[:], arr[0].proj, arr[0].param = [float(x) for x in view.ravel()], proj, 1.0
+        h.camera(np.eye(4), step=0.5)
+        assert lib.vr_render_backward_views(h.h, cid, 1, arr, g.ctypes.data, gl.ctypes.data, None, None) == (0 if counts else err)
+        for mode in (0, 1):
+            h.camera(view, proj, 1.0, mode=mode, step=0.5)
+            launches(lib)
+            assert h.frame(cid) == (0 if counts else err)
+            assert any(k == "k_raycast" for k, _ in launches(lib)) == counts
