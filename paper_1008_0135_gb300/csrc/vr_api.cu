@@ -72,6 +72,10 @@ void mem_free(vr_ctx *c, void *p) {
     else cudaFree(p);
 }
 
+void mem_settle(vr_ctx *c) {
+    if (c->mem) cudaStreamSynchronize(c->load_stream);
+}
+
 void layout_strides(const int dim[3], int layout, int str[3]) {
     // the contiguous axis first, then the other two in x, y, z order
     int ord[3];
@@ -1103,6 +1107,7 @@ int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
 void free_cube(vr_ctx *c, Cube *cb) {
     free_atlases(c, cb);
     for (void *p : {(void *)cb->d_wstore, (void *)cb->d_src, cb->d_pool, (void *)cb->d_tmpl, (void *)cb->d_bs}) mem_free(c, p);
+    mem_settle(c);
     delete cb;
 }
 
@@ -1744,6 +1749,7 @@ static int vr_compress_cube_body(vr_ctx *c, int cube_id) {
     CK(cudaDeviceSynchronize());
     free_atlases(c, cb);
     for (void *p : {(void *)cb->d_src, cb->d_pool, (void *)cb->d_tmpl, (void *)cb->d_bs}) mem_free(c, p);
+    mem_settle(c);
     cb->d_src = nullptr;
     cb->d_pool = nullptr;
     cb->d_tmpl = nullptr;

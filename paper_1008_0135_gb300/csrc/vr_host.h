@@ -284,6 +284,9 @@ constexpr size_t kIdleSlots = 16;
 // by work on load_stream or after waiting for it.
 cudaError_t mem_alloc(vr_ctx *c, void **p, size_t bytes);
 void mem_free(vr_ctx *c, void *p);
+// Gives what the pool holds above kIdleBytes back to the device, which it only does when something is
+// waited for: calls that leave memory behind end with this.
+void mem_settle(vr_ctx *c);
 void idle_release(vr_ctx *c);                     // everything idle back to the device
 // f(), once more after everything idle is given back if the device was out of memory
 template <typename F>

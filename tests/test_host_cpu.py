@@ -132,3 +132,23 @@ def test_directions_too_short_to_count_samples_along_are_refused(lib, R, proj, c
             launches(lib)
             assert h.frame(cid) == (0 if counts else err)
             assert any(k == "k_raycast" for k, _ in launches(lib)) == counts
+
+
+@pytest.mark.parametrize("how", ["free", "compress", "rebrick"])
+def test_memory_that_a_cube_leaves_is_bounded_when_the_call_returns(lib, how):
+    """At most 2 GiB of it stays with the context (vr_create), not what the next wait would give back."""
+    n, kept = (1000, 1000, 700), 2 << 30                       # 2.6 GiB of voxels, 2.7 of bricks
+    with Host(lib) as h:
+        base = lib.fake_reserved()
+        cid = h.load(n)
+        if how != "compress":
+            h.ok(h.brick(cid, (128, 128, 128), 7))
+        if how == "free":
+            h.ok(lib.vr_free_cube(h.h, cid))
+            assert lib.fake_reserved() - base <= kept
+        elif how == "compress":
+            h.ok(lib.vr_compress_cube(h.h, cid))
+            assert lib.fake_reserved() - base <= kept + 544 * 125 * 125 * 88
+        else:
+            h.ok(lib.vr_set_brick_layouts(h.h, cid, 1))
+            assert lib.fake_reserved() - base <= kept + int(2.2 * 4 * n[0] * n[1] * n[2])

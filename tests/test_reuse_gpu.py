@@ -100,3 +100,16 @@ def test_serving_loops_hand_their_slots_on():
     server.close()
     check(rs)
     ctx.close()
+
+
+def test_a_freed_cube_leaves_no_more_than_its_bound():
+    """What vr_free_cube keeps above 2 GiB is back with the device when it returns (32 MiB for other users)."""
+    import torch
+    ctx = _ctx()
+    cid = ctx.load_cube(np.zeros((700, 1000, 1000), np.float32))
+    torch.cuda.synchronize()
+    with_cube = torch.cuda.mem_get_info()[0]
+    ctx.free_cube(cid)
+    freed = torch.cuda.mem_get_info()[0] - with_cube
+    ctx.close()
+    assert freed >= 4 * 700 * 1000 * 1000 - (2 << 30) - (32 << 20)
