@@ -93,8 +93,9 @@ typedef struct {
 /* Creates a context on CUDA device `device`.  cache_bytes bounds the HBM brick cache used for
  * cubes whose bricks are streamed from host memory (0 = no streaming cache).  *out receives
  * the context; it is released by vr_destroy.  A context keeps, unused, up to 2 GiB of the device
- * memory and 1 GiB of the atlas arrays of cubes it freed, and up to 16 frame slots (2 GiB) of
- * closed serving loops, for its next ones; its own allocations take all of that back when the
+ * memory and 1 GiB of the atlas arrays of cubes it freed, up to 16 frame slots (2 GiB) of
+ * closed serving loops and the scratch of the largest voxel gradient (16 bytes a voxel, at most
+ * 4 GiB), for its next ones; its own allocations take all of that back when the
  * device is out of memory, vr_destroy releases it.  Errors: VR_ERR_ARG (null out, bad device),
  * VR_ERR_CUDA, VR_ERR_OOM. */
 int vr_create(vr_ctx **out, int device, size_t cache_bytes);

@@ -52,6 +52,10 @@ void idle_release(vr_ctx *c) {
     c->idle_arrays.clear();
     for (auto &s : c->idle_slots) idle_slot_free(s);
     c->idle_slots.clear();
+    if (c->d_corner.p && !c->corner_busy) {            // (cudaFree waits for the last gather)
+        cudaFree(c->d_corner.p);
+        c->d_corner = DevBuf<float4>{};
+    }
     if (c->mem) {
         cudaStreamSynchronize(c->load_stream);
         cudaMemPoolTrimTo(c->mem, 0);
@@ -674,17 +678,32 @@ int backward_corners(vr_ctx *c, Cube *cb, int n_views, cudaStream_t s, float4 **
     }
     const double samples = (double)n_views * c->cam.W * c->cam.H * std::sqrt(diag2) / (double)c->step;
     if (n * sizeof(float4) > kCornerBytes || samples < 0.2 * vox) return VR_OK;
-    const int rc = ensure(c->d_corner, n, c);
-    if (rc == VR_ERR_OOM) {                            // no room: one atomic per corner
-        cudaGetLastError();
-        return VR_OK;
+    if (c->d_corner.cap < n) {                         // (not ensure: no room to grow beyond kCornerBytes)
+        if (c->d_corner.p) CK(cudaFree(c->d_corner.p));
+        c->d_corner = DevBuf<float4>{};
+        const cudaError_t e = alloc_retry(c, [&] { return cudaMalloc(&c->d_corner.p, n * sizeof(float4)); });
+        if (e == cudaErrorMemoryAllocation) {          // no room: one atomic per corner
+            c->d_corner = DevBuf<float4>{};
+            return VR_OK;
+        }
+        CK(e);
+        c->d_corner.cap = n;
     }
-    if (rc != VR_OK) return rc;
     if (c->frame_pending) CK(cudaStreamWaitEvent(s, c->frame_done, 0));   // the last call's gather may still read them
     CK(cudaMemsetAsync(c->d_corner.p, 0, n * sizeof(float4), s));
     *out = c->d_corner.p;
     return VR_OK;
 }
+
+// While a gradient call is using the corner sums, an allocation of its own that finds no memory must not
+// release them.
+struct CornersBusy {
+    vr_ctx *c;
+    explicit CornersBusy(vr_ctx *ctx) : c(ctx) { c->corner_busy = true; }
+    CornersBusy(const CornersBusy &) = delete;
+    CornersBusy &operator=(const CornersBusy &) = delete;
+    ~CornersBusy() { c->corner_busy = false; }
+};
 
 // The adjoint of the current camera's frame: composite backward, ray replay, and the table
 // gradient either reduced into grad_lut (FP64 sum rounded once) or, with acc, added to the FP64
@@ -2246,6 +2265,7 @@ static int vr_render_backward_body(vr_ctx *c, int cube_id, const float *grad_out
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     float4 *corners = nullptr;
     if (grad_voxels && (rc = backward_corners(c, cb, 1, s, &corners)) != VR_OK) return rc;
+    const CornersBusy busy(c);
     if ((rc = backward_view(c, cb, grad_out, grad_lut, nullptr, false, grad_voxels, corners, s)) != VR_OK) return rc;
     if (!corners) return VR_OK;
     CK(launch_corner_gather(corners, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], grad_voxels, s));
@@ -2280,6 +2300,7 @@ static int vr_render_backward_views_body(vr_ctx *c, int cube_id, int n_views, co
     const size_t per_view = (size_t)W * H * 4;
     float4 *corners = nullptr;
     if (grad_voxels && (rc = backward_corners(c, cb, n_views, s, &corners)) != VR_OK) return rc;
+    const CornersBusy busy(c);
     // last view first: its fragments are usually the last frame's (render the batch, then
     // differentiate it), reused when the camera is unchanged
     for (int v = n_views - 1; v >= 0; --v) {

@@ -208,7 +208,9 @@ struct vr_ctx {
     vrh::DevBuf<char> d_stage;
     vrh::DevBuf<char> d_frags;        // bytes
     vrh::DevBuf<float4> d_gfrag;
-    vrh::DevBuf<float4> d_corner;       // corner sums of the voxel gradient (backward_corners)
+    vrh::DevBuf<float4> d_corner;       // corner sums of the voxel gradient (backward_corners); idle_release
+                                        // gives them back unless a gradient call is using them
+    bool corner_busy = false;
     vrh::DevBuf<float> d_gpart;
     vrh::DevBuf<double> d_gacc;         // FP64 table-gradient sum over the views of a batch
     vrh::DevBuf<double> d_gchunk;       // FP64 chunk sums of a view's table-gradient partials

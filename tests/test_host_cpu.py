@@ -152,3 +152,31 @@ def test_memory_that_a_cube_leaves_is_bounded_when_the_call_returns(lib, how):
         else:
             h.ok(lib.vr_set_brick_layouts(h.h, cid, 1))
             assert lib.fake_reserved() - base <= kept + int(2.2 * 4 * n[0] * n[1] * n[2])
+
+
+def test_the_scratch_of_a_voxel_gradient_is_exact_and_given_back(lib):
+    def backward(h, cid, n, nlut=2):
+        lut = np.zeros((nlut, 4), np.float32)
+        h.ok(lib.vr_set_transfer_function(h.h, lut.ctypes.data, nlut, 0.0, 1.0))
+        h.camera(_view(np.eye(3), (-n / 2, -n / 2, -2 * n)), param=1.5 * n, W=512, H=512, step=0.5)
+        return lib.vr_render_backward(h.h, cid, h.out.ctypes.data, h.out.ctypes.data, h.out.ctypes.data, None)
+
+    size = lambda n: 16 * (n + 1) ** 2 * (n + 2)
+    with Host(lib) as h:
+        small, large = h.load((200, 200, 200)), h.load((204, 204, 204))
+        h.ok(h.brick(small, (256, 256, 256)))
+        h.ok(h.brick(large, (256, 256, 256)))
+        h.ok(backward(h, small, 200))
+        before = lib.fake_reserved()
+        h.ok(backward(h, large, 204))                     # not 1.5 times the last one's
+        assert lib.fake_reserved() - before < size(204) - size(200) + (16 << 20)
+        # an allocation of the call itself that finds no memory leaves the sums it is using
+        lib.fake_limit(lib.fake_reserved() + (1 << 20))
+        before = lib.fake_reserved()
+        assert backward(h, large, 204, nlut=4096) == -2
+        assert before - lib.fake_reserved() < size(204) // 2
+        # another call's takes them back
+        cube, cid = np.zeros((150, 200, 200), np.float32), C.c_int()
+        h.ok(lib.vr_load_cube(h.h, cube.ctypes.data, 0, 200, 200, 150, 0, None, None, C.byref(cid)))
+        lib.fake_limit((1 << 64) - 1)
+        h.ok(backward(h, small, 200))
