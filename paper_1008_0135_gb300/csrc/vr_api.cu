@@ -869,7 +869,7 @@ bool own_device_floats(const void *p, size_t bytes, int dev) {
            range(&base, &size, q) == 0 && q - base <= size && bytes <= size - (q - base);
 }
 
-// Releases a cube's slice atlases (to the context's idle arrays while those are few).  Frames in
+// Releases a cube's slice atlases (to the context's idle arrays).  Frames in
 // flight may still gather from them: the device is drained first (atlases go only with the bricking).
 void free_atlases(vr_ctx *c, Cube *cb) {
     if (cb->atlas_arr.empty() && cb->atlas_tex.empty()) return;
@@ -888,12 +888,19 @@ void free_atlases(vr_ctx *c, Cube *cb) {
         }
         a.kind = cb->atlas_kind;
         a.bytes = (size_t)a.w * a.h * (a.kind == 0 || a.kind == 3 ? 4 : 2);
-        if (a.tex && a.surf && a.w > 0 && kept + a.bytes <= kIdleArrayBytes && c->idle_arrays.size() < 256) {
-            kept += a.bytes;
-            c->idle_arrays.push_back(a);
-        } else {
+        if (!(a.tex && a.surf && a.w > 0 && a.bytes <= kIdleArrayBytes)) {
             idle_array_free(a);
+            continue;
         }
+        // the oldest go: what a viewer's last cubes left is what its next ones are like
+        size_t gone = 0;
+        while (kept + a.bytes > kIdleArrayBytes || c->idle_arrays.size() - gone >= kIdleArrays) {
+            kept -= c->idle_arrays[gone].bytes;
+            idle_array_free(c->idle_arrays[gone++]);
+        }
+        c->idle_arrays.erase(c->idle_arrays.begin(), c->idle_arrays.begin() + gone);
+        kept += a.bytes;
+        c->idle_arrays.push_back(a);
     }
     cb->atlas_tex.clear();
     cb->atlas_surf.clear();

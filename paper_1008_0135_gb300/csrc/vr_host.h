@@ -280,7 +280,7 @@ void layout_strides(const int dim[3], int layout, int str[3]);
 MarchGrid march_grid(const vr_ctx *c, const Cube *cb);
 
 constexpr size_t kIdleBytes = size_t(2) << 30, kIdleArrayBytes = size_t(1) << 30;
-constexpr size_t kIdleSlots = 16;
+constexpr size_t kIdleSlots = 16, kIdleArrays = 256;
 // Memory of a cube.  Allocated and freed on load_stream: the caller of mem_free has drained whatever
 // reads it (cudaFree's implicit wait is not there), and what mem_alloc returned is written first
 // by work on load_stream or after waiting for it.

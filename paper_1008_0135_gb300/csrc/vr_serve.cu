@@ -93,8 +93,8 @@ bool slot_open(vr_ctx *parent, FrameSlot &sl) {
            cudaEventCreateWithFlags(&sl.c->frame_done, cudaEventDisableTiming) == cudaSuccess;
 }
 
-// The slot's work is done (its stream was waited for): what it holds is left to the context while that
-// is little, else released.
+// The slot's work is done (its stream was waited for): what it holds is left to the context, which
+// releases its oldest idle slots for it.
 void slot_close(vr_ctx *parent, FrameSlot &sl) {
     IdleSlot is;
     is.s = sl.s;
@@ -116,8 +116,17 @@ void slot_close(vr_ctx *parent, FrameSlot &sl) {
     size_t kept = is.bytes();
     for (auto &o : parent->idle_slots) kept += o.bytes();
     const bool whole = is.s && is.done && is.upload_done && is.frame_done;
-    if (whole && kept <= kIdleBytes && parent->idle_slots.size() < kIdleSlots) parent->idle_slots.push_back(is);
-    else idle_slot_free(is);
+    if (!whole || is.bytes() > kIdleBytes) {
+        idle_slot_free(is);
+        return;
+    }
+    auto &idle = parent->idle_slots;
+    while (kept > kIdleBytes || idle.size() >= kIdleSlots) {
+        kept -= idle.front().bytes();
+        idle_slot_free(idle.front());
+        idle.erase(idle.begin());
+    }
+    idle.push_back(is);
 }
 
 double ms_since(std::chrono::steady_clock::time_point t0) {

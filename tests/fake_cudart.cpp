@@ -66,6 +66,7 @@ API void fake_reset() { last = cudaSuccess; launches.clear(); limit = ~size_t(0)
 API void fake_limit(size_t bytes) { limit = bytes; }
 API size_t fake_reserved() { return used + idle; }
 API int fake_arrays() { return (int)arrays.size(); }
+API int fake_surface_arrays_made() { return surf_calls; }
 API void fake_fail_surface_array(int nth, int error) { surf_calls = 0; surf_fail = nth; surf_error = error; }
 API void *fake_device_alloc(size_t n) { void *p = nullptr; take(&p, n, false); return p; }
 API const char *fake_launches() {

@@ -180,3 +180,18 @@ def test_the_scratch_of_a_voxel_gradient_is_exact_and_given_back(lib):
         h.ok(lib.vr_load_cube(h.h, cube.ctypes.data, 0, 200, 200, 150, 0, None, None, C.byref(cid)))
         lib.fake_limit((1 << 64) - 1)
         h.ok(backward(h, small, 200))
+
+
+@pytest.mark.parametrize("others,again", [([(3 + k, 4, 5) for k in range(260)], (90, 80, 70)),       # more arrays than are kept
+                                          ([(500, 500, 330 + k) for k in range(5)], (400, 300, 200))])  # more bytes: 335 MB each
+def test_the_arrays_of_the_last_cubes_are_the_ones_kept(lib, others, again):
+    """A viewer that has opened cubes of many sizes and now opens one size again and again."""
+    with Host(lib) as h:
+        made = []
+        for n in others + 3 * [again]:
+            cid, before = h.load(n), lib.fake_surface_arrays_made()
+            h.ok(h.brick(cid, (512, 512, 512)))
+            made.append(lib.fake_surface_arrays_made() - before)
+            h.ok(lib.vr_free_cube(h.h, cid))
+        assert made[-3:] == [1, 0, 0]
+        assert lib.fake_arrays() <= 256 and lib.fake_reserved() <= (3 << 30) + (1 << 20)
