@@ -183,7 +183,7 @@ def test_the_scratch_of_a_voxel_gradient_is_exact_and_given_back(lib):
 
 
 @pytest.mark.parametrize("others,again", [([(3 + k, 4, 5) for k in range(260)], (90, 80, 70)),       # more arrays than are kept
-                                          ([(500, 500, 330 + k) for k in range(5)], (400, 300, 200))])  # more bytes: 335 MB each
+                                          ([(500, 500 - 9 * k, 330) for k in range(5)], (400, 300, 200))])  # more bytes: 340 MB each
 def test_the_arrays_of_the_last_cubes_are_the_ones_kept(lib, others, again):
     """A viewer that has opened cubes of many sizes and now opens one size again and again."""
     with Host(lib) as h:
