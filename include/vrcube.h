@@ -96,12 +96,16 @@ typedef struct {
  * memory and 1 GiB of the atlas arrays of cubes it freed, up to 16 frame slots (2 GiB) of
  * closed serving loops and the scratch of the largest voxel gradient (16 bytes a voxel, at most
  * 4 GiB), for its next ones; its own allocations take all of that back when the
- * device is out of memory, vr_destroy releases it.  Errors: VR_ERR_ARG (null out, bad device),
+ * device is out of memory, vr_release_idle and vr_destroy release it.  Errors: VR_ERR_ARG (null out, bad device),
  * VR_ERR_CUDA, VR_ERR_OOM. */
 int vr_create(vr_ctx **out, int device, size_t cache_bytes);
 
 /* Waits for the context's outstanding work, then frees everything it owns.  NULL is a no-op. */
 void vr_destroy(vr_ctx *ctx);
+
+/* Gives what the context keeps unused (see vr_create) back to the device, for other users of it, once
+ * the work that used it is done.  Not while a server of the context is open.  Errors: VR_ERR_ARG. */
+int vr_release_idle(vr_ctx *ctx);
 
 /* Loads a cube (Section 2.3: "the whole cube or a manually specified sub-cube").
  * voxels: nx*ny*nz elements of `dtype` (VR_F32 only) in host (VR_HOST) or device (VR_DEVICE)

@@ -192,6 +192,11 @@ class Context:
     def free_cube(self, cube_id: int):
         _check(self._L.vr_free_cube(self._h, cube_id), "vr_free_cube")
 
+    def release_idle(self):
+        """Gives the memory that freed cubes, closed serving loops and gradients left to the context back
+        to the device."""
+        _check(self._L.vr_release_idle(self._h), "vr_release_idle")
+
     def compute_minmax(self, cube_id: int):
         lo, hi = C.c_float(), C.c_float()
         _check(self._L.vr_compute_minmax(self._h, cube_id, C.byref(lo), C.byref(hi)),

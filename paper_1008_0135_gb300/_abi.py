@@ -60,6 +60,7 @@ P, I, I64, F, VP = C.POINTER, C.c_int, C.c_int64, C.c_float, C.c_void_p
 SIGNATURES = {
     "vr_create": (I, [P(VP), I, C.c_size_t]),
     "vr_destroy": (None, [VP]),
+    "vr_release_idle": (I, [VP]),
     "vr_load_cube": (I, [VP, VP, I, I64, I64, I64, I, P(I64), P(I64), P(I)]),
     "vr_load_cube_procedural": (I, [VP, C.c_uint64, I64, I64, I64, P(I)]),
     "vr_set_fault_injection": (I, [VP, I, I64]),

@@ -1475,6 +1475,16 @@ static void vr_destroy_body(vr_ctx *c) {
     delete c;
 }
 
+static int vr_release_idle_body(vr_ctx *c) {
+    if (!c) return arg_fail("null ctx");
+    const int rc = set_dev(c);
+    if (rc == VR_OK) idle_release(c);
+    return rc;
+}
+int vr_release_idle(vr_ctx *c) {
+    return abi_guard([&] { return vr_release_idle_body(c); });
+}
+
 static int vr_load_cube_body(vr_ctx *c, const void *voxels, int dtype, int64_t nx, int64_t ny, int64_t nz, int where,
                  const int64_t *sub_origin, const int64_t *sub_extent, int *cube_id);
 int vr_load_cube(vr_ctx *c, const void *voxels, int dtype, int64_t nx, int64_t ny, int64_t nz, int where,

@@ -195,3 +195,22 @@ def test_the_arrays_of_the_last_cubes_are_the_ones_kept(lib, others, again):
             h.ok(lib.vr_free_cube(h.h, cid))
         assert made[-3:] == [1, 0, 0]
         assert lib.fake_arrays() <= 256 and lib.fake_reserved() <= (3 << 30) + (1 << 20)
+
+
+def test_idle_memory_can_be_released(lib):
+    with Host(lib) as h:
+        for _ in range(2):
+            cid = h.load((100, 100, 100))
+            h.ok(h.brick(cid, (64, 64, 64)))
+            h.camera(_view(np.eye(3), (-50, -50, -200)), param=150.0, W=512, H=512)
+            h.ok(lib.vr_render_backward(h.h, cid, h.out.ctypes.data, h.out.ctypes.data, h.out.ctypes.data, None))
+            h.ok(lib.vr_free_cube(h.h, cid))
+        kept = lib.fake_reserved()
+        h.ok(lib.vr_release_idle(h.h))
+        # voxels, bricks and atlases, and the sums
+        assert kept - lib.fake_reserved() > 4 * 3 * 100 ** 3 + 16 * 101 * 101 * 102
+        assert lib.fake_arrays() == 0
+        cid = h.load((100, 100, 100))
+        h.ok(h.brick(cid, (64, 64, 64)))
+        h.ok(h.frame(cid))
+    assert lib.vr_release_idle(None) == -1
