@@ -175,7 +175,6 @@ void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0) {
     while ((double)inv * rows < 1.0) inv = std::nextafterf(inv, 2.0f);
     b.at_inv = inv;
     b.at_neg = -(float)rows;
-    b.at_rows = rows;
 }
 
 // What the 2D-gather size admits is decided by the squarest arrangement (2^l columns, no copies).
@@ -1053,7 +1052,7 @@ int stage_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
         const int *dm = cb->tmpl[i].dim;
         extent(i, w, h);
         const char *src = static_cast<const char *>(cb->d_pool) + (size_t)cb->loff[3 * i] * bsz;
-        e = cb->atlas_pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, 0ull, s)
+        e = cb->atlas_pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, s)
                            : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, s);
         if (e == cudaSuccess)
             e = cudaMemcpy2DToArrayAsync(cb->atlas_arr[cb->atlas_of[i]], (size_t)cell.x0 * esz, cell.y0, tmp, w * esz, w * esz,

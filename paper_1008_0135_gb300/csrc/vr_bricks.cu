@@ -297,9 +297,8 @@ cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz
 }
 
 cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
-                             unsigned long long surf, cudaStream_t s) {
-    return surf ? pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackSurf{(cudaSurfaceObject_t)surf}, s)
-                : pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackLinear{static_cast<char *>(atlas), pitch}, s);
+                             cudaStream_t s) {
+    return pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackLinear{static_cast<char *>(atlas), pitch}, s);
 }
 
 template <int S>

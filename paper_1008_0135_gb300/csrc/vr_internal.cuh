@@ -77,7 +77,6 @@ struct DrawBrick {
     float at_org[2];               // 1 + the first column's corner in the array
     float at_dim[2];               // dim[0], dim[1]
     float at_inv, at_neg;          // 1 / K rounded up, -K
-    int at_rows;                   // K
     int skip;                      // global termination: every sample of this brick adds nothing
                                    // (its values map only to zero opacity), walk through it
     long long pad_off;             // staged frames (fetch 4): element offset of the brick's copy
@@ -131,10 +130,9 @@ cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz
 cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows,
                                    unsigned long long surf, cudaStream_t s);
 // Packs one x-contiguous 16-bit brick into its pair atlas (dz - 1 tiles of dx x dy 32-bit
-// texels in columns of `rows`): through surface `surf` when non-zero, else into
-// the pitch-linear `atlas` of row pitch `pitch` bytes.
+// texels in columns of `rows`), a pitch-linear buffer of row pitch `pitch` bytes.
 cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
-                             unsigned long long surf, cudaStream_t s);
+                             cudaStream_t s);
 // Writes every brick's stored region (records: geometry, data_off, str) into the pool, and, with
 // cells, into its atlas as well (pair: pair texels of 16-bit codes).
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
