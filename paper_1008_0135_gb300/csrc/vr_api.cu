@@ -179,9 +179,9 @@ void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0) {
 
 // What the 2D-gather size admits is decided by the squarest arrangement (2^l columns, no copies).
 // Columns are then as tall as fit, evened out: fewest copies (258^3 bricks: 3 columns of 86 slices
-// and a copy, 1.2 % more texels).  Between the two rules lie bricks of about a billion texels
-// (stored cubes from 993^3 to 1024^3): they are admitted, with rows = 0, and read the linear copy.
-int atlas_geom(int device, const int dim[3], bool pair, AtlasGeom &g) {
+// and a copy, 1.2 % more texels).  Without copies they fit whenever the squarest arrangement does; with
+// them bricks near the limit do not (cubes from 993^3, flat bricks of 4 slices from 11000^2).
+int atlas_geom(int device, const int dim[3], bool pair, bool copies, AtlasGeom &g) {
     int gw = 0, gh = 0;
     CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, device));
     CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, device));
@@ -191,9 +191,10 @@ int atlas_geom(int device, const int dim[3], bool pair, AtlasGeom &g) {
     if (((long long)dim[0] << l) > gw || (long long)((nt + (1 << l) - 1) >> l) * dim[1] > gh)
         return fail(VR_ERR_UNSUPPORTED, "bricks too large for a slice atlas (2D gather limit)");
     g = AtlasGeom{};
-    const int fit = gh / dim[1], extra = pair ? 0 : 1;
+    g.copies = copies;
+    const int fit = gh / dim[1], extra = copies ? 1 : 0;
     const int cols = nt <= fit ? 1 : (fit > extra ? (nt + fit - extra - 1) / (fit - extra) : gw);
-    if ((long long)cols * dim[0] > gw) return VR_OK;         // rows = 0: no room for the copies
+    if ((long long)cols * dim[0] > gw) return VR_OK;
     g.rows = (nt + cols - 1) / cols;
     g.w = cols * dim[0];
     g.h = (g.rows + (cols > 1 ? extra : 0)) * dim[1];
@@ -206,7 +207,7 @@ FrameLayout frame_layout(const vr_ctx *c, const Cube *cb) {
     // resident cubes: atlases built with the pool; streamed and compressed cubes: atlases of the
     // brick cache's slots, packed as bricks become resident
     // (within kAtlasReach: atlas frames clamp no index, see there)
-    const bool atlas = (cb->streamed ? (cb->layouts & 8) != 0 && cb->atlas_fit : !cb->atlas_tex.empty()) &&
+    const bool atlas = (cb->streamed ? (cb->layouts & 8) != 0 : !cb->atlas_tex.empty()) &&
                        (!c->cam_set || within_reach(c, cb));
     // with atlases, the image axis is fixed first: the one with the smaller z component
     const int only = atlas ? (std::fabs(c->cam.R[5]) < std::fabs(c->cam.R[2]) ? 1 : 0) : -1;
@@ -589,7 +590,7 @@ FrameConsts make_consts(vr_ctx *c, Cube *cb) {
     // axis its loads are nearly coalesced and the stencil cache's bookkeeping costs more than
     // it saves; with a poor alignment it pays
     // (MIP frames: no stencil cache).  Cameras beyond kAtlasReach: clamped indices.
-    if (fl.atlas) fc.fetch = cb->atlas_pair && !cb->streamed ? 5 : 2;
+    if (fl.atlas) fc.fetch = cb->atlas_pair && !cb->streamed ? 5 : cb->atlas_copies ? 2 : 3;
     else if (c->cam_set && !within_reach(c, cb)) fc.fetch = 0;
     // (masked frames read rows at every view, only those of enabled channels: 227 against 300 us a 641x479 frame
     // with every third channel off)
@@ -942,13 +943,15 @@ int make_atlases(vr_ctx *c, Cube *cb) {
     const int nbr = (int)cb->tmpl.size();
     const bool pair = (cb->layouts & 32) && cb->storage != VR_F32;
     std::vector<AtlasGeom> geo(nbr);
-    cb->atlas_fit = true;
+    cb->atlas_copies = !pair;
     for (int i = 0; i < nbr; ++i) {
-        const int rc = atlas_geom(c->device, cb->tmpl[i].dim, pair, geo[i]);
+        const int rc = atlas_geom(c->device, cb->tmpl[i].dim, pair, cb->atlas_copies, geo[i]);
         if (rc != VR_OK) return rc;
-        if (geo[i].rows == 0) cb->atlas_fit = false;
+        if (geo[i].rows == 0) {              // no room for copies: none in the whole cube
+            cb->atlas_copies = false;
+            i = -1;
+        }
     }
-    if (!cb->atlas_fit) return VR_OK;        // frames read the linear copy
     int gw = 0, gh = 0;
     CK(cudaDeviceGetAttribute(&gw, cudaDevAttrMaxTexture2DGatherWidth, c->device));
     CK(cudaDeviceGetAttribute(&gh, cudaDevAttrMaxTexture2DGatherHeight, c->device));
@@ -958,7 +961,7 @@ int make_atlases(vr_ctx *c, Cube *cb) {
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return geo[a].h > geo[b].h; });
     struct Dim { int w, h; };
     std::vector<Dim> dims;                   // of each array
-    cb->atlas_cells.assign(nbr, AtlasCell{0ull, 0, 0, 1});
+    cb->atlas_cells.assign(nbr, AtlasCell{0ull, 0, 0, 1, 0});
     cb->atlas_of.assign(nbr, 0);
     int x = 0, y = 0, shelf = 0;
     for (int i : ord) {
@@ -969,7 +972,7 @@ int make_atlases(vr_ctx *c, Cube *cb) {
             x = y = shelf = 0;
         }
         Dim &d = dims.back();
-        cb->atlas_cells[i] = AtlasCell{0ull, x, y, g.rows};
+        cb->atlas_cells[i] = AtlasCell{0ull, x, y, g.rows, g.copies ? 1 : 0};
         cb->atlas_of[i] = (int)dims.size() - 1;
         x += g.w;
         shelf = std::max(shelf, g.h);
@@ -1037,7 +1040,7 @@ int stage_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
         const int *dm = cb->tmpl[i].dim, rows = cb->atlas_cells[i].rows, nt = cb->atlas_pair ? dm[2] - 1 : dm[2];
         const int cols = (nt + rows - 1) / rows;
         w = (size_t)cols * dm[0];
-        h = (size_t)(cols > 1 ? rows + (cb->atlas_pair ? 0 : 1) : nt) * dm[1];
+        h = (size_t)(cols > 1 ? rows + (cb->atlas_copies ? 1 : 0) : nt) * dm[1];
     };
     size_t w, h;
     for (size_t i = 0; i < cb->tmpl.size(); ++i) {
@@ -1053,7 +1056,7 @@ int stage_atlases(vr_ctx *c, Cube *cb, cudaStream_t s) {
         extent(i, w, h);
         const char *src = static_cast<const char *>(cb->d_pool) + (size_t)cb->loff[3 * i] * bsz;
         e = cb->atlas_pair ? launch_pair_pack(src, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, s)
-                           : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], cell.rows, tmp, w * esz, s);
+                           : launch_atlas_pack(src, (int)esz, dm[0], dm[1], dm[2], cell.rows, cell.copies != 0, tmp, w * esz, s);
         if (e == cudaSuccess)
             e = cudaMemcpy2DToArrayAsync(cb->atlas_arr[cb->atlas_of[i]], (size_t)cell.x0 * esz, cell.y0, tmp, w * esz, w * esz,
                                          h, cudaMemcpyDeviceToDevice, s);

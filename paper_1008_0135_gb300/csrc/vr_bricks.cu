@@ -132,7 +132,7 @@ k_brick_build(const float *__restrict__ cube, int nx, int ny, int nz, const Draw
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     using T = decltype(encode<S>(0.0f, 0, true, 0.0f));
     T *out = static_cast<T *>(pool);
-    AtlasCell cell{0ull, 0, 0, 1};
+    AtlasCell cell{0ull, 0, 0, 1, 0};
     if (ATLAS) cell = cells[blockIdx.y];
     for (long long r = ((long long)blockIdx.x * 8 + warp) * kRows; r < rows; r += (long long)gridDim.x * 8 * kRows) {
         const float *row[kRows], *up[kRows];
@@ -150,7 +150,7 @@ k_brick_build(const float *__restrict__ cube, int nx, int ny, int nz, const Draw
                 const int c = z / cell.rows, zr = z - c * cell.rows;
                 ax[k] = cell.x0 + c * dx;
                 ay[k] = cell.y0 + zr * dy + y;
-                twice[k] = ATLAS == 1 && zr == 0 && c > 0 ? cell.y0 + cell.rows * dy + y : -1;
+                twice[k] = ATLAS == 1 && cell.copies && zr == 0 && c > 0 ? cell.y0 + cell.rows * dy + y : -1;
             }
             if (ATLAS == 2) {                        // no tile for the last slice
                 up[k] = cube + ((long long)clampi(b.org[2] + z + 1, 0, nz - 1) * ny + gy) * nx;
@@ -258,13 +258,13 @@ struct PackSurf {
     }
 };
 template <typename T, bool PAIR, typename Dst>
-__global__ void __launch_bounds__(256) k_atlas_pack(PackSrc<T, PAIR> src, int dx, int dy, int nt, int rows, Dst dst) {
+__global__ void __launch_bounds__(256) k_atlas_pack(PackSrc<T, PAIR> src, int dx, int dy, int nt, int rows, bool copies, Dst dst) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long n = (long long)dy * nt;
     for (long long r = (long long)blockIdx.x * 8 + warp; r < n; r += (long long)gridDim.x * 8) {
         const int z = (int)(r / dy), y = (int)(r - (long long)z * dy);
         const int c = z / rows, zr = z - c * rows;
-        const bool twice = !PAIR && zr == 0 && c > 0;
+        const bool twice = copies && zr == 0 && c > 0;
         for (int x = lane; x < dx; x += 32) {
             const auto v = src.get((size_t)r, x);
             dst.put(v, c * dx + x, zr * dy + y);
@@ -274,31 +274,31 @@ __global__ void __launch_bounds__(256) k_atlas_pack(PackSrc<T, PAIR> src, int dx
 }
 
 template <typename T, bool PAIR, typename Dst>
-static cudaError_t pack(const void *brick, int dx, int dy, int nt, int rows, Dst dst, cudaStream_t s) {
+static cudaError_t pack(const void *brick, int dx, int dy, int nt, int rows, bool copies, Dst dst, cudaStream_t s) {
     const long long n = (long long)dy * nt;
     if (n <= 0 || dx <= 0) return cudaSuccess;
     const int grid = (int)std::min<long long>((n + 7) / 8, 152 * 8);
-    k_atlas_pack<T, PAIR, Dst><<<grid, 256, 0, s>>>(PackSrc<T, PAIR>{static_cast<const T *>(brick), dx, dy}, dx, dy, nt, rows, dst);
+    k_atlas_pack<T, PAIR, Dst><<<grid, 256, 0, s>>>(PackSrc<T, PAIR>{static_cast<const T *>(brick), dx, dy}, dx, dy, nt, rows, copies, dst);
     return cudaGetLastError();
 }
 
-cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows,
+cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows, bool copies,
                                    unsigned long long surf, cudaStream_t s) {
     const PackSurf d{(cudaSurfaceObject_t)surf};
-    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, d, s)
-                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, d, s);
+    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, copies, d, s)
+                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, copies, d, s);
 }
 
-cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, void *atlas,
+cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, bool copies, void *atlas,
                               size_t pitch, cudaStream_t s) {
     const PackLinear d{static_cast<char *>(atlas), pitch};
-    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, d, s)
-                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, d, s);
+    return esz == 4 ? pack<unsigned int, false>(brick, dx, dy, dz, rows, copies, d, s)
+                    : pack<unsigned short, false>(brick, dx, dy, dz, rows, copies, d, s);
 }
 
 cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
                              cudaStream_t s) {
-    return pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, PackLinear{static_cast<char *>(atlas), pitch}, s);
+    return pack<unsigned short, true>(brick, dx, dy, dz - 1, rows, false, PackLinear{static_cast<char *>(atlas), pitch}, s);
 }
 
 template <int S>

@@ -102,8 +102,8 @@ struct Cube {
     std::vector<int> atlas_of;         // brick -> array
     std::vector<std::pair<int, int>> atlas_dims;   // of each array
     int atlas_kind = 0;                // their texels (IdleArray::kind)
-    bool atlas_fit = true;             // (layout bit 3) the bricks' slices fit an array with the copies
-                                       // the columns carry; false: frames read the linear copy
+    bool atlas_copies = true;          // (layout bit 3) columns carry a copy of the next one's first slice;
+                                       // false: a brick's slices fit no array with them
     bool atlas_pair = false;           // the atlases are pair atlases (layout bit 5, 16-bit bricks)
     // streamed cubes: bricks are produced on the host and cached in HBM on demand
     bool streamed = false;
@@ -259,13 +259,15 @@ FrameLayout frame_layout(const vr_ctx *c, const Cube *cb);
 double ray_reach(const vr_ctx *c, const Cube *cb);
 // Whether the current camera's rays start near enough that no stencil index needs a clamp.
 bool within_reach(const vr_ctx *c, const Cube *cb);
-// Slice atlases: an array of w x h texels with columns of `rows` slices.
+// Slice atlases: an array of w x h texels with columns of `rows` slices (copies: and a copy each).
 struct AtlasGeom {
     int rows = 0, w = 0, h = 0;
+    bool copies = false;
 };
-// The atlas of a stored brick of dim[0] x dim[1] x dim[2] (pair: pair atlas) on the current
-// device.  VR_ERR_UNSUPPORTED beyond the 2D-gather size.
-int atlas_geom(int device, const int dim[3], bool pair, AtlasGeom &g);
+// The atlas of a stored brick of dim[0] x dim[1] x dim[2] (pair: pair atlas, without copies) on the
+// current device; rows = 0 where there is no room for the copies.  VR_ERR_UNSUPPORTED beyond the
+// 2D-gather size.
+int atlas_geom(int device, const int dim[3], bool pair, bool copies, AtlasGeom &g);
 // Puts an atlas (its texture, rows a column, corner in the array) in a brick's record.
 void set_atlas(DrawBrick &b, unsigned long long tex, int rows, int x0, int y0);
 // Strides of the copy of a dim[0] x dim[1] x dim[2] brick whose axis a is contiguous, its rows

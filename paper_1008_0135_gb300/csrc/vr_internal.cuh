@@ -40,7 +40,7 @@ struct FrameConsts {
                                    // the linear brick at clamped indices (cameras far away), 1 =
                                    // loads of the corners a ray's last cell did not hold (poorly
                                    // aligned layout), 2 = 2 gathers from the brick's slice-atlas
-                                   // texture, 4 = slabs of the brick staged in shared memory by
+                                   // texture, 3 = the same where no slice is stored twice, 4 = slabs of the brick staged in shared memory by
                                    // bulk copies from the copy with 16-byte rows (DVR, FP32
                                    // bricks), 5 = 1 gather from the brick's pair atlas (16-bit
                                    // bricks), 6 / 7 / 8 = 4 pairs of loads from a linear brick
@@ -73,7 +73,8 @@ struct DrawBrick {
                                    // array in which the stored slices (FP32 values or 16-bit
                                    // codes, dim[0] x dim[1] texels) stand below one another in
                                    // columns of K, each column but the last followed by a copy of
-                                   // the next one's first slice (pair atlases: no copies)
+                                   // the next one's first slice (none in pair atlases and where
+                                   // there is no room for them)
     float at_org[2];               // 1 + the first column's corner in the array
     float at_dim[2];               // dim[0], dim[1]
     float at_inv, at_neg;          // 1 / K rounded up, -K
@@ -117,17 +118,17 @@ cudaError_t launch_brick_maxabs(const float *cube, int nx, int ny, int nz, const
                                 int nbricks, unsigned int *maxbits, unsigned int *range,
                                 cudaStream_t s);
 // Where a brick's atlas is written: the surface over its array (0: none), the corner of its first
-// column and K, the slices a column.
+// column and K, the slices a column; copies: columns end with a copy of the next one's first slice.
 struct AtlasCell {
     unsigned long long surf;
-    int x0, y0, rows;
+    int x0, y0, rows, copies;
 };
 // Packs one x-contiguous stored brick (dx*dy*dz elements of esz = 4 or 2 bytes) into its slice
-// atlas (columns of `rows` slices, placed as DrawBrick::atlas says): into a pitch-linear
-// buffer of row pitch `pitch` bytes, or through a surface.
-cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, void *atlas,
+// atlas (columns of `rows` slices, placed as DrawBrick::atlas says, with copies or without): into a
+// pitch-linear buffer of row pitch `pitch` bytes, or through a surface.
+cudaError_t launch_atlas_pack(const void *brick, int esz, int dx, int dy, int dz, int rows, bool copies, void *atlas,
                               size_t pitch, cudaStream_t s);
-cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows,
+cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, int dz, int rows, bool copies,
                                    unsigned long long surf, cudaStream_t s);
 // Packs one x-contiguous 16-bit brick into its pair atlas (dz - 1 tiles of dx x dy 32-bit
 // texels in columns of `rows`), a pitch-linear buffer of row pitch `pitch` bytes.
@@ -148,13 +149,13 @@ cudaError_t launch_wavelet_encode(const float *cube, int nx, int ny, int nz, uns
                                   cudaStream_t s);
 // Decodes the stored regions of up to kWaveletJobs bricks (global voxels clamp(org + [0, dim))) from
 // the block store: x-contiguous FP32 into dst, or (surf) into slice atlases with columns of `rows`
-// slices from (x0, y0) of the array behind the surface.  b0, nb: filled by the launcher.
+// slices (copies as in AtlasCell) from (x0, y0) of the array behind the surface.  b0, nb: filled by the launcher.
 constexpr int kWaveletJobs = 16;
 struct WaveletJob {
     int org[3], dim[3];
     float *dst;
     unsigned long long surf;
-    int x0, y0, rows;
+    int x0, y0, rows, copies;
     int b0[3], nb[3];              // first block and blocks per axis the region touches
 };
 struct WaveletJobs {

@@ -334,11 +334,17 @@ __device__ __forceinline__ float4 gather_slice(unsigned long long tex, float2 xy
 // The footprints of slices iz and iz + 1, two gathers.  Slice iz + 1 always lies dy rows below:
 // the slice that heads a column is stored again below the column before it.  (Slices side by side
 // instead of below one another: FP32 frames 3.3 % slower, texture cache set conflicts.)
-template <int S>
+// WRAP: no slice is stored again, so the next one's place is its own (bricks near the gather size, which have
+// no room for the copies).
+template <bool WRAP>
+__device__ __forceinline__ float2 next_slice_xy(const Atlas &a, float2 ixy, float iz, float2 xy) {
+    return WRAP ? atlas_xy(a, ixy, __fadd_rn(iz, 1.0f)) : __fadd2_rn(xy, pair2(0.0f, a.dim.y));
+}
+template <int S, bool WRAP>
 __device__ __forceinline__ void gather_slices(const Atlas &a, float2 ixy, float iz, float4 &g0, float4 &g1) {
     const float2 xy = atlas_xy(a, ixy, iz);
     g0 = gather_slice<S>(a.tex, xy);
-    g1 = gather_slice<S>(a.tex, __fadd2_rn(xy, pair2(0.0f, a.dim.y)));
+    g1 = gather_slice<S>(a.tex, next_slice_xy<WRAP>(a, ixy, iz, xy));
 }
 // The same as the stencil v[x + 2y + 4z].
 __device__ __forceinline__ void gathers_to_stencil(const float4 &g0, const float4 &g1, float v[8]) {
@@ -375,7 +381,7 @@ __device__ __forceinline__ void unpack_pair(const uint4 g, float4 &g0, float4 &g
 template <int S, int F>
 __device__ __forceinline__ void gather_stencil(const Atlas &a, float2 ixy, float iz, float4 &g0, float4 &g1) {
     if constexpr (F == 5) unpack_pair<S>(gather_pair(a, ixy, iz), g0, g1);
-    else gather_slices<S>(a, ixy, iz, g0, g1);
+    else gather_slices<S, F == 3>(a, ixy, iz, g0, g1);
 }
 
 // Whether fetch mode F reads rows of a linear copy without clamps, and the copy's contiguous axis.
@@ -383,10 +389,10 @@ constexpr bool straight(int F) { return F >= 6; }
 constexpr int row_axis(int F) { return F - 6; }
 
 // Samples whose stencils a fragment kernel's segment loop fetches before it composites the first.
-constexpr int ahead(int F) { return F == 2 ? VR_AHEAD : F == 5 ? VR_AHEAD_PAIR : F >= 6 ? VR_AHEAD_ROWS : 1; }
+constexpr int ahead(int F) { return F == 2 || F == 3 ? VR_AHEAD : F == 5 ? VR_AHEAD_PAIR : F >= 6 ? VR_AHEAD_ROWS : 1; }
 
-// Whether fetch mode F reads a texture (the slice atlas, 2, or the pair atlas, 5).
-constexpr bool gathers(int F) { return F == 2 || F == 5; }
+// Whether fetch mode F reads a texture (the slice atlas, 2 and 3, or the pair atlas, 5).
+constexpr bool gathers(int F) { return F == 2 || F == 3 || F == 5; }
 
 template <int S>
 __device__ __forceinline__ void fetch8(const void *src, int i0, const Strides &t, float v[8]) {
@@ -557,10 +563,10 @@ __device__ __forceinline__ unsigned gather_masked(const Atlas &atl, const CellF 
         m = plane_bits(fc, s_mask, small_float_int(c.iz), org_z);
         g0 = g1 = make_float4(vcode, vcode, vcode, vcode);
     }
-    if constexpr (MASK && F == 2) {
+    if constexpr (MASK && F != 5) {
         const float2 xy = atlas_xy(atl, c.ixy, c.iz);
         if (m & 1) g0 = gather_slice<S>(atl.tex, xy);
-        if (m & 2) g1 = gather_slice<S>(atl.tex, __fadd2_rn(xy, pair2(0.0f, atl.dim.y)));
+        if (m & 2) g1 = gather_slice<S>(atl.tex, next_slice_xy<F == 3>(atl, c.ixy, c.iz, xy));
     } else if (m) {
         gather_stencil<S, F>(atl, c.ixy, c.iz, g0, g1);
     }
@@ -865,7 +871,7 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
 template <int MODE, int F>
 constexpr int rc_min_blocks() {
     if (MODE != 0) return VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1;
-    return F == 2 ? VR_ATLAS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : straight(F) ? VR_ROWS_MIN_BLOCKS : 1;
+    return F == 2 || F == 3 ? VR_ATLAS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : straight(F) ? VR_ROWS_MIN_BLOCKS : 1;
 }
 
 template <int S, int MODE, int F, bool MASK>
@@ -1599,9 +1605,9 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 // 256^3 cube, 8 views at 512^2, step 0.5, forward frames cast again: 18.5 -> 12.0 -> 11.2 ms with both
 // gradients, 9.9 -> 8.9 -> 8.1 ms with the table's alone.
 // ATLAS: the replay reads the stencils from the bricks' slice atlases (the forward's texels)
-// instead of the linear copy; then no index is clamped (make_consts).
+// instead of the linear copy; then no index is clamped (make_consts).  WRAP: fetch mode 3.
 constexpr int kAdjThreads = 128;
-template <bool ATLAS, int VOX>
+template <bool ATLAS, int VOX, bool WRAP>
 __global__ void __launch_bounds__(kAdjThreads, VR_ADJ_MIN_BLOCKS)
 k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const float *__restrict__ pool,
@@ -1656,7 +1662,7 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
     };
     CellF cn = cell_at(0.0f);
     float4 n0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), n1 = n0;
-    if (ATLAS && live) gather_slices<0>(atl, cn.ixy, cn.iz, n0, n1);
+    if (ATLAS && live) gather_slices<0, WRAP>(atl, cn.ixy, cn.iz, n0, n1);
     while (__any_sync(0xffffffffu, live)) {
         int li = -1;
         float4 lo = make_float4(0.0f, 0.0f, 0.0f, 0.0f), hi = lo;    // the sample's adds to entries li and li + 1
@@ -1666,7 +1672,7 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
             jf = __fadd_rn(jf, 1.0f);
             cn = cell_at(fminf(jf, nf - 1.0f));
             if (ATLAS) {
-                gather_slices<0>(atl, cn.ixy, cn.iz, n0, n1);
+                gather_slices<0, WRAP>(atl, cn.ixy, cn.iz, n0, n1);
             } else {                               // indices clamped to the stored brick
                 cl.ixy = pair2(fminf(fmaxf(cl.ixy.x, 0.0f), (float)mx), fminf(fmaxf(cl.ixy.y, 0.0f), (float)my));
                 cl.iz = fminf(fmaxf(cl.iz, 0.0f), (float)mz);
@@ -1945,6 +1951,7 @@ cudaError_t launch_rc_s(const FrameConsts &fc, const float4 *lut, const DrawBric
     switch (fc.fetch) {
         case 1: return VR_RC(0, 1, false);      // (masked frames read rows)
         case 2: return VR_RC_MODE(2);
+        case 3: return VR_RC_MODE(3);
         case 6: return VR_RC_MODE(6);
         case 7: return VR_RC_MODE(7);
         case 8: return VR_RC_MODE(8);
@@ -1989,12 +1996,10 @@ cudaError_t launch_march_s(const FrameConsts &fc, const float4 *lut, DrawBrick *
             return fc.chmask ? launch_march<S, 5, true>(fc, lut, bricks, g, pool, out, ctr, s)
                              : launch_march<S, 5, false>(fc, lut, bricks, g, pool, out, ctr, s);
     }
-    const bool atlas = fc.fetch == 2;
-    if (fc.chmask)
-        return atlas ? launch_march<S, 2, true>(fc, lut, bricks, g, pool, out, ctr, s)
-                     : launch_march<S, 0, true>(fc, lut, bricks, g, pool, out, ctr, s);
-    return atlas ? launch_march<S, 2, false>(fc, lut, bricks, g, pool, out, ctr, s)
-                 : launch_march<S, 0, false>(fc, lut, bricks, g, pool, out, ctr, s);
+#define VR_MARCH(F) (fc.chmask ? launch_march<S, F, true>(fc, lut, bricks, g, pool, out, ctr, s) \
+                               : launch_march<S, F, false>(fc, lut, bricks, g, pool, out, ctr, s))
+    return fc.fetch == 2 ? VR_MARCH(2) : fc.fetch == 3 ? VR_MARCH(3) : VR_MARCH(0);
+#undef VR_MARCH
 }
 
 cudaError_t launch_raymarch(const FrameConsts &fc, const float4 *lut, DrawBrick *bricks, const MarchGrid &g,
@@ -2042,14 +2047,14 @@ cudaError_t launch_composite_backward(const FrameConsts &fc, const DrawBrick *db
     return cudaGetLastError();
 }
 
-template <bool ATLAS, int VOX>
+template <bool ATLAS, int VOX, bool WRAP>
 static cudaError_t adjoint(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items, int nitems,
                            const float *pool, const float4 *frags, const float4 *gfrag, float *glut_partial, int rows, void *gvox,
                            cudaStream_t s) {
     static DeviceAttrs da;
-    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<ATLAS, VOX>), (int)(32 * kMaxLut), da);
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<ATLAS, VOX, WRAP>), (int)(32 * kMaxLut), da);
     if (e != cudaSuccess) return e;
-    k_adjoint<ATLAS, VOX><<<nitems * (256 / kAdjThreads), kAdjThreads, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
+    k_adjoint<ATLAS, VOX, WRAP><<<nitems * (256 / kAdjThreads), kAdjThreads, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
     return cudaGetLastError();
 }
 
@@ -2060,9 +2065,11 @@ cudaError_t launch_adjoint(const FrameConsts &fc, const float4 *lut, const DrawB
     if (nitems <= 0) return cudaSuccess;
     const cudaError_t e = cudaMemsetAsync(glut_partial, 0, sizeof(float) * 8 * (size_t)fc.nlut * rows, s);
     if (e != cudaSuccess) return e;
-#define VR_ADJ(A, V, G) adjoint<A, V>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s)
-    if (fc.fetch == 2) return corners ? VR_ADJ(true, 2, corners) : gvox ? VR_ADJ(true, 1, gvox) : VR_ADJ(true, 0, nullptr);
-    return corners ? VR_ADJ(false, 2, corners) : gvox ? VR_ADJ(false, 1, gvox) : VR_ADJ(false, 0, nullptr);
+#define VR_ADJ(A, V, W, G) adjoint<A, V, W>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s)
+#define VR_ADJ_VOX(A, W) (corners ? VR_ADJ(A, 2, W, corners) : gvox ? VR_ADJ(A, 1, W, gvox) : VR_ADJ(A, 0, W, nullptr))
+    if (fc.fetch == 3) return VR_ADJ_VOX(true, true);
+    return fc.fetch == 2 ? VR_ADJ_VOX(true, false) : VR_ADJ_VOX(false, false);
+#undef VR_ADJ_VOX
 #undef VR_ADJ
 }
 

@@ -584,12 +584,15 @@ static std::shared_ptr<BrickJob> produce_brick(Workers *pool, Cube *cb, const Dr
 
 // Slice atlases of cache slots (streamed and compressed cubes whose layout mask has bit 3):
 // every brick of a cube uses the columns of the cube's largest stored brick, so any of its
-// bricks fits a slot's array.
+// bricks fits a slot's array.  Sets the cube's atlas_copies.
 static int slot_atlas_geom(vr_ctx *c, Cube *cb, AtlasGeom &g) {
     int mx[3] = {0, 0, 0};
     for (auto &b : cb->tmpl)
         for (int a = 0; a < 3; ++a) mx[a] = std::max(mx[a], b.dim[a]);
-    return atlas_geom(c->device, mx, false, g);
+    int rc = atlas_geom(c->device, mx, false, true, g);
+    if (rc == VR_OK && g.rows == 0) rc = atlas_geom(c->device, mx, false, false, g);
+    cb->atlas_copies = g.copies;
+    return rc;
 }
 
 // Gives slot `si` an atlas array for cube `cb`'s bricks, creating or replacing it when it has
@@ -654,7 +657,7 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
     if (rc != VR_OK) return rc;
     if (s.surf) {
         CK(launch_atlas_pack_surf(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2],
-                                  g.rows, (unsigned long long)s.surf, k->copy));
+                                  g.rows, g.copies, (unsigned long long)s.surf, k->copy));
         s.rows = g.rows;
         s.atlas_ok = true;
         return VR_OK;
@@ -669,8 +672,8 @@ static int slot_atlas_pack(vr_ctx *c, Cube *cb, int si, const DrawBrick &b, cons
         k->pack_bytes = need;
     }
     const int cols = (b.dim[2] + g.rows - 1) / g.rows;
-    const size_t w = (size_t)cols * b.dim[0], h = (size_t)(cols > 1 ? g.rows + 1 : b.dim[2]) * b.dim[1];
-    CK(launch_atlas_pack(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2], g.rows,
+    const size_t w = (size_t)cols * b.dim[0], h = (size_t)(cols > 1 ? g.rows + (g.copies ? 1 : 0) : b.dim[2]) * b.dim[1];
+    CK(launch_atlas_pack(k->d_base + (size_t)si * k->slot_bytes, (int)esz, b.dim[0], b.dim[1], b.dim[2], g.rows, g.copies,
                          k->pack_tmp, w * esz, k->copy));
     CK(cudaMemcpy2DToArrayAsync(s.arr, 0, 0, k->pack_tmp, w * esz, w * esz, h, cudaMemcpyDeviceToDevice, k->copy));
     s.rows = g.rows;
@@ -696,6 +699,7 @@ static int decode_slots(vr_ctx *c, Cube *cb, const std::vector<std::pair<size_t,
             jb.surf = (unsigned long long)s.surf;
             jb.x0 = jb.y0 = 0;
             jb.rows = std::max(s.rows, 1);
+            jb.copies = cb->atlas_copies ? 1 : 0;
             if (s.used) CK(cudaStreamWaitEvent(k->copy, s.last_use, 0));
         }
         CK(launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], jobs, (int)(m1 - m0), surf, k->copy));
@@ -715,7 +719,7 @@ static int make_resident(vr_ctx *c, Cube *cb, std::vector<DrawBrick> &db, size_t
     int rc = VR_OK;
     if ((cb->layouts & 8) && (rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
     // whether this frame reads atlases (layout bit 3, a camera near enough) or linear copies
-    const bool atlas = (cb->layouts & 8) && g.rows > 0 && frame_layout(c, cb).atlas;
+    const bool atlas = (cb->layouts & 8) && frame_layout(c, cb).atlas;
     std::vector<std::pair<size_t, int>> misses;   // (db index, slot)
     for (size_t i = d0; i < d1; ++i) {
         auto it = k->where.find(key_of(cb->id, db[i].brick));
@@ -1128,8 +1132,6 @@ int cache_prepare_atlases(vr_ctx *c, Cube *cb) {
     if ((rc = cache_size(c, max_bytes)) != VR_OK) return rc;
     AtlasGeom g;
     if ((rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
-    cb->atlas_fit = g.rows > 0;
-    if (!cb->atlas_fit) return VR_OK;        // frames read the slots' linear bricks
     const int n = (int)std::min<size_t>((size_t)k->nslots, cb->tmpl.size());
     for (int i = 0; i < n; ++i)
         if ((rc = slot_atlas_alloc(c, cb, i, g)) != VR_OK) return rc;
@@ -1151,6 +1153,7 @@ int streamed_brick(Cube *cb, int64_t brick, void *data, int *exp2) {
         jb.surf = 0ull;
         jb.x0 = jb.y0 = 0;
         jb.rows = 1;
+        jb.copies = 0;
         cudaError_t er = launch_wavelet_decode(cb->d_wstore, (int)cb->n[0], (int)cb->n[1], (int)cb->n[2], jobs, 1, false, 0);
         if (er == cudaSuccess) er = cudaMemcpy(data, tmp, (size_t)b.bytes, cudaMemcpyDeviceToHost);
         cudaFree(tmp);

@@ -274,7 +274,7 @@ k_wavelet_decode(const unsigned char *__restrict__ store, int nx, int ny, int nz
     // slice z of the atlas: row zr of column c, and, at the head of a later column, again below the one before
     auto put_atlas = [&](int x, int y, int c, int zr, float v) {
         surf2Dwrite<float>(v, (cudaSurfaceObject_t)jb.surf, (jb.x0 + c * dx + x) * 4, jb.y0 + zr * dy + y, cudaBoundaryModeZero);
-        if (zr == 0 && c > 0)
+        if (jb.copies && zr == 0 && c > 0)
             surf2Dwrite<float>(v, (cudaSurfaceObject_t)jb.surf, (jb.x0 + (c - 1) * dx + x) * 4, jb.y0 + jb.rows * dy + y,
                                cudaBoundaryModeZero);
     };

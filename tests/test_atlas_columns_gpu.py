@@ -59,3 +59,41 @@ def test_atlas_frames_equal_linear_frames(ctx, shape, brick, storage, mask):
         assert all(np.array_equal(a, b) for a, b in zip(want, got))
         assert max(float(np.abs(a).max()) for a in want) > 0.05
     ctx.free_cube(cid)
+
+
+# stored bricks of 4 and 6 slices that a gather array only takes without the columns' copies (11002^2 x 4: two
+# columns of two slices; 7002 x 11002 x 6: three; the second with a small brick beside it)
+@pytest.mark.parametrize("shape,brick", [((11000, 11000, 2), (11000, 11000, 2)), ((7040, 11000, 4), (7000, 11000, 4))])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16", "compressed"])
+def test_bricks_near_the_gather_size_keep_their_atlases(shape, brick, storage):
+    import torch
+    gpu_ctx().close()
+    import paper_1008_0135_gb300 as P
+    sto = "f32" if storage == "compressed" else storage
+    ctx = P.Context(0, cache_bytes=6 << 30 if storage == "compressed" else 0)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    cid = ctx.load_cube(3.0 * torch.randn(shape[::-1], device="cuda", generator=g))
+    ctx.set_transfer_function(synth.random_lut(3, n=37), -8.0, 9.0)
+    if storage == "compressed":
+        ctx.compress_cube(cid)
+    got = []
+    for mask in (1, 9):
+        ctx.set_brick_layouts(cid, mask)
+        ctx.set_bricking(cid, brick, 1, sto)
+        got.append(_frames(ctx, cid, shape, False))
+        if storage == "f32":                             # the adjoint: corner sums and single atomics
+            for W, H in ((70, 52), (40, 30)):
+                cam = synth.random_camera(np.random.default_rng(W), shape, W, H, proj=1)
+                ctx.set_camera_dict(cam)
+                ctx.set_render_params("dvr", 1.0, 0.97)
+                grad = torch.randn((H, W, 4), device="cuda", generator=torch.Generator(device="cuda").manual_seed(W))
+                gl, gv = torch.empty((37, 4), device="cuda"), torch.zeros(shape[::-1], device="cuda")
+                ctx.render_backward(cid, grad, gl, gv)
+                got[-1] += [gl.cpu().numpy(), gv[:, ::7, ::5].cpu().numpy()]
+                del gv
+    ctx.close()
+    assert max(float(np.abs(a).max()) for a in got[0][:6]) > 0.05
+    for i, (a, b) in enumerate(zip(*got)):
+        # frames bit for bit; gradients to the order of their FP32 sums
+        assert np.array_equal(a, b) if i < 12 else np.abs(a - b).max() <= 2e-4 * np.abs(a).max()

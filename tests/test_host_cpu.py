@@ -214,3 +214,20 @@ def test_idle_memory_can_be_released(lib):
         h.ok(h.brick(cid, (64, 64, 64)))
         h.ok(h.frame(cid))
     assert lib.vr_release_idle(None) == -1
+
+
+@pytest.mark.parametrize("n", [(11000, 11000, 2), (7000, 11000, 4), (1000, 1000, 1000)])
+@pytest.mark.parametrize("storage", [0, 1])
+def test_bricks_near_the_gather_size_are_read_from_atlases(lib, n, storage):
+    """Admitted bricks all get an atlas, without copies of slices where those do not fit (fetch mode 3)."""
+    with Host(lib) as h:
+        cid = h.load(n)
+        h.ok(h.brick(cid, n, 9, storage))
+        assert lib.fake_arrays() == 1
+        h.camera(_view(np.eye(3), (-n[0] / 2, -n[1] / 2, -2 * n[0])), param=1.5 * n[0], step=1.0)
+        launches(lib)
+        h.ok(h.frame(cid))
+        assert [a[2] for k, a in launches(lib) if k == "k_raycast"] == [3]
+        h.ok(lib.vr_set_termination(h.h, 1))
+        h.ok(h.frame(cid))
+        assert [a[1] for k, a in launches(lib) if k == "k_raymarch"] == [3]
