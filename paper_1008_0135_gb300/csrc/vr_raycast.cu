@@ -751,14 +751,20 @@ __device__ __forceinline__ void thread_pixel(int lanes, const TileItem &it, int 
 // Threads of a ray-cast CTA.  A CTA's registers and table are held until its last ray ends, so half
 // a work item (4 warps) leaves fewer of them idle than a whole one: MIP 2 - 3 % faster, atlases
 // up to 11 %.  The stencil cache wants the whole item: its rows share lines in L1 (2.24 ms, halves 2.35).
+// (HALF below.)  DVR CTAs each hold a whole table, though, and above some hundred entries the tables of
+// twice as many CTAs take the shared memory that L1 and the texture cache would have, then the warps.
+// 768x768x512 at step 1, 1024^2, us with halves / whole items: slice atlas FP32 256 entries 1242 / 1303,
+// 768 1305 / 1321, 1024 2014 / 1325, 4096 5815 / 3060; pair atlas BF16 768 922 / 982, 1024 1303 / 990; rows
+// FP32 256 1492 / 1529, 384 1564 / 1562, 512 1687 / 1627, 1024 2940 / 1879, 4096 7519 / 4297.
+constexpr int kHalfTable = 768, kHalfTableRows = 384;
 template <int MODE, int F>
-constexpr int rc_threads() {
-    return MODE == 1 || gathers(F) || straight(F) ? 128 : 256;
+constexpr bool rc_halves() {
+    return MODE == 1 || gathers(F) || straight(F);
 }
 
 // The 32 rays of one warp: strip `strip` (0..7) of work item `it`; writes their fragments and
 // adds the warp's samples to the counters.
-template <int S, int MODE, int F, bool MASK>
+template <int S, int MODE, int F, bool MASK, bool HALF>
 __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__restrict__ lut,
                                          DrawBrick *__restrict__ dbs, const TileItem it, int strip, int lane,
                                          const void *__restrict__ pool, void *__restrict__ frags,
@@ -800,10 +806,10 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
             // the pixel's place is formed again here, so that the sample loop's registers hold only its own state
             unsigned tid;
             asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
-            if constexpr (rc_threads<MODE, F>() < 256) {
+            if constexpr (HALF) {
                 unsigned cta;
                 asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
-                tid += cta * rc_threads<MODE, F>() & 255u;
+                tid += cta * 128 & 255u;
             }
             int wx, wy;
             thread_pixel(fc.lanes_y, it, (int)(tid >> 5), (int)(tid & 31), wx, wy);
@@ -866,21 +872,22 @@ __device__ __forceinline__ void rc_strip(const FrameConsts &fc, const float4 *__
     }
 }
 
-// CTAs per SM the registers of k_raycast<., MODE, F, .> must allow (1: no constraint beyond one):
+// CTAs per SM the registers of k_raycast<., MODE, F, ., HALF> must allow (1: no constraint beyond one):
 // the fewest that the samples fetched ahead fit without spills.
-template <int MODE, int F>
+template <int MODE, int F, bool HALF>
 constexpr int rc_min_blocks() {
     if (MODE != 0) return VR_MIP_MIN_BLOCKS > 0 ? VR_MIP_MIN_BLOCKS : 1;
-    return F == 2 || F == 3 ? VR_ATLAS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : straight(F) ? VR_ROWS_MIN_BLOCKS : 1;
+    const int halves = F == 2 || F == 3 ? VR_ATLAS_MIN_BLOCKS : F == 5 ? VR_PAIR_MIN_BLOCKS : straight(F) ? VR_ROWS_MIN_BLOCKS : 1;
+    return HALF ? halves : (halves + 1) / 2;
 }
 
-template <int S, int MODE, int F, bool MASK>
-__global__ void __launch_bounds__(rc_threads<MODE, F>(), rc_min_blocks<MODE, F>())
+template <int S, int MODE, int F, bool MASK, bool HALF>
+__global__ void __launch_bounds__(HALF ? 128 : 256, rc_min_blocks<MODE, F, HALF>())
 k_raycast(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const void *__restrict__ pool, void *__restrict__ frags,
           Counters *__restrict__ ctr) {
     extern __shared__ float4 s_lut[];
-    constexpr int per = 256 / rc_threads<MODE, F>();      // CTAs of a work item
+    constexpr int per = HALF ? 2 : 1;                     // CTAs of a work item
     const int warp = (blockIdx.x % per) * (8 / per) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const TileItem it = items[blockIdx.x / per];
     unsigned char *s_mask = nullptr;
@@ -890,7 +897,7 @@ k_raycast(const FrameConsts fc, const float4 *__restrict__ lut, DrawBrick *__res
     }
     if (MODE == 0) load_table(lut, fc.nlut, s_lut);
     if (MODE == 0 || MASK) __syncthreads();
-    rc_strip<S, MODE, F, MASK>(fc, lut, dbs, it, warp, lane, pool, frags, ctr, s_lut, s_mask);
+    rc_strip<S, MODE, F, MASK, HALF>(fc, lut, dbs, it, warp, lane, pool, frags, ctr, s_lut, s_mask);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -1606,9 +1613,12 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 // gradients, 9.9 -> 8.9 -> 8.1 ms with the table's alone.
 // ATLAS: the replay reads the stencils from the bricks' slice atlases (the forward's texels)
 // instead of the linear copy; then no index is clamped (make_consts).  WRAP: fetch mode 3.
-constexpr int kAdjThreads = 128;
-template <bool ATLAS, int VOX, bool WRAP>
-__global__ void __launch_bounds__(kAdjThreads, VR_ADJ_MIN_BLOCKS)
+// THREADS: CTAs of half a work item up to so many table entries, as for the ray cast.  256^3, 2 views at 512^2, table gradient alone, us with halves /
+// whole items: atlas 256 entries 2030 / 2255, 1024 2350 / 2394, 2048 2710 / 2493, 4096 6095 / 3656; linear 256
+// 2905 / 3000, 640 3145 / 3148, 1024 4370 / 3270, 4096 8175 / 6028.
+constexpr int kHalfTableAdj = 1024, kHalfTableAdjLinear = 640;
+template <bool ATLAS, int VOX, bool WRAP, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 128 ? VR_ADJ_MIN_BLOCKS : 2)
 k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick *__restrict__ dbs,
           const TileItem *__restrict__ items, const float *__restrict__ pool,
           const float4 *__restrict__ frags, const float4 *__restrict__ gfrag,
@@ -1616,7 +1626,7 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
     extern __shared__ float4 s_lut[];
     load_table(lut, fc.nlut, s_lut);
     __syncthreads();
-    constexpr int per = 256 / kAdjThreads;       // CTAs of a work item
+    constexpr int per = 256 / THREADS;           // CTAs of a work item
     const TileItem it = items[blockIdx.x / per];
     const DrawBrick &b = dbs[it.db];
     const int warp = (blockIdx.x % per) * (8 / per) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -1903,21 +1913,29 @@ cudaError_t set_carveout(const void *kernel, size_t smem_per_cta, DeviceAttrs &d
     return e;
 }
 
-template <int S, int MODE, int F, bool MASK>
-cudaError_t launch_rc(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items,
+template <int S, int MODE, int F, bool MASK, bool HALF>
+cudaError_t launch_rc_kernel(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items,
                       int nitems, const void *pool, void *frags, Counters *ctr, cudaStream_t s) {
     static DeviceAttrs da;
+    constexpr int threads = HALF ? 128 : 256;
     const size_t smem = (MODE == 0 ? table_bytes(fc.nlut) : 0) + (MASK ? (size_t)fc.mask_planes : 0);
-    const void *kern = reinterpret_cast<const void *>(k_raycast<S, MODE, F, MASK>);
+    const void *kern = reinterpret_cast<const void *>(k_raycast<S, MODE, F, MASK, HALF>);
     cudaError_t e = ensure_smem_limit(kern, (int)(2 * sizeof(float4) * kMaxLut) + kMaskPlanes, da);
     if (e != cudaSuccess) return e;
     if (MODE == 0) {
-        e = set_carveout(kern, smem, da, rc_threads<MODE, F>() / 32);
+        e = set_carveout(kern, smem, da, threads / 32);
         if (e != cudaSuccess) return e;
     }
-    constexpr int threads = rc_threads<MODE, F>();
-    k_raycast<S, MODE, F, MASK><<<nitems * (256 / threads), threads, smem, s>>>(fc, lut, const_cast<DrawBrick *>(db), items, pool, frags, ctr);
+    k_raycast<S, MODE, F, MASK, HALF><<<nitems * (256 / threads), threads, smem, s>>>(fc, lut, const_cast<DrawBrick *>(db), items, pool, frags, ctr);
     return cudaGetLastError();
+}
+template <int S, int MODE, int F, bool MASK>
+cudaError_t launch_rc(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items,
+                      int nitems, const void *pool, void *frags, Counters *ctr, cudaStream_t s) {
+    if constexpr (MODE == 0 && rc_halves<MODE, F>())
+        if (fc.nlut > (straight(F) ? kHalfTableRows : kHalfTable))
+            return launch_rc_kernel<S, MODE, F, MASK, false>(fc, lut, db, items, nitems, pool, frags, ctr, s);
+    return launch_rc_kernel<S, MODE, F, MASK, rc_halves<MODE, F>()>(fc, lut, db, items, nitems, pool, frags, ctr, s);
 }
 
 template <bool MASK>
@@ -2047,14 +2065,15 @@ cudaError_t launch_composite_backward(const FrameConsts &fc, const DrawBrick *db
     return cudaGetLastError();
 }
 
-template <bool ATLAS, int VOX, bool WRAP>
+template <bool ATLAS, int VOX, bool WRAP, int THREADS>
 static cudaError_t adjoint(const FrameConsts &fc, const float4 *lut, const DrawBrick *db, const TileItem *items, int nitems,
                            const float *pool, const float4 *frags, const float4 *gfrag, float *glut_partial, int rows, void *gvox,
                            cudaStream_t s) {
     static DeviceAttrs da;
-    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(k_adjoint<ATLAS, VOX, WRAP>), (int)(32 * kMaxLut), da);
+    const auto kern = k_adjoint<ATLAS, VOX, WRAP, THREADS>;
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(kern), (int)(32 * kMaxLut), da);
     if (e != cudaSuccess) return e;
-    k_adjoint<ATLAS, VOX, WRAP><<<nitems * (256 / kAdjThreads), kAdjThreads, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
+    kern<<<nitems * (256 / THREADS), THREADS, 32 * (size_t)fc.nlut, s>>>(fc, lut, db, items, pool, frags, gfrag, glut_partial, rows, gvox);
     return cudaGetLastError();
 }
 
@@ -2065,7 +2084,8 @@ cudaError_t launch_adjoint(const FrameConsts &fc, const float4 *lut, const DrawB
     if (nitems <= 0) return cudaSuccess;
     const cudaError_t e = cudaMemsetAsync(glut_partial, 0, sizeof(float) * 8 * (size_t)fc.nlut * rows, s);
     if (e != cudaSuccess) return e;
-#define VR_ADJ(A, V, W, G) adjoint<A, V, W>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s)
+#define VR_ADJ(A, V, W, G) (fc.nlut <= (A ? kHalfTableAdj : kHalfTableAdjLinear) ? adjoint<A, V, W, 128>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s) \
+                                                     : adjoint<A, V, W, 256>(fc, lut, db, items, nitems, pool, frags, gfrag, glut_partial, rows, G, s))
 #define VR_ADJ_VOX(A, W) (corners ? VR_ADJ(A, 2, W, corners) : gvox ? VR_ADJ(A, 1, W, gvox) : VR_ADJ(A, 0, W, nullptr))
     if (fc.fetch == 3) return VR_ADJ_VOX(true, true);
     return fc.fetch == 2 ? VR_ADJ_VOX(true, false) : VR_ADJ_VOX(false, false);

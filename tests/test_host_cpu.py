@@ -231,3 +231,17 @@ def test_bricks_near_the_gather_size_are_read_from_atlases(lib, n, storage):
         h.ok(lib.vr_set_termination(h.h, 1))
         h.ok(h.frame(cid))
         assert [a[1] for k, a in launches(lib) if k == "k_raymarch"] == [3]
+
+
+@pytest.mark.parametrize("layouts,storage,last", [(9, 0, 768), (41, 1, 768), (7, 0, 384)])
+def test_large_tables_are_shared_by_whole_work_items(lib, layouts, storage, last):
+    with Host(lib) as h:
+        cid = h.load((64, 60, 62))
+        h.ok(h.brick(cid, (32, 32, 32), layouts, storage))
+        h.camera(_view(np.eye(3), (-32, -32, -100)))
+        for n in (2, last, last + 1, 4096):
+            lut = np.zeros((n, 4), np.float32)
+            h.ok(lib.vr_set_transfer_function(h.h, lut.ctypes.data, n, 0.0, 1.0))
+            launches(lib)
+            h.ok(h.frame(cid))
+            assert [a[4] for k, a in launches(lib) if k == "k_raycast"] == [int(n <= last)]
