@@ -724,7 +724,11 @@ int backward_view(vr_ctx *c, Cube *cb, const float *grad_out, float *grad_lut, d
     const bool reuse = c->frag_valid && c->frag_cube == cb->id && c->frag_gen == c->state_gen &&
                        c->d_frags.p == frags_before;
     const int nitems = (int)wl.items.size();
-    // a partial table gradient for every CTA; where those would pass 256 MB two CTAs share a row
+    // Rows of partial table gradients, one a work item: a CTA of a whole item has a row to itself, CTAs of
+    // half an item share it with one of another item.  Where the rows would pass 256 MB twice as many
+    // CTAs share one, which is not a bound but the size that rows of 16 bytes an entry would have: a row
+    // keeps the two ends of an interval apart (32 bytes), so that a sum of 512 rays' adds to one end
+    // has as many terms as one of 256 rays' to an entry.
     int rows = std::max(nitems, 1);
     if ((size_t)rows * 32 * fc.nlut > (size_t(256) << 20)) rows = (rows + 1) / 2;
     if ((rc = ensure(c->d_gpart, (size_t)rows * 8 * fc.nlut, c)) != VR_OK) return rc;

@@ -197,8 +197,8 @@ __global__ void __launch_bounds__(256) k_copy(const float *__restrict__ src, flo
     for (long long j = 4 * n4 + t; j < n; j += nt) dst[j] = src[j];
 }
 
-// CTAs a brick: enough of them over all bricks to fill the chip a few times, at most one per
-// 8 kRows rows of the tallest brick.
+// CTAs a brick: enough of them over all bricks to fill the chip a few times, 16 to 2048 (those beyond a
+// brick's rows find nothing to do).
 int row_ctas(int nbricks) { return std::min(2048, std::max(16, (152 * 8 * 4 + nbricks - 1) / nbricks)); }
 
 }  // namespace

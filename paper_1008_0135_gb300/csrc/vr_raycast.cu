@@ -1594,7 +1594,7 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 //   dL/dc_j = gC T_{j-1} a_j
 //   dL/da_j = T_{j-1} [ gC.c_j - (gC.(C_b - C_{<=j}) + gT T_b) / T_j ]   (T_j = T_{j-1}(1-a_j))
 //   last composited sample: dL/da_j = T_{j-1} [ gC.c_j - gT ]
-// Table gradients accumulate per CTA in a partial row in L2 (two float4 atomics per sample; eight
+// Table gradients accumulate in partial rows in L2, each of a few CTAs (two float4 atomics per sample; eight
 // float atomics per sample into shared-memory copies were 13 % slower per batch, their retries of
 // contended adds and the copy-out included).
 // Voxel gradients accumulate per ray for the 8 corners of its current cell and are added when the
@@ -1631,7 +1631,7 @@ k_adjoint(const FrameConsts fc, const float4 *__restrict__ lut, const DrawBrick 
     const DrawBrick &b = dbs[it.db];
     const int warp = (blockIdx.x % per) * (8 / per) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool odd = lane & 1;
-    // this CTA's table-gradient partial (rows are zeroed before the launch)
+    // the partial row of this CTA and of those rows apart (zeroed before the launch)
     float4 *g_row = reinterpret_cast<float4 *>(glut_partial) + (long long)(blockIdx.x % rows) * 2 * fc.nlut + (odd ? 1 : 0);
     // a warp's 32 rays are adjacent pixels along the image axis the brick layout follows
     int rx, ry;
@@ -1818,7 +1818,7 @@ k_corner_gather(const float4 *__restrict__ corners, int nx, int ny, int nz, floa
     }
 }
 
-// Final reduction of the per-CTA table-gradient partials, in FP64 and in two stages so that
+// Final reduction of the table-gradient partials, in FP64 and in two stages so that
 // every entry's sum is spread over many threads yet formed in a fixed order: chunk y sums the
 // partials of parts [y q, (y + 1) q) in part order, then the chunk sums are added in chunk order.
 // A partial holds, per interval, 4 channels for its lower entry and 4 for its upper one: an
