@@ -64,17 +64,23 @@ def test_slots_decoded_into_atlases_serve_linear_frames_and_other_cubes():
         c.set_bricking(cid, (24, 24, 24), 1, "f32")
         c.set_render_params("dvr", 0.8, 0.98)
         frames = []
-        for cam in (near, far, near):
-            c.set_camera_dict(cam)
-            frames.append(c.render_frame(cid).cpu().numpy())
-        other = c.load_cube(cube)          # 16-bit slots of another cube replace the arrays
+        c.set_camera_dict(near)
+        frames.append(c.render_frame(cid).cpu().numpy())
+        # another cube, whose stored bricks (40x20x20) fit the slots cut for 26^3 but not their arrays: its
+        # bricking replaces the arrays of as many slots as it has bricks, the first cube's among them
+        other = c.load_cube((3.0 * rng.standard_normal((36, 54, 76))).astype(np.float32))
         c.compress_cube(other)
         c.set_brick_layouts(other, mask)
-        c.set_bricking(other, (22, 44, 40), 1, "f32")
-        c.set_camera_dict(near)
+        c.set_bricking(other, (38, 18, 18), 1, "f32")
+        misses, hits = c.stats()["cache_misses"], c.stats()["cache_hits"]
+        frames.append(c.render_frame(cid).cpu().numpy())      # all still in their slots, their atlases gone
+        assert c.stats()["cache_misses"] == misses and c.stats()["cache_hits"] == hits + 12
+        for cam in (far, near):
+            c.set_camera_dict(cam)
+            frames.append(c.render_frame(cid).cpu().numpy())
         c.render_frame(other)
         frames.append(c.render_frame(cid).cpu().numpy())
         got.append(frames)
         c.close()
     assert all(np.array_equal(a, b) for a, b in zip(*got))
-    assert np.abs(got[0][1]).max() > 0.05
+    assert np.abs(got[0][2]).max() > 0.05
