@@ -1113,7 +1113,7 @@ int build_bricks(vr_ctx *c, Cube *cb, cudaStream_t s) {
             CK(cudaMemcpyAsync(cb->d_tmpl, rec.data(), sizeof(DrawBrick) * nbr, cudaMemcpyHostToDevice, s));
             if (first) CK(launch_brick_maxabs(cb->d_src, nx, ny, nz, cb->d_tmpl, nbr, cb->d_bs, d_range, s));
             CK(launch_brick_build(cb->d_src, nx, ny, nz, cb->d_tmpl, nbr, cb->d_bs, cb->storage, cb->d_pool, d_exps,
-                                  first && surf ? d_cells : nullptr, cb->atlas_pair, s));
+                                  first && surf ? d_cells : nullptr, cb->atlas_pair, cb->atlas_copies, s));
             first = false;
         }
     CK(cudaMemcpyAsync(bs.data(), cb->d_bs, sizeof(unsigned int) * bs.size(), cudaMemcpyDeviceToHost, s));

@@ -111,7 +111,8 @@ __device__ __forceinline__ auto encode(float v, int e, bool usual, float scale) 
     }
 }
 
-// ATLAS 0: the pool alone.  1: also the brick's slice atlas, 2: also its pair atlas (16-bit codes
+// ATLAS 0: the pool alone.  1: also the brick's slice atlas with copies of the columns' heads (3: without, its
+// own instantiation: a test of the cell in the rows' loop takes 553 us instead of 441), 2: also its pair atlas (16-bit codes
 // of slices z and z + 1 in one texel), through its array's surface: one pass over the source
 // instead of a pass for the pool and one per brick reading the pool back.  Bound by HBM (source
 // read, pool and atlas written): 741 MB into FP16 bricks of 130^3 with atlases 770 us and 120
@@ -150,7 +151,7 @@ k_brick_build(const float *__restrict__ cube, int nx, int ny, int nz, const Draw
                 const int c = z / cell.rows, zr = z - c * cell.rows;
                 ax[k] = cell.x0 + c * dx;
                 ay[k] = cell.y0 + zr * dy + y;
-                twice[k] = ATLAS == 1 && cell.copies && zr == 0 && c > 0 ? cell.y0 + cell.rows * dy + y : -1;
+                twice[k] = ATLAS == 1 && zr == 0 && c > 0 ? cell.y0 + cell.rows * dy + y : -1;
             }
             if (ATLAS == 2) {                        // no tile for the last slice
                 up[k] = cube + ((long long)clampi(b.org[2] + z + 1, 0, nz - 1) * ny + gy) * nx;
@@ -165,7 +166,7 @@ k_brick_build(const float *__restrict__ cube, int nx, int ny, int nz, const Draw
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
                 out[dst[k] + (long long)x * b.str[0]] = v[k];
-                if constexpr (ATLAS == 1) {
+                if constexpr (ATLAS == 1 || ATLAS == 3) {
                     surf2Dwrite<T>(v[k], (cudaSurfaceObject_t)cell.surf, (ax[k] + x) * (int)sizeof(T), ay[k], cudaBoundaryModeZero);
                     if (twice[k] >= 0)
                         surf2Dwrite<T>(v[k], (cudaSurfaceObject_t)cell.surf, (ax[k] - dx + x) * (int)sizeof(T), twice[k], cudaBoundaryModeZero);
@@ -303,12 +304,14 @@ cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows
 
 template <int S>
 static cudaError_t build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks, int nbricks,
-                         const unsigned int *maxbits, void *pool, int *exps, const AtlasCell *cells, bool pair, cudaStream_t s) {
+                         const unsigned int *maxbits, void *pool, int *exps, const AtlasCell *cells, bool pair, bool copies, cudaStream_t s) {
     const dim3 grid(row_ctas(nbricks), nbricks);
     if (!cells)
         k_brick_build<S, 0><<<grid, 256, 0, s>>>(cube, nx, ny, nz, bricks, maxbits, pool, exps, cells);
-    else if (S == 0 || !pair)
+    else if (copies)
         k_brick_build<S, 1><<<grid, 256, 0, s>>>(cube, nx, ny, nz, bricks, maxbits, pool, exps, cells);
+    else if (S == 0 || !pair)
+        k_brick_build<S, 3><<<grid, 256, 0, s>>>(cube, nx, ny, nz, bricks, maxbits, pool, exps, cells);
     else if constexpr (S != 0)
         k_brick_build<S, 2><<<grid, 256, 0, s>>>(cube, nx, ny, nz, bricks, maxbits, pool, exps, cells);
     return cudaGetLastError();
@@ -316,11 +319,11 @@ static cudaError_t build(const float *cube, int nx, int ny, int nz, const DrawBr
 
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                int nbricks, const unsigned int *maxbits, int storage, void *pool,
-                               int *exps, const AtlasCell *cells, bool pair, cudaStream_t s) {
+                               int *exps, const AtlasCell *cells, bool pair, bool copies, cudaStream_t s) {
     if (nbricks <= 0) return cudaSuccess;
-    if (storage == 0) return build<0>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, s);
-    if (storage == 1) return build<1>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, s);
-    return build<2>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, s);
+    if (storage == 0) return build<0>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, copies, s);
+    if (storage == 1) return build<1>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, copies, s);
+    return build<2>(cube, nx, ny, nz, bricks, nbricks, maxbits, pool, exps, cells, pair, copies, s);
 }
 
 }  // namespace vr

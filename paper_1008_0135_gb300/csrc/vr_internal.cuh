@@ -135,10 +135,10 @@ cudaError_t launch_atlas_pack_surf(const void *brick, int esz, int dx, int dy, i
 cudaError_t launch_pair_pack(const void *brick, int dx, int dy, int dz, int rows, void *atlas, size_t pitch,
                              cudaStream_t s);
 // Writes every brick's stored region (records: geometry, data_off, str) into the pool, and, with
-// cells, into its atlas as well (pair: pair texels of 16-bit codes).
+// cells, into its atlas as well (pair: pair texels of 16-bit codes; copies: the cells').
 cudaError_t launch_brick_build(const float *cube, int nx, int ny, int nz, const DrawBrick *bricks,
                                int nbricks, const unsigned int *maxbits, int storage, void *pool,
-                               int *exps, const AtlasCell *cells, bool pair, cudaStream_t s);
+                               int *exps, const AtlasCell *cells, bool pair, bool copies, cudaStream_t s);
 cudaError_t launch_raycast(const FrameConsts &fc, const float4 *lut, const DrawBrick *db,
                            const TileItem *items, int nitems, const void *pool, void *frags,
                            Counters *ctr, cudaStream_t s);
