@@ -20,8 +20,8 @@
 #include "vr_internal.cuh"
 
 // Tuning knobs of the ray-cast kernels (build-time): unroll factor of the linear sample loops, samples
-// fetched ahead (slice atlases, pair atlases, linear rows), the CTAs of 128 threads per SM the
-// register allocation must allow for DVR frames read through these and for MIP frames (0: no
+// fetched ahead (slice atlases, pair atlases, linear rows), the CTAs of 128 threads per SM (half as many of
+// 256) the register allocation must allow for DVR frames read through these and for MIP frames (0: no
 // constraint), and the same for the one-pass (global termination, 256 threads) kernel and the adjoint.
 #ifndef VR_SAMPLE_UNROLL
 #define VR_SAMPLE_UNROLL 1
@@ -750,7 +750,8 @@ __device__ __forceinline__ void thread_pixel(int lanes, const TileItem &it, int 
 
 // Threads of a ray-cast CTA.  A CTA's registers and table are held until its last ray ends, so half
 // a work item (4 warps) leaves fewer of them idle than a whole one: MIP 2 - 3 % faster, atlases
-// up to 11 %.  The stencil cache wants the whole item: its rows share lines in L1 (2.24 ms, halves 2.35).
+// up to 11 %.  (The halves of an item on two SMs both read the lines between them: FP32 frames of sparse rays
+// move 6 % more DRAM bytes, 1720x1720x256 3.46 instead of 3.26 GB, in 0.89 instead of 0.92 ms.)  The stencil cache wants the whole item: its rows share lines in L1 (2.24 ms, halves 2.35).
 // (HALF below.)  DVR CTAs each hold a whole table, though, and above some hundred entries the tables of
 // twice as many CTAs take the shared memory that L1 and the texture cache would have, then the warps.
 // 768x768x512 at step 1, 1024^2, us with halves / whole items: slice atlas FP32 256 entries 1242 / 1303,
@@ -1605,7 +1606,7 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 // 9.8 instead of 12.7 ms a batch of 8 views; with half of them 10.7) above the replay's gathers.  With
 // one atomic per corner it was bound by instruction issue: three variants of the flush, each run
 // by the few lanes that needed it, 17.8 of 32 lanes active and 1.25 G warp instructions a view
-// against 26.4 and 0.54 G.
+// against 27.5 and 0.64 G (1.54 and 0.90 ms).
 // Small launches are bound by the chain of samples: the next sample's gathers are issued ahead (one
 // 256^2 view of 64^3 with the table's gradient alone 128 -> 117 us).  CTAs of half a work item, which
 // hold their registers until their longest ray ends, and no spills (5 an SM, 91 registers): 117 -> 110.
@@ -1613,8 +1614,8 @@ __device__ __forceinline__ void flush_corners(float4 *__restrict__ corners, cons
 // gradients, 9.9 -> 8.9 -> 8.1 ms with the table's alone.
 // ATLAS: the replay reads the stencils from the bricks' slice atlases (the forward's texels)
 // instead of the linear copy; then no index is clamped (make_consts).  WRAP: fetch mode 3.
-// THREADS: CTAs of half a work item up to so many table entries, as for the ray cast.  256^3, 2 views at 512^2, table gradient alone, us with halves /
-// whole items: atlas 256 entries 2030 / 2255, 1024 2350 / 2394, 2048 2710 / 2493, 4096 6095 / 3656; linear 256
+// THREADS: CTAs of half a work item up to so many table entries, as for the ray cast.  256^3, 2 views at
+// 512^2, table gradient alone, us with halves / whole items: atlas 256 entries 2030 / 2255, 1024 2350 / 2394, 2048 2710 / 2493, 4096 6095 / 3656; linear 256
 // 2905 / 3000, 640 3145 / 3148, 1024 4370 / 3270, 4096 8175 / 6028.
 constexpr int kHalfTableAdj = 1024, kHalfTableAdjLinear = 640;
 template <bool ATLAS, int VOX, bool WRAP, int THREADS>
