@@ -1123,6 +1123,9 @@ int render_streamed_global(vr_ctx *c, Cube *cb, float *out, int out_where, cudaS
 // for its bricks and gives as many slots as it has bricks (at most all slots) an atlas array, so
 // that frames only pack.  Arrays already fit for its bricks are kept.
 int cache_prepare_atlases(vr_ctx *c, Cube *cb) {
+    // (first: the frames of a cube whose slots cannot be had now go by its atlas_copies too)
+    AtlasGeom g;
+    const int geom = slot_atlas_geom(c, cb, g);
     int rc = cache_create(c);
     if (rc) return rc;
     BrickCache *k = c->cache;
@@ -1130,8 +1133,7 @@ int cache_prepare_atlases(vr_ctx *c, Cube *cb) {
     size_t max_bytes = 0;
     for (auto &b : cb->tmpl) max_bytes = std::max(max_bytes, (size_t)b.bytes);
     if ((rc = cache_size(c, max_bytes)) != VR_OK) return rc;
-    AtlasGeom g;
-    if ((rc = slot_atlas_geom(c, cb, g)) != VR_OK) return rc;
+    if (geom != VR_OK) return fail(geom, "bricks too large for a slice atlas (2D gather limit)");
     const int n = (int)std::min<size_t>((size_t)k->nslots, cb->tmpl.size());
     for (int i = 0; i < n; ++i)
         if ((rc = slot_atlas_alloc(c, cb, i, g)) != VR_OK) return rc;

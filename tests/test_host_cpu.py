@@ -245,3 +245,19 @@ def test_large_tables_are_shared_by_whole_work_items(lib, layouts, storage, last
             launches(lib)
             h.ok(h.frame(cid))
             assert [a[4] for k, a in launches(lib) if k == "k_raycast"] == [int(n <= last)]
+
+
+def test_a_cache_that_could_not_be_sized_at_first_serves_large_bricks_right(lib):
+    """The layout call finds no memory, the frame later does: slots without copies, read without them."""
+    n = (11000, 11000, 2)
+    with Host(lib, cache=4 << 30) as h:
+        cid = h.load(n)
+        h.ok(lib.vr_compress_cube(h.h, cid))
+        h.ok(lib.vr_set_bricking(h.h, cid, *n, 1, 0))
+        lib.fake_limit(lib.fake_reserved())
+        assert lib.vr_set_brick_layouts(h.h, cid, 9) == -2
+        lib.fake_limit((1 << 64) - 1)
+        h.camera(_view(np.eye(3), (-5500, -5500, -22000)), param=16500.0, step=1.0)
+        launches(lib)
+        h.ok(h.frame(cid))
+        assert [a[2] for k, a in launches(lib) if k == "k_raycast"] == [3]
