@@ -136,6 +136,7 @@ class Context:
         self.device = device
         self.cam = None
         self.mode = VR_DVR
+        self._cube_bytes = {}         # of the cubes that update_cube may write
 
     def close(self):
         if getattr(self, "_h", None):
@@ -170,6 +171,8 @@ class Context:
         cid = C.c_int()
         _check(self._L.vr_load_cube(self._h, ptr, VR_F32, nx, ny, nz, loc, so, se, C.byref(cid)),
                "vr_load_cube")
+        ext = sub_extent if sub_extent is not None else (nx, ny, nz)
+        self._cube_bytes[cid.value] = 4 * int(ext[0]) * int(ext[1]) * int(ext[2])
         return cid.value
 
     def load_cube_procedural(self, seed: int, shape_xyz) -> int:
@@ -185,7 +188,11 @@ class Context:
                "vr_set_fault_injection")
 
     def update_cube(self, cube_id: int, voxels, stream=None):
+        """voxels: float32, as many as the cube has (of a longer buffer the first ones are taken)."""
         ptr, loc = _buffer(voxels)
+        have = voxels.numel() * voxels.element_size() if _is_torch(voxels) else np.asarray(voxels).nbytes
+        if have < self._cube_bytes.get(cube_id, 0):
+            raise ValueError("update_cube: fewer voxels than the cube has")
         sh = _stream_handle(stream) if loc == VR_DEVICE else 0
         _check(self._L.vr_update_cube(self._h, cube_id, ptr, loc, sh), "vr_update_cube")
 

@@ -261,3 +261,19 @@ def test_a_cache_that_could_not_be_sized_at_first_serves_large_bricks_right(lib)
         launches(lib)
         h.ok(h.frame(cid))
         assert [a[2] for k, a in launches(lib) if k == "k_raycast"] == [3]
+
+
+def test_the_binding_refuses_an_update_shorter_than_the_cube(lib, monkeypatch):
+    import paper_1008_0135_gb300 as P
+    monkeypatch.setattr(_abi, "_lib", lib)
+    lib.fake_reset()
+    ctx = P.Context(0)
+    cid = ctx.load_cube(np.zeros((5, 7, 9), np.float32))
+    sub = ctx.load_cube(np.zeros((5, 7, 9), np.float32), sub_origin=(1, 1, 1), sub_extent=(4, 3, 2))
+    for good in (np.zeros((5, 7, 9), np.float32), np.zeros(400, np.float32)):
+        ctx.update_cube(cid, good)
+    ctx.update_cube(sub, np.zeros((2, 3, 4), np.float32))
+    for c, n in ((cid, 314), (sub, 23)):
+        with pytest.raises(ValueError):
+            ctx.update_cube(c, np.zeros(n, np.float32))
+    ctx.close()
