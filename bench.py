@@ -747,7 +747,7 @@ def empty_space_leg(ctx, device, steps=16):
                               bytes="upper bound: stored bytes of every drawn brick / ray-cast time "
                                     "(segments stop early, so a drawn brick is not read whole); "
                                     "dram: that times the DRAM traffic / algorithmic bytes ratio of "
-                                    "the GASS-recipe slab capture (0.651)")
+                                    "the GASS-recipe slab capture (0.650)")
     ctx.free_cube(cid)
     res["workload"] = (f"GASS-scale 2048x2048x1600, {cfg['W']}x{cfg['H']} orbit, step "
                        f"{cfg['step']}, table with zero opacity below 3.0 (noise sd 0.5)")
