@@ -584,15 +584,13 @@ static std::shared_ptr<BrickJob> produce_brick(Workers *pool, Cube *cb, const Dr
 
 // Slice atlases of cache slots (streamed and compressed cubes whose layout mask has bit 3):
 // every brick of a cube uses the columns of the cube's largest stored brick, so any of its
-// bricks fits a slot's array.  Sets the cube's atlas_copies.
-static int slot_atlas_geom(vr_ctx *c, Cube *cb, AtlasGeom &g) {
+// bricks fits a slot's array.
+static int slot_atlas_geom(vr_ctx *c, const Cube *cb, AtlasGeom &g) {
     int mx[3] = {0, 0, 0};
     for (auto &b : cb->tmpl)
         for (int a = 0; a < 3; ++a) mx[a] = std::max(mx[a], b.dim[a]);
-    int rc = atlas_geom(c->device, mx, false, true, g);
-    if (rc == VR_OK && g.rows == 0) rc = atlas_geom(c->device, mx, false, false, g);
-    cb->atlas_copies = g.copies;
-    return rc;
+    const int rc = atlas_geom(c->device, mx, false, true, g);
+    return rc == VR_OK && g.rows == 0 ? atlas_geom(c->device, mx, false, false, g) : rc;
 }
 
 // Gives slot `si` an atlas array for cube `cb`'s bricks, creating or replacing it when it has
@@ -1123,9 +1121,11 @@ int render_streamed_global(vr_ctx *c, Cube *cb, float *out, int out_where, cudaS
 // for its bricks and gives as many slots as it has bricks (at most all slots) an atlas array, so
 // that frames only pack.  Arrays already fit for its bricks are kept.
 int cache_prepare_atlases(vr_ctx *c, Cube *cb) {
-    // (first: the frames of a cube whose slots cannot be had now go by its atlas_copies too)
+    // (first: the frames of a cube whose slots cannot be had now go by its atlas_copies too; and here
+    // alone, since frames on several threads read it)
     AtlasGeom g;
     const int geom = slot_atlas_geom(c, cb, g);
+    if (geom == VR_OK) cb->atlas_copies = g.copies;
     int rc = cache_create(c);
     if (rc) return rc;
     BrickCache *k = c->cache;
